@@ -295,8 +295,8 @@ int hisq_batch_cg(hisq_batch* batch, double* x, const double* b, const double* m
  * h = 0, +x, +y, +z, +t, -x, -y, -z, -t, with T_+mu psi(x) = F_mu(x) psi(x+mu) and
  * T_-mu psi(x) = F_mu(x-mu)^dag psi(x-mu) through the context's folded FP32 fat links.
  * Network: 1 -> channels -> 1 (channels = 8), linear; input an even-site vector embedded
- * with zeros on odd sites, output restricted to even sites. Channel mixing runs on the
- * tensor cores in BF16 with FP32 accumulation; master weights are FP32.
+ * with zeros on odd sites, output restricted to even sites. Weights enter rounded to BF16,
+ * arithmetic is FP32; master weights are FP32.
  * Weights: w1 [channels][1][9], w2 [1][channels][9], complex as (re, im) float pairs.
  * Network vectors: device, complex64 [nvec][V/2][3] (even sites).
  */

@@ -21,12 +21,12 @@ __device__ __forceinline__ void griddep_launch_dependents() {
 // launch stays a plain graph node: there the solves gained nothing from programmatic edges (FP32 mixed
 // CG within 0.1% at 48^3x12, 0.6% at 32^3x8) and the plain FP64 CG lost 2.4%.
 template <typename... Params, typename... Args>
-static cudaError_t launch_dependent(hisq_ctx* ctx, void (*kern)(Params...), int grid, int block,
-                                    Args&&... args) {
+static cudaError_t launch_dependent_smem(hisq_ctx* ctx, void (*kern)(Params...), dim3 grid, int block, size_t smem,
+                                         Args&&... args) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)grid);
+  cfg.gridDim = grid;
   cfg.blockDim = dim3((unsigned)block);
-  cfg.dynamicSmemBytes = 0;
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = ctx->stream;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -34,6 +34,10 @@ static cudaError_t launch_dependent(hisq_ctx* ctx, void (*kern)(Params...), int 
   cfg.attrs = at;
   cfg.numAttrs = ctx->pdl && !ctx->capturing ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kern, std::forward<Args>(args)...);
+}
+template <typename... Params, typename... Args>
+static cudaError_t launch_dependent(hisq_ctx* ctx, void (*kern)(Params...), dim3 grid, int block, Args&&... args) {
+  return launch_dependent_smem(ctx, kern, grid, block, 0, std::forward<Args>(args)...);
 }
 
 }  // namespace hisq

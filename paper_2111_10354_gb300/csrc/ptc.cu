@@ -1,5 +1,5 @@
-// Gauge-equivariant parallel-transport convolution (PTC) network on the GPU: forward layers,
-// backward (input and weight gradients), Adam, and the preconditioner apply z = N(r).
+// Gauge-equivariant parallel-transport convolution (PTC) network on the GPU: the preconditioner apply
+// z = N(r), the training loss and both layers' weight gradients, Adam, and the flexible CG that uses it.
 //
 // Layer: psi'_a(x) = sum_b sum_h W[a,b,h] (T_h psi_b)(x), 9 hops h = 0, +x..+t, -x..-t, with
 //   T_+mu psi(x) = F_mu(x) psi(x+mu),  T_-mu psi(x) = F_mu(x-mu)^dag psi(x-mu)
@@ -7,13 +7,11 @@
 // Network: layer 1 (1 -> C channels, full lattice), layer 2 (C -> 1, even sites); its input is an
 // even-site vector embedded with zeros on odd sites.
 //
-// Work split: the parallel transport (3x3 link times colour vector) runs on CUDA cores; the
-// channel mixing -- per colour, a [128 sites x 2*9*Cin] x [2*9*Cin x 2*Cout] real contraction of
-// the transported vectors with the complex weights written as 2x2 real blocks -- runs on the
-// fifth-generation tensor cores: operands in BF16 staged in shared memory (K-major), FP32
-// accumulators in TMEM, one thread issuing tcgen05.mma, completion through an mbarrier, results
-// read back with tcgen05.ld. The weight gradient (a contraction over sites) runs the same way
-// with the site index as K. Master weights and Adam moments are FP32.
+// The network is linear in its input and in each layer's weights, and both the apply and the training use
+// that: the two layers compose into one map whose mixing of the hops is an 8 x 8 matrix, and the loss
+// depends on the fields only through an 8 x 8 matrix of inner products (k_ptc_grad). Transports, mixing and
+// inner products are FP32 arithmetic on the CUDA cores with the weights rounded to BF16, sums across blocks
+// FP64. Master weights and Adam moments are FP32.
 #include <math.h>
 #include <string.h>
 
@@ -22,17 +20,15 @@
 
 #include "internal.cuh"
 #include "pdl.cuh"
+#include "reduce_warp.cuh"
 #include "trace.h"
-#include "tc.cuh"
 
 namespace hisq {
 
 bool is_device_ptr(const void* p);
 double dslash_bytes(const hisq_ctx* ctx, int lp, int sp, int nrhs);
 
-constexpr int PTC_TILE = 128;            // sites per tile = MMA M
 constexpr int NHOP = 9;
-constexpr uint32_t WAIT_LIMIT = 1u << 22;  // bounded mbarrier polls (an MMA tile takes microseconds)
 
 struct PtcGeom {
   Geom g;
@@ -40,535 +36,7 @@ struct PtcGeom {
   size_t blk_bytes;
 };
 
-__device__ __forceinline__ int lex_of(const Geom& g, int x, int y, int z, int t) {
-  return x + g.stride[1] * y + g.stride[2] * z + g.stride[3] * t;
-}
-
-// T_h psi at site idx (coordinates c) for one channel: psi full-lattice [V][3] float2.
-__device__ __forceinline__ void transport(const PtcGeom& G, const float2* __restrict__ psi, const int c[4], int idx,
-                                          int h, cplx<float> out[3]) {
-  if (h == 0) {
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      float2 v = psi[(size_t)idx * 3 + k];
-      out[k] = {v.x, v.y};
-    }
-    return;
-  }
-  const Geom& g = G.g;
-  const int mu = (h - 1) & 3;
-  const bool fwd = h <= 4;
-  int cm = c[mu] + (fwd ? 1 : -1);
-  int n = idx + (fwd ? g.stride[mu] : -g.stride[mu]);
-  if (cm >= g.L[mu]) n -= g.L[mu] * g.stride[mu];
-  if (cm < 0) n += g.L[mu] * g.stride[mu];
-  const int par = (c[0] + c[1] + c[2] + c[3]) & 1;
-  // forward: F_mu(x) from block (parity(x), fat, mu) at cb(x); backward: F_mu(x-mu) at cb(x-mu)
-  const int lpar = fwd ? par : 1 - par;
-  const int lcb = fwd ? (idx >> 1) : (n >> 1);
-  const char* blk = G.fat32 + (size_t)(lpar * 8 + mu) * G.blk_bytes;
-  cplx<float> U[9];
-  LinkIO<float>::load(blk, g.half, lcb, U);
-  cplx<float> v[3];
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    float2 w = psi[(size_t)n * 3 + k];
-    v[k] = {w.x, w.y};
-  }
-#pragma unroll
-  for (int i = 0; i < 3; ++i) {
-    out[i] = {0.f, 0.f};
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      if (fwd) cmac(out[i], U[3 * i + j], v[j]);
-      else cmac_conj(out[i], U[3 * j + i], v[j]);
-    }
-  }
-}
-
-// T_h psi_b at site idx for CIN channels at once: the link is loaded once per hop and the CIN
-// neighbour vectors are loaded together (memory-level parallelism).
-template <int CIN>
-__device__ __forceinline__ void transport_multi(const PtcGeom& G, const float2* __restrict__ psi, const int c[4],
-                                                int idx, int h, cplx<float> (&out)[CIN][3]) {
-  const Geom& g = G.g;
-  const size_t cstride = (size_t)g.V * 3;
-  if (h == 0) {
-#pragma unroll
-    for (int b = 0; b < CIN; ++b)
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        const float2 v = psi[b * cstride + (size_t)idx * 3 + k];
-        out[b][k] = {v.x, v.y};
-      }
-    return;
-  }
-  const int mu = (h - 1) & 3;
-  const bool fwd = h <= 4;
-  const int cm = c[mu] + (fwd ? 1 : -1);
-  int n = idx + (fwd ? g.stride[mu] : -g.stride[mu]);
-  if (cm >= g.L[mu]) n -= g.L[mu] * g.stride[mu];
-  if (cm < 0) n += g.L[mu] * g.stride[mu];
-  const int par = (c[0] + c[1] + c[2] + c[3]) & 1;
-  const int lpar = fwd ? par : 1 - par;
-  const int lcb = fwd ? (idx >> 1) : (n >> 1);
-  cplx<float> U[9];
-  LinkIO<float>::load(G.fat32 + (size_t)(lpar * 8 + mu) * G.blk_bytes, g.half, lcb, U);
-  float2 v[CIN][3];
-#pragma unroll
-  for (int b = 0; b < CIN; ++b)
-#pragma unroll
-    for (int k = 0; k < 3; ++k) v[b][k] = psi[b * cstride + (size_t)n * 3 + k];
-#pragma unroll
-  for (int b = 0; b < CIN; ++b)
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      cplx<float> a = {0.f, 0.f};
-#pragma unroll
-      for (int j = 0; j < 3; ++j) {
-        const cplx<float> w = {v[b][j].x, v[b][j].y};
-        if (fwd) cmac(a, U[3 * i + j], w);
-        else cmac_conj(a, U[3 * j + i], w);
-      }
-      out[b][i] = a;
-    }
-}
-
-// A pair (re, im) of bf16 at columns (col, col+1), col even: one 4-byte store.
-__device__ __forceinline__ void put_bf16x2(unsigned char* tile, int row, int col, int K2, float re, float im) {
-  *reinterpret_cast<__nv_bfloat162*>(tile + tc::kmajor_offset(row, col, K2)) = __floats2bfloat162_rn(re, im);
-}
-
-// Site of output row `row` of tile `tile`: full lattice (lexicographic) or even sites (cb order).
-__device__ __forceinline__ bool tile_site(const Geom& g, bool even_only, int tile, int row, int c[4], int* idx,
-                                          int* out_index) {
-  const int n = even_only ? g.half : g.V;
-  const int i = tile * PTC_TILE + row;
-  if (i >= n) return false;
-  if (even_only) {
-    site_coords(g, 0, i, c);
-    *idx = lex_index(g, c);
-  } else {
-    c[0] = i % g.L[0];
-    c[1] = (i / g.L[0]) % g.L[1];
-    c[2] = (i / (g.L[0] * g.L[1])) % g.L[2];
-    c[3] = i / (g.L[0] * g.L[1] * g.L[2]);
-    *idx = i;
-  }
-  *out_index = i;
-  return true;
-}
-
-__device__ __forceinline__ void put_bf16(unsigned char* tile, int row, int col, int K2, float v) {
-  *reinterpret_cast<__nv_bfloat16*>(tile + tc::kmajor_offset(row, col, K2)) = __float2bfloat16_rn(v);
-}
-
-// ------------------------------------------------------------------ forward layer
-// out_a(x) = sum_{b,h} W[a][b][h] T_h in_b (x). in: [CIN][V][3] float2 (full lattice);
-// out: [COUT][n_out][3] float2 with n_out = V (full) or V/2 (even sites, cb order).
-// W: [COUT][CIN][9] float2 (FP32 master weights, rounded to BF16 for the tensor cores).
-// Feature order is hop-major, k = h * CIN + b: with CIN = 8 each hop fills exactly one 16-column
-// MMA K-step, so the operand tile can be staged a few hops at a time (HPP hops per pass, all
-// passes accumulating into the same TMEM tile), which keeps the shared-memory footprint small
-// enough for several CTAs per SM to overlap their fill, MMA and read-out phases.
-template <int CIN>
-struct FwdShape {
-  static constexpr int HPP = CIN == 8 ? 3 : NHOP;                        // hops per pass
-  static constexpr int NPASS = (NHOP + HPP - 1) / HPP;
-  static constexpr int K2A = ((2 * CIN * HPP + 15) / 16) * 16;           // A columns per pass
-  static constexpr int K2B = CIN == 8 ? 2 * CIN * NHOP : K2A;            // B columns (all hops)
-};
-
-template <int CIN, int COUT, bool OUT_EVEN>
-__global__ void __launch_bounds__(256) k_ptc_forward(const PtcGeom G, const float2* __restrict__ in,
-                                                     float2* __restrict__ out, const float2* __restrict__ W,
-                                                     int* err, const int* skip) {
-  if (skip && *skip) return;  // a solver cycle that has already finished (uniform)
-  using S = FwdShape<CIN>;
-  constexpr int K2A = S::K2A, K2B = S::K2B, HPP = S::HPP, NPASS = S::NPASS;
-  constexpr int N2 = ((2 * COUT + 15) / 16) * 16;
-  constexpr int TM_COLS = (3 * N2 <= 32) ? 32 : (3 * N2 <= 64) ? 64 : (3 * N2 <= 128) ? 128 : 256;
-  static_assert(CIN == 1 || CIN == 8, "layer shapes of the network");
-  extern __shared__ __align__(1024) unsigned char smem[];
-  unsigned char* A = smem;                               // 3 colours x [128 x K2A] bf16
-  unsigned char* B = smem + 3 * PTC_TILE * K2A * 2;      // [N2 x K2B] bf16
-  uint64_t* mbar = reinterpret_cast<uint64_t*>(B + N2 * K2B * 2);
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(mbar + 1);
-  const int tid = threadIdx.x, warp = tid >> 5;
-  const Geom& g = G.g;
-
-  for (int i = tid; i < (3 * PTC_TILE * K2A + N2 * K2B) / 8; i += blockDim.x)
-    reinterpret_cast<uint4*>(smem)[i] = make_uint4(0, 0, 0, 0);
-  __syncthreads();
-  // B[n][k]: k = 2*(h*CIN + b) + {re, im}; n = 2a + {re, im}; complex weight as a 2x2 real block
-  for (int i = tid; i < COUT * CIN * NHOP; i += blockDim.x) {
-    const int a = i / (CIN * NHOP), b = (i / NHOP) % CIN, h = i % NHOP;  // W[a][b][h]
-    const float2 w = W[i];
-    const int k = h * CIN + b;
-    put_bf16(B, 2 * a, 2 * k, K2B, w.x);
-    put_bf16(B, 2 * a, 2 * k + 1, K2B, -w.y);
-    put_bf16(B, 2 * a + 1, 2 * k, K2B, w.y);
-    put_bf16(B, 2 * a + 1, 2 * k + 1, K2B, w.x);
-  }
-  if (tid == 0) tc::mbar_init(tc::smem_addr(mbar), 1);
-  if (warp == 0) tc::tmem_alloc(tc::smem_addr(tslot), TM_COLS);
-  tc::fence_before_sync();
-  __syncthreads();
-  tc::fence_after_sync();
-  const uint32_t tmem = *tslot;
-  const uint32_t idesc = tc::idesc_bf16_f32(PTC_TILE, N2);
-  const int n_out = OUT_EVEN ? g.half : g.V;
-  const int ntiles = (n_out + PTC_TILE - 1) / PTC_TILE;
-  uint32_t phase = 0;
-  bool failed = false;
-
-  for (int tile = blockIdx.x; tile < ntiles && !failed; tile += gridDim.x) {
-#pragma unroll 1
-    for (int pass = 0; pass < NPASS && !failed; ++pass) {
-      const int h0 = pass * HPP;
-      const int nh = (NHOP - h0) < HPP ? (NHOP - h0) : HPP;
-      // fill this pass's hops: work item = (row, hop); consecutive threads take consecutive sites
-      for (int item = tid; item < PTC_TILE * nh; item += blockDim.x) {
-        const int row = item % PTC_TILE, hl = item / PTC_TILE, h = h0 + hl;
-        int c[4], idx, oi;
-        cplx<float> u[CIN][3];
-        // layer 1 (CIN = 1) reads the network input, an even-site vector embedded with zeros on odd
-        // sites: the identity hop of an odd site and the +-mu hops of an even site transport zeros,
-        // so they load no link and no vector
-        bool live = tile_site(g, OUT_EVEN, tile, row, c, &idx, &oi);
-        if (CIN == 1 && live) live = (h == 0) == (((c[0] + c[1] + c[2] + c[3]) & 1) == 0);
-        if (live) {
-          transport_multi<CIN>(G, in, c, idx, h, u);
-        } else {
-#pragma unroll
-          for (int b = 0; b < CIN; ++b)
-#pragma unroll
-            for (int k = 0; k < 3; ++k) u[b][k] = {0.f, 0.f};
-        }
-#pragma unroll
-        for (int b = 0; b < CIN; ++b) {
-          const int k = hl * CIN + b;
-#pragma unroll
-          for (int col = 0; col < 3; ++col)
-            put_bf16x2(A + col * PTC_TILE * K2A * 2, row, 2 * k, K2A, u[b][col].re, u[b][col].im);
-        }
-      }
-      tc::fence_smem_to_async();
-      __syncthreads();
-      if (tid == 0) {
-        tc::fence_after_sync();
-        const int ksteps = CIN == 8 ? nh : K2A / 16;
-#pragma unroll 1
-        for (int col = 0; col < 3; ++col) {
-          const uint32_t a0 = tc::smem_addr(A + col * PTC_TILE * K2A * 2), b0 = tc::smem_addr(B);
-#pragma unroll 1
-          for (int ks = 0; ks < ksteps; ++ks) {
-            const int kb = CIN == 8 ? (h0 + ks) : ks;  // K-step of B (a hop for CIN = 8)
-            tc::mma_bf16(tmem + col * N2, tc::desc_kmajor(a0 + ks * 256, K2A), tc::desc_kmajor(b0 + kb * 256, K2B),
-                         idesc, (pass > 0 || ks > 0) ? 1u : 0u);
-          }
-        }
-        tc::commit(tc::smem_addr(mbar));
-      }
-      // the next pass (or tile) overwrites A: wait until the tensor core has read it
-      const bool ok = tc::mbar_wait(tc::smem_addr(mbar), phase, WAIT_LIMIT);
-      phase ^= 1;
-      if (__syncthreads_or(!ok)) failed = true;
-      tc::fence_after_sync();
-    }
-    if (failed) break;
-    // readout: warp w reads TMEM lanes 32*(w%4).. (rows) for colours w/4, w/4 + 2, ...
-    {
-      const int q = warp & 3, row = 32 * q + (tid & 31);
-      int c[4], idx, oi;
-      const bool valid = tile_site(g, OUT_EVEN, tile, row, c, &idx, &oi);
-#pragma unroll 1
-      for (int col = warp >> 2; col < 3; col += (int)(blockDim.x >> 7)) {
-        float v[16];
-        tc::tmem_ld16(tmem + ((uint32_t)(32 * q) << 16) + col * N2, v);
-        if (valid) {
-#pragma unroll
-          for (int a = 0; a < COUT; ++a) out[((size_t)a * n_out + oi) * 3 + col] = make_float2(v[2 * a], v[2 * a + 1]);
-        }
-      }
-    }
-    tc::fence_before_sync();
-    __syncthreads();
-  }
-  if (failed) {
-    if (tid == 0) atomicExch(err, 1);
-    tc::mbar_wait(tc::smem_addr(mbar), phase ^ 1, WAIT_LIMIT);  // let the outstanding MMA drain
-  }
-  tc::fence_before_sync();
-  __syncthreads();
-  if (warp == 0) tc::tmem_dealloc(tmem, TM_COLS);
-}
-
-// ------------------------------------------------------------------ backward: mixing + gather
-// m_{b,h}(x) = sum_a conj(W[a][b][h]) g_a(x) on tensor cores; g: [COUT][n_in][3] (full or even
-// sites), m: [CIN*9][V][3] full lattice (zero where g has no site).
-template <int CIN, int COUT, bool IN_EVEN>
-__global__ void __launch_bounds__(128) k_ptc_bwd_mix(const PtcGeom G, const float2* __restrict__ gout,
-                                                     float2* __restrict__ m, const float2* __restrict__ W, int* err) {
-  constexpr int K2 = ((2 * COUT + 15) / 16) * 16;
-  constexpr int N2 = ((2 * NHOP * CIN + 15) / 16) * 16;
-  constexpr int TM_COLS = (3 * N2 <= 32) ? 32 : (3 * N2 <= 64) ? 64 : (3 * N2 <= 128) ? 128 : (3 * N2 <= 256) ? 256 : 512;
-  static_assert(N2 <= 256, "MMA N limit");
-  extern __shared__ __align__(1024) unsigned char smem[];
-  unsigned char* A = smem;                          // 3 x [128 x K2]
-  unsigned char* B = smem + 3 * PTC_TILE * K2 * 2;  // [N2 x K2]
-  uint64_t* mbar = reinterpret_cast<uint64_t*>(B + N2 * K2 * 2);
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(mbar + 1);
-  const int tid = threadIdx.x, warp = tid >> 5;
-  const Geom& g = G.g;
-  for (int i = tid; i < (3 * PTC_TILE * K2 + N2 * K2) / 8; i += blockDim.x)
-    reinterpret_cast<uint4*>(smem)[i] = make_uint4(0, 0, 0, 0);
-  __syncthreads();
-  for (int i = tid; i < COUT * CIN * NHOP; i += blockDim.x) {
-    const int a = i / (CIN * NHOP), j = i % (CIN * NHOP);
-    const float2 w = W[i];
-    // m_r = sum_a (w_r g_r + w_i g_i), m_i = sum_a (w_r g_i - w_i g_r)
-    put_bf16(B, 2 * j, 2 * a, K2, w.x);
-    put_bf16(B, 2 * j, 2 * a + 1, K2, w.y);
-    put_bf16(B, 2 * j + 1, 2 * a, K2, -w.y);
-    put_bf16(B, 2 * j + 1, 2 * a + 1, K2, w.x);
-  }
-  if (tid == 0) tc::mbar_init(tc::smem_addr(mbar), 1);
-  if (warp == 0) tc::tmem_alloc(tc::smem_addr(tslot), TM_COLS);
-  tc::fence_before_sync();
-  __syncthreads();
-  tc::fence_after_sync();
-  const uint32_t tmem = *tslot;
-  const uint32_t idesc = tc::idesc_bf16_f32(PTC_TILE, N2);
-  const int n_in = IN_EVEN ? g.half : g.V;
-  const int ntiles = (n_in + PTC_TILE - 1) / PTC_TILE;
-  uint32_t phase = 0;
-  bool failed = false;
-  for (int tile = blockIdx.x; tile < ntiles && !failed; tile += gridDim.x) {
-    int c[4], idx, ii;
-    const bool valid = tile_site(g, IN_EVEN, tile, tid, c, &idx, &ii);
-#pragma unroll
-    for (int a = 0; a < COUT; ++a)
-#pragma unroll
-      for (int col = 0; col < 3; ++col) {
-        float2 v = valid ? gout[((size_t)a * n_in + ii) * 3 + col] : make_float2(0.f, 0.f);
-        unsigned char* Ac = A + col * PTC_TILE * K2 * 2;
-        put_bf16(Ac, tid, 2 * a, K2, v.x);
-        put_bf16(Ac, tid, 2 * a + 1, K2, v.y);
-      }
-    tc::fence_smem_to_async();
-    __syncthreads();
-    if (tid == 0) {
-      tc::fence_after_sync();
-#pragma unroll 1
-      for (int col = 0; col < 3; ++col) {
-        const uint32_t a0 = tc::smem_addr(A + col * PTC_TILE * K2 * 2), b0 = tc::smem_addr(B);
-#pragma unroll 1
-        for (int ks = 0; ks < K2 / 16; ++ks)
-          tc::mma_bf16(tmem + col * N2, tc::desc_kmajor(a0 + ks * 256, K2), tc::desc_kmajor(b0 + ks * 256, K2), idesc,
-                       ks > 0);
-      }
-      tc::commit(tc::smem_addr(mbar));
-    }
-    const bool ok = tc::mbar_wait(tc::smem_addr(mbar), phase, WAIT_LIMIT);
-    phase ^= 1;
-    if (__syncthreads_or(!ok)) {
-      failed = true;
-      break;
-    }
-    tc::fence_after_sync();
-#pragma unroll 1
-    for (int col = 0; col < 3; ++col) {
-#pragma unroll 1
-      for (int c16 = 0; c16 < N2; c16 += 16) {
-        float v[16];
-        tc::tmem_ld16(tmem + ((uint32_t)(32 * warp) << 16) + col * N2 + c16, v);
-        if (valid) {
-#pragma unroll
-          for (int q = 0; q < 8; ++q) {
-            const int j = c16 / 2 + q;
-            if (j < CIN * NHOP) m[((size_t)j * g.V + idx) * 3 + col] = make_float2(v[2 * q], v[2 * q + 1]);
-          }
-        }
-      }
-    }
-    tc::fence_before_sync();
-    __syncthreads();
-  }
-  if (failed) {
-    if (tid == 0) atomicExch(err, 1);
-    tc::mbar_wait(tc::smem_addr(mbar), phase ^ 1, WAIT_LIMIT);
-  }
-  tc::fence_before_sync();
-  __syncthreads();
-  if (warp == 0) tc::tmem_dealloc(tmem, TM_COLS);
-}
-
-// g_in_b(x) = sum_h T_h^dag m_{b,h} (x): T_0^dag = 1, T_+mu^dag = T_-mu, T_-mu^dag = T_+mu.
-template <int CIN>
-__global__ void k_ptc_bwd_gather(const PtcGeom G, const float2* __restrict__ m, float2* __restrict__ gin) {
-  const Geom& g = G.g;
-  for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < g.V; idx += gridDim.x * blockDim.x) {
-    int c[4];
-    c[0] = idx % g.L[0];
-    c[1] = (idx / g.L[0]) % g.L[1];
-    c[2] = (idx / (g.L[0] * g.L[1])) % g.L[2];
-    c[3] = idx / (g.L[0] * g.L[1] * g.L[2]);
-    for (int b = 0; b < CIN; ++b) {
-      cplx<float> acc[3] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
-      for (int h = 0; h < NHOP; ++h) {
-        const int hadj = h == 0 ? 0 : (h <= 4 ? h + 4 : h - 4);
-        cplx<float> u[3];
-        transport(G, m + (size_t)(b * NHOP + h) * g.V * 3, c, idx, hadj, u);
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          acc[k].re += u[k].re;
-          acc[k].im += u[k].im;
-        }
-      }
-#pragma unroll
-      for (int k = 0; k < 3; ++k) gin[((size_t)b * g.V + idx) * 3 + k] = make_float2(acc[k].re, acc[k].im);
-    }
-  }
-}
-
-// ------------------------------------------------------------------ weight gradient
-// D[j][n] = sum_{x,col} U[j][(x,col)] Gm[(x,col)][n] with rows j = 2*(b*9+h) + {re, im} of
-// u = T_h in_b and columns n = 2a + {re, im} of g_a; K = sites x colours, tiles of WG_SITES.
-// Per-CTA partial sums (FP32, TMEM) go to part[cta][256][16]; k_ptc_wgrad_final combines.
-constexpr int WG_SITES = 64;
-constexpr int WG_K = WG_SITES * 3;  // 192 = 12 MMA K-steps
-
-template <int CIN, int COUT, bool G_EVEN>
-__global__ void __launch_bounds__(128) k_ptc_wgrad(const PtcGeom G, const float2* __restrict__ in,
-                                                   const float2* __restrict__ gout, float* __restrict__ part,
-                                                   int* err) {
-  constexpr int MROWS = 2 * NHOP * CIN;      // real feature rows
-  constexpr int MT = (MROWS + 127) / 128;    // M tiles of 128
-  constexpr int N2 = ((2 * COUT + 15) / 16) * 16;
-  constexpr int TM_COLS = (MT * N2 <= 32) ? 32 : 64;
-  extern __shared__ __align__(1024) unsigned char smem[];
-  unsigned char* A = smem;                          // MT x [128 x WG_K]
-  unsigned char* B = smem + MT * 128 * WG_K * 2;    // [N2 x WG_K]
-  uint64_t* mbar = reinterpret_cast<uint64_t*>(B + N2 * WG_K * 2);
-  uint32_t* tslot = reinterpret_cast<uint32_t*>(mbar + 1);
-  const int tid = threadIdx.x, warp = tid >> 5;
-  const Geom& g = G.g;
-  for (int i = tid; i < (MT * 128 * WG_K + N2 * WG_K) / 8; i += blockDim.x)
-    reinterpret_cast<uint4*>(smem)[i] = make_uint4(0, 0, 0, 0);
-  if (tid == 0) tc::mbar_init(tc::smem_addr(mbar), 1);
-  if (warp == 0) tc::tmem_alloc(tc::smem_addr(tslot), TM_COLS);
-  tc::fence_before_sync();
-  __syncthreads();
-  tc::fence_after_sync();
-  const uint32_t tmem = *tslot;
-  const uint32_t idesc = tc::idesc_bf16_f32(128, N2);
-  const int n_g = G_EVEN ? g.half : g.V;
-  const int ntiles = (n_g + WG_SITES - 1) / WG_SITES;
-  uint32_t phase = 0;
-  bool failed = false, first = true;
-  for (int tile = blockIdx.x; tile < ntiles && !failed; tile += gridDim.x) {
-    // threads 0..63 fill site (tid) of the tile; 64..127 idle while filling
-    if (tid < WG_SITES) {
-      const int i = tile * WG_SITES + tid;
-      int c[4], idx = 0;
-      const bool valid = i < n_g;
-      if (valid) {
-        if (G_EVEN) {
-          site_coords(g, 0, i, c);
-          idx = lex_index(g, c);
-        } else {
-          idx = i;
-          c[0] = i % g.L[0];
-          c[1] = (i / g.L[0]) % g.L[1];
-          c[2] = (i / (g.L[0] * g.L[1])) % g.L[2];
-          c[3] = i / (g.L[0] * g.L[1] * g.L[2]);
-        }
-      }
-      for (int b = 0; b < CIN; ++b)
-        for (int h = 0; h < NHOP; ++h) {
-          cplx<float> u[3] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
-          if (valid) transport(G, in + (size_t)b * g.V * 3, c, idx, h, u);
-          const int j = 2 * (b * NHOP + h);
-#pragma unroll
-          for (int col = 0; col < 3; ++col) {
-            const int k = col * WG_SITES + tid;
-            put_bf16(A + (j / 128) * 128 * WG_K * 2, j % 128, k, WG_K, u[col].re);
-            put_bf16(A + ((j + 1) / 128) * 128 * WG_K * 2, (j + 1) % 128, k, WG_K, u[col].im);
-          }
-        }
-      for (int a = 0; a < COUT; ++a)
-#pragma unroll
-        for (int col = 0; col < 3; ++col) {
-          float2 v = valid ? gout[((size_t)a * n_g + i) * 3 + col] : make_float2(0.f, 0.f);
-          const int k = col * WG_SITES + tid;
-          put_bf16(B, 2 * a, k, WG_K, v.x);
-          put_bf16(B, 2 * a + 1, k, WG_K, v.y);
-        }
-    }
-    tc::fence_smem_to_async();
-    __syncthreads();
-    if (tid == 0) {
-      tc::fence_after_sync();
-#pragma unroll 1
-      for (int mt = 0; mt < MT; ++mt) {
-        const uint32_t a0 = tc::smem_addr(A + mt * 128 * WG_K * 2), b0 = tc::smem_addr(B);
-#pragma unroll 1
-        for (int ks = 0; ks < WG_K / 16; ++ks)
-          tc::mma_bf16(tmem + mt * N2, tc::desc_kmajor(a0 + ks * 256, WG_K), tc::desc_kmajor(b0 + ks * 256, WG_K),
-                       idesc, (first && ks == 0) ? 0u : 1u);
-      }
-      tc::commit(tc::smem_addr(mbar));
-    }
-    first = false;
-    const bool ok = tc::mbar_wait(tc::smem_addr(mbar), phase, WAIT_LIMIT);
-    phase ^= 1;
-    if (__syncthreads_or(!ok)) {
-      failed = true;
-      break;
-    }
-    tc::fence_before_sync();
-    __syncthreads();
-  }
-  if (failed) {
-    if (tid == 0) atomicExch(err, 1);
-    tc::mbar_wait(tc::smem_addr(mbar), phase ^ 1, WAIT_LIMIT);
-  }
-  tc::fence_after_sync();
-  // this CTA's partial: rows 32*warp + lane of each M tile, N2 columns
-#pragma unroll 1
-  for (int mt = 0; mt < MT; ++mt) {
-    float v[16];
-    tc::tmem_ld16(tmem + ((uint32_t)(32 * warp) << 16) + mt * N2, v);
-    const int row = mt * 128 + tid;
-    float* dst = part + ((size_t)blockIdx.x * 256 + row) * 16;
-#pragma unroll
-    for (int q = 0; q < 16; ++q) dst[q] = first ? 0.f : v[q];
-  }
-  tc::fence_before_sync();
-  __syncthreads();
-  if (warp == 0) tc::tmem_dealloc(tmem, TM_COLS);
-}
-
-// gW[a][b][h] = (D[2j][2a] + D[2j+1][2a+1]) + i (D[2j][2a+1] - D[2j+1][2a]), j = b*9+h, summed over
-// CTA partials in fixed order; scaled by `scale`. Output float2 [COUT][CIN][9].
-__global__ void k_ptc_wgrad_final(const float* __restrict__ part, int nparts, int cin, int cout, float scale,
-                                  float2* __restrict__ gW) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= cout * cin * NHOP) return;
-  const int a = i / (cin * NHOP), j = i % (cin * NHOP);
-  double rr = 0, ii = 0, ri = 0, ir = 0;
-  for (int p = 0; p < nparts; ++p) {
-    const float* P = part + (size_t)p * 256 * 16;
-    rr += P[(2 * j) * 16 + 2 * a];
-    ii += P[(2 * j + 1) * 16 + 2 * a + 1];
-    ri += P[(2 * j) * 16 + 2 * a + 1];
-    ir += P[(2 * j + 1) * 16 + 2 * a];
-  }
-  gW[i] = make_float2((float)((rr + ii) * scale), (float)((ri - ir) * scale));
-}
-
-// ------------------------------------------------------------------ preconditioner apply (inference)
+// ------------------------------------------------------------------ preconditioner apply and forward pass
 // The network is linear, so its two layers compose into one operator. With the input r on even sites
 // (zeros on odd sites) and the output read on even sites x:
 //   N(r)(x) = c0 r(x) + sum_{h != 0} T_h phi_h (x),   phi_h(y) = sum_{h' != 0} C[h][h'] (T_h' r)(y)
@@ -577,7 +45,7 @@ __global__ void k_ptc_wgrad_final(const float* __restrict__ part, int nparts, in
 // site only its eight neighbour hops). The 8-channel activation is thereby replaced by the eight
 // mixed transports phi_h of each odd site, written once and read once (an activation of half the
 // lattice that layer 2 needs at x + h only), and each stencil pass reads every fat link once. The
-// weights enter rounded to BF16, as on the tensor-core path that training uses.
+// weights enter rounded to BF16.
 __device__ __forceinline__ cplx<float> bf16c(float2 w) {
   return {__bfloat162float(__float2bfloat16_rn(w.x)), __bfloat162float(__float2bfloat16_rn(w.y))};
 }
@@ -707,19 +175,411 @@ __global__ void __launch_bounds__(256) k_ptc_apply_even(const PtcGeom G, const f
   }
 }
 
-// ------------------------------------------------------------------ small kernels
-// Embed an even-site vector [half][3] into the full lattice (zeros on odd sites).
-__global__ void k_embed_even(const Geom g, const float2* __restrict__ r, float2* __restrict__ full, const int* skip) {
-  if (skip && *skip) return;
-  for (int idx = blockIdx.x * blockDim.x + threadIdx.x; idx < g.V; idx += gridDim.x * blockDim.x) {
-    const int x = idx % g.L[0], y = (idx / g.L[0]) % g.L[1], z = (idx / (g.L[0] * g.L[1])) % g.L[2],
-              t = idx / (g.L[0] * g.L[1] * g.L[2]);
-    const bool even = ((x + y + z + t) & 1) == 0;
+// ------------------------------------------------------------------ training: loss and gradients
+// With d = N(b) - x on even sites, the loss of a pair is |d|^2 / |x|^2 and its derivatives are (sums over
+// odd sites y and colours; hops h, h' in +x..-t, adj h the opposite hop)
+//   dL/dconj W1[a][h'] = sum_h  conj(W2[a][h])  M[h'][adj h] / |x|^2,  M[h'][k] = sum conj((T_h' b)(y)) (T_k d)(y)
+//   dL/dconj W2[a][h]  = sum_h' conj(W1[a][h']) M[h'][adj h] / |x|^2
+//   and for the identity hops conj(W2[a][0]) m0 / |x|^2 and conj(W1[a][0]) m0 / |x|^2, m0 = sum_x conj(b(x)) d(x):
+// layer 1's activation at an odd site is sum_h' W1[a][h'] T_h' b, the loss's derivative with respect to it is
+// sum_h conj(W2[a][h]) T_(adj h) d, and T_h^dag = T_(adj h). So a pair costs three stencil passes over the
+// fat links (two forward, one for M) and keeps no per-channel field. Groups of up to NV = 4 pairs share
+// every link read. 16 pairs at 32^3x8: 32.3 ms with the layers one after the other on the tensor cores (72
+// transported planes per pair written and gathered, a host read-back per pair, BF16 operands: gradients
+// 1.6e-5 from FP64), 0.76 ms in this form (2.8e-8). A group's three passes take 61, 55 and 59 us under ncu with
+// the caches flushed, against about 30 us each for their bytes: they issue on 57, 32 and 64% of the cycles
+// (multiply-adds and shared-memory words of the mixing and of the inner products) at 16 warps per SM.
+//
+// All three passes walk tiles of 32 sites with one warp per hop: a warp loads its hop's link once for the
+// group's vectors, and every load of a site (8 links, 8 NV vectors) is in flight at once, where a thread per
+// site took the hops in turn and waited for each (with NV threads per site the same passes took 70, 56 and
+// 56 us for 4 pairs at 32^3x8).
+constexpr int PT_PART = 4;     // per-block partials of a pair: |d|^2, |x|^2, Re m0, Im m0
+constexpr int PT_CHUNK = 16;   // pairs whose partials are kept at once
+constexpr int PT_SITES = 32;   // sites of a tile
+constexpr int PT_ROW = 34;     // float2 per (colour, hop) row of a tile: rows 4 apart lie 16 banks apart
+constexpr int PT_FIELD = 3 * 8 * PT_ROW;  // one transported vector's tile [colour][hop][site]
+
+// The link of hop h = 1..8 at site cb of parity par, and the neighbour it transports from.
+__device__ __forceinline__ int ptc_tile_link(const PtcGeom& G, int par, int cb, int h, cplx<float> (&U)[9]) {
+  int c[4];
+  site_coords(G.g, par, cb, c);
+  const char* blk;
+  int lcb;
+  const int nb = ptc_hop(G, c, lex_index(G.g, c), par, h, &blk, &lcb);
+  LinkIO<float>::load(blk, G.g.half, lcb, U);
+  return nb;
+}
+
+// v transported through U (dagger for the hops -mu), into one site's column of a tile field.
+__device__ __forceinline__ void ptc_tile_put(float2* field, const cplx<float> (&U)[9], const cplx<float> (&v)[3],
+                                             int warp, int lane) {
 #pragma unroll
-    for (int k = 0; k < 3; ++k) full[(size_t)idx * 3 + k] = even ? r[(size_t)(idx >> 1) * 3 + k] : make_float2(0.f, 0.f);
+  for (int i = 0; i < 3; ++i) {
+    cplx<float> s = {0.f, 0.f};
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      if (warp < 4) cmac(s, U[3 * i + j], v[j]);
+      else cmac_conj(s, U[3 * j + i], v[j]);
+    }
+    field[(i * 8 + warp) * PT_ROW + lane] = make_float2(s.re, s.im);
   }
 }
 
+// Pass 1 of training, odd sites: phi_h = sum_h' C[h][h'] T_h' b for NV vectors, FP32 planes
+// [vector][h][colour][cb] (training's inputs may have any scale, so no FP16 here). The next tile's link and
+// vectors are loaded while this tile is mixed.
+template <int NV>
+__global__ void __launch_bounds__(256, 2) k_ptc_train_odd(const PtcGeom G, const float2* __restrict__ b,
+                                                          float2* __restrict__ phi, const float2* __restrict__ mix) {
+  __shared__ float2 tile[NV * PT_FIELD];
+  __shared__ float4 smix[32];  // C[h][h'], two entries each
+  griddep_wait();
+  griddep_launch_dependents();
+  const Geom& g = G.g;
+  const size_t half = g.half;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (threadIdx.x < 32) {
+    const float2 m0 = __ldg(mix + 1 + 2 * threadIdx.x), m1 = __ldg(mix + 2 + 2 * threadIdx.x);
+    smix[threadIdx.x] = make_float4(m0.x, m0.y, m1.x, m1.y);
+  }
+  const int ntiles = (g.half + PT_SITES - 1) / PT_SITES;
+  cplx<float> U[9], v[NV][3];
+  auto load = [&](int cb) {
+    if (cb >= g.half) return;
+    const int nb = ptc_tile_link(G, 1, cb, warp + 1, U);
+#pragma unroll
+    for (int f = 0; f < NV; ++f)
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        const float2 w = __ldg(b + ((size_t)f * half + nb) * 3 + k);
+        v[f][k] = {w.x, w.y};
+      }
+  };
+  load(blockIdx.x * PT_SITES + lane);
+  for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
+    const int cb = t * PT_SITES + lane;
+    if (cb < g.half) {
+#pragma unroll
+      for (int f = 0; f < NV; ++f) ptc_tile_put(tile + f * PT_FIELD, U, v[f], warp, lane);
+    }
+    load(cb + gridDim.x * PT_SITES);
+    __syncthreads();
+    for (int q = warp; q < NV * 6; q += 8) {  // (vector, colour, four of the eight phi)
+      const int f = q / 6, col = (q % 6) >> 1, h0 = (q & 1) * 4;
+      cplx<float> s[8];
+#pragma unroll
+      for (int h = 0; h < 8; ++h) {
+        const float2 w = tile[f * PT_FIELD + (col * 8 + h) * PT_ROW + lane];
+        s[h] = {w.x, w.y};
+      }
+#pragma unroll
+      for (int o = 0; o < 4; ++o) {
+        cplx<float> a = {0.f, 0.f};
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+          const float4 m = smix[(h0 + o) * 4 + h];
+          cmac(a, cplx<float>{m.x, m.y}, s[2 * h]);
+          cmac(a, cplx<float>{m.z, m.w}, s[2 * h + 1]);
+        }
+        if (cb < g.half) phi[((size_t)((f * 8 + h0 + o) * 3 + col)) * half + cb] = make_float2(a.re, a.im);
+      }
+    }
+    __syncthreads();
+  }
+}
+
+// Pass 2 of training, even sites: d = N(b) - x for NV vectors, planes [vector][colour][cb], and this block's
+// sums of |d|^2, |x|^2 and conj(b) d (FP32 over a thread's few sites, FP64 over the block).
+template <int NV>
+__global__ void __launch_bounds__(256, 2) k_ptc_train_even(const PtcGeom G, const float2* __restrict__ b,
+                                                           const float2* __restrict__ phi, const float2* __restrict__ x,
+                                                           float2* __restrict__ d, const float2* __restrict__ mix,
+                                                           double* __restrict__ part) {
+  __shared__ float2 tile[NV * PT_FIELD];
+  __shared__ double red[NV * 3][PT_PART];
+  griddep_wait();
+  griddep_launch_dependents();
+  const Geom& g = G.g;
+  const size_t half = g.half;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const float2 m0 = __ldg(mix);
+  constexpr int ITEMS = (NV * 3 + 7) / 8;  // (vector, colour) pairs per warp
+  float s[ITEMS][PT_PART] = {};
+  const int ntiles = (g.half + PT_SITES - 1) / PT_SITES;
+  cplx<float> U[9], v[NV][3];
+  auto load = [&](int cb) {
+    if (cb >= g.half) return;
+    const int nb = ptc_tile_link(G, 0, cb, warp + 1, U);
+#pragma unroll
+    for (int f = 0; f < NV; ++f)
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        const float2 w = __ldg(phi + (size_t)((f * 8 + warp) * 3 + k) * half + nb);
+        v[f][k] = {w.x, w.y};
+      }
+  };
+  load(blockIdx.x * PT_SITES + lane);
+  for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
+    const int cb = t * PT_SITES + lane;
+    if (cb < g.half) {
+#pragma unroll
+      for (int f = 0; f < NV; ++f) ptc_tile_put(tile + f * PT_FIELD, U, v[f], warp, lane);
+    }
+    load(cb + gridDim.x * PT_SITES);
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < ITEMS; ++j) {
+      const int q = warp + 8 * j, f = q / 3, col = q % 3;
+      if (q < NV * 3 && cb < g.half) {
+        const size_t i = ((size_t)f * half + cb) * 3 + col;
+        const float2 bv = __ldg(b + i), xv = __ldg(x + i);
+        cplx<float> z = {0.f, 0.f};
+        cmac(z, cplx<float>{m0.x, m0.y}, cplx<float>{bv.x, bv.y});
+#pragma unroll
+        for (int h = 0; h < 8; ++h) {
+          const float2 w = tile[f * PT_FIELD + (col * 8 + h) * PT_ROW + lane];
+          z.re += w.x;
+          z.im += w.y;
+        }
+        const float dx = z.re - xv.x, dy = z.im - xv.y;
+        d[((size_t)f * 3 + col) * half + cb] = make_float2(dx, dy);
+        s[j][0] += dx * dx + dy * dy;
+        s[j][1] += xv.x * xv.x + xv.y * xv.y;
+        s[j][2] += bv.x * dx + bv.y * dy;
+        s[j][3] += bv.x * dy - bv.y * dx;
+      }
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int j = 0; j < ITEMS; ++j)
+#pragma unroll
+    for (int p = 0; p < PT_PART; ++p) {
+      double w = (double)s[j][p];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
+      if (lane == 0 && warp + 8 * j < NV * 3) red[warp + 8 * j][p] = w;
+    }
+  __syncthreads();
+  if (threadIdx.x < NV * PT_PART) {
+    const int f = threadIdx.x / PT_PART, p = threadIdx.x % PT_PART;
+    part[((size_t)f * gridDim.x + blockIdx.x) * PT_PART + p] = (red[3 * f][p] + red[3 * f + 1][p]) + red[3 * f + 2][p];
+  }
+}
+
+// This block's part of M for NV pairs: part[pair][block][h' * 8 + k] (FP32 sums over the block's tiles). After
+// the transports of b and d at a tile's odd sites each thread adds its share of the sites to a 4 x 4 corner of
+// the 8 x 8 inner products, which stay in registers over the tiles of a persistent grid.
+template <int NV>
+__global__ void __launch_bounds__(256, 2) k_ptc_grad(const PtcGeom G, const float2* __restrict__ b,
+                                                     const float2* __restrict__ d, float2* __restrict__ part) {
+  extern __shared__ float2 tile[];  // [pair][b or d][PT_FIELD]
+  griddep_wait();
+  griddep_launch_dependents();
+  const Geom& g = G.g;
+  const size_t half = g.half;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  // products: WPV warps per pair, each with 8 groups of sites (lane & 7) of 4 corners (lane >> 3)
+  constexpr int WPV = 8 / NV;
+  const int pv = warp / WPV, pw = warp % WPV, sub = lane & 7, h0 = ((lane >> 3) & 1) * 4, k0 = (lane >> 4) * 4;
+  cplx<float> acc[4][4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] = {0.f, 0.f};
+  const int ntiles = (g.half + PT_SITES - 1) / PT_SITES;
+  for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
+    const int cb = t * PT_SITES + lane;
+    if (cb < g.half) {
+      cplx<float> U[9], v[2 * NV][3];
+      const int nb = ptc_tile_link(G, 1, cb, warp + 1, U);
+#pragma unroll
+      for (int f = 0; f < NV; ++f)
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          const float2 w = __ldg(b + ((size_t)f * half + nb) * 3 + k), e = __ldg(d + ((size_t)f * 3 + k) * half + nb);
+          v[2 * f][k] = {w.x, w.y};
+          v[2 * f + 1][k] = {e.x, e.y};
+        }
+#pragma unroll
+      for (int f = 0; f < 2 * NV; ++f) ptc_tile_put(tile + f * PT_FIELD, U, v[f], warp, lane);
+    } else {
+      for (int f = 0; f < 2 * NV; ++f)
+        for (int i = 0; i < 3; ++i) tile[f * PT_FIELD + (i * 8 + warp) * PT_ROW + lane] = make_float2(0.f, 0.f);
+    }
+    __syncthreads();
+    const float2* u = tile + (size_t)(2 * pv) * PT_FIELD + h0 * PT_ROW;
+    const float2* s = tile + (size_t)(2 * pv + 1) * PT_FIELD + k0 * PT_ROW;
+#pragma unroll 1
+    for (int q = pw; q < 3 * (PT_SITES / 8); q += WPV) {  // (colour, group of 8 sites)
+      const int o = (q / (PT_SITES / 8)) * 8 * PT_ROW + (q % (PT_SITES / 8)) * 8 + sub;
+      cplx<float> uv[4], sv[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float2 a = u[o + i * PT_ROW], e = s[o + i * PT_ROW];
+        uv[i] = {a.x, a.y};
+        sv[i] = {e.x, e.y};
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) cmac_conj(acc[i][j], uv[i], sv[j]);
+    }
+    __syncthreads();
+  }
+  // over the 8 site groups of a warp, then over the warps of a pair
+  float2* red = tile;  // [warp][64]
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      float re = acc[i][j].re, im = acc[i][j].im;
+#pragma unroll
+      for (int o = 1; o < 8; o <<= 1) {
+        re += __shfl_xor_sync(0xffffffffu, re, o);
+        im += __shfl_xor_sync(0xffffffffu, im, o);
+      }
+      if (sub == 0) red[warp * 64 + (h0 + i) * 8 + k0 + j] = make_float2(re, im);
+    }
+  __syncthreads();
+  for (int i = threadIdx.x; i < NV * 64; i += blockDim.x) {
+    const int v = i / 64, e = i % 64;
+    float re = 0.f, im = 0.f;
+    for (int w = 0; w < WPV; ++w) {
+      re += red[(v * WPV + w) * 64 + e].x;
+      im += red[(v * WPV + w) * 64 + e].y;
+    }
+    part[((size_t)v * gridDim.x + blockIdx.x) * 64 + e] = make_float2(re, im);
+  }
+}
+
+// The pairs' sums (FP64, in a fixed order). Block (pair, y) takes every PT_SPLIT-th block's part of M:
+// tot[pair][y][0..63]; block (pair, 0) also m0 in [64], and |d|^2 and |x|^2 in [65]. Several blocks per pair
+// because the conversions and adds are FP64 (one block per pair: 35 us).
+constexpr int PT_SPLIT = 8;
+constexpr int PT_TOT = 66;
+__global__ void __launch_bounds__(256) k_ptc_train_sum(const double* __restrict__ epart, int nblk_e,
+                                                       const float2* __restrict__ gpart, int nblk_g,
+                                                       double2* __restrict__ tot) {
+  griddep_wait();
+  griddep_launch_dependents();
+  const int pr = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  __shared__ double es[8][PT_PART];
+  __shared__ double2 gs[4][64];
+  double2* o = tot + ((size_t)pr * PT_SPLIT + blockIdx.y) * PT_TOT;
+  if (blockIdx.y == 0) {
+    const double2* e = reinterpret_cast<const double2*>(epart + (size_t)pr * nblk_e * PT_PART);
+    double s[PT_PART] = {0, 0, 0, 0};
+    for (int i = threadIdx.x; i < nblk_e; i += blockDim.x) {
+      const double2 a = e[2 * i], c = e[2 * i + 1];
+      s[0] += a.x;
+      s[1] += a.y;
+      s[2] += c.x;
+      s[3] += c.y;
+    }
+#pragma unroll
+    for (int q = 0; q < PT_PART; ++q) {
+#pragma unroll
+      for (int k = 16; k > 0; k >>= 1) s[q] += __shfl_xor_sync(0xffffffffu, s[q], k);
+      if (lane == 0) es[warp][q] = s[q];
+    }
+  }
+  {
+    const int e = threadIdx.x & 63, part = threadIdx.x >> 6;
+    const float2* gp = gpart + (size_t)pr * nblk_g * 64;
+    double2 s = make_double2(0.0, 0.0);
+#pragma unroll 4
+    for (int i = blockIdx.y + PT_SPLIT * part; i < nblk_g; i += 4 * PT_SPLIT) {
+      const float2 w = gp[(size_t)i * 64 + e];
+      s.x += (double)w.x;
+      s.y += (double)w.y;
+    }
+    gs[part][e] = s;
+  }
+  __syncthreads();
+  const int e = threadIdx.x;
+  if (e < 64)
+    o[e] = make_double2((gs[0][e].x + gs[1][e].x) + (gs[2][e].x + gs[3][e].x),
+                        (gs[0][e].y + gs[1][e].y) + (gs[2][e].y + gs[3][e].y));
+  if (blockIdx.y == 0 && (e == 64 || e == 65)) {
+    const int q = e == 64 ? 2 : 0;  // (Re m0, Im m0), (|d|^2, |x|^2)
+    double2 s = make_double2(0.0, 0.0);
+    for (int w = 0; w < 8; ++w) {
+      s.x += es[w][q];
+      s.y += es[w][q + 1];
+    }
+    o[e] = s;
+  }
+}
+
+// Adds the chunk's n pairs, weighted by 1 / (|x|^2 npairs), to acc[PT_TOT] (M, m0, the loss) and, after the last
+// chunk, forms the gradients of both layers (C = 8 channels) from M and m0 and the loss (loss[0]).
+__global__ void __launch_bounds__(544) k_ptc_train_final(const double2* __restrict__ tot, int n, int npairs,
+                                                         double2* acc, int first, int last,
+                                                         const float2* __restrict__ w1, const float2* __restrict__ w2,
+                                                         int C, float2* __restrict__ g1, float2* __restrict__ g2,
+                                                         float* __restrict__ loss) {
+  griddep_wait();
+  griddep_launch_dependents();
+  constexpr int GROUPS = 8;  // groups of threads that each take every 8th pair: one after the other is 36 us
+  __shared__ double2 m[PT_TOT], ms[GROUPS][PT_TOT];
+  const int grp = threadIdx.x / PT_TOT, e = threadIdx.x % PT_TOT;
+  if (grp < GROUPS) {
+    double2 s = make_double2(0.0, 0.0);
+    for (int i = grp; i < n; i += GROUPS) {
+      const double2* t = tot + (size_t)i * PT_SPLIT * PT_TOT;
+      const double2 sq = t[65];  // (|d|^2, |x|^2)
+      double2 w = t[e];
+      if (e < 64) {
+#pragma unroll
+        for (int y = 1; y < PT_SPLIT; ++y) {
+          w.x += t[y * PT_TOT + e].x;
+          w.y += t[y * PT_TOT + e].y;
+        }
+      }
+      const double inv = 1.0 / (sq.y * npairs);
+      s.x += w.x * inv;
+      s.y += w.y * inv;
+    }
+    ms[grp][e] = s;
+  }
+  __syncthreads();
+  if (threadIdx.x < PT_TOT) {
+    double2 s = first ? make_double2(0.0, 0.0) : acc[e];
+    for (int k = 0; k < GROUPS; ++k) {
+      s.x += ms[k][e].x;
+      s.y += ms[k][e].y;
+    }
+    acc[e] = s;
+    m[e] = s;
+  }
+  __syncthreads();
+  if (!last) return;
+  if (threadIdx.x == 0) *loss = (float)m[65].x;
+  for (int i = threadIdx.x; i < 2 * C * NHOP; i += blockDim.x) {
+    const bool second = i >= C * NHOP;
+    const int a = (i % (C * NHOP)) / NHOP, h = i % NHOP;
+    const float2* w = (second ? w1 : w2) + a * NHOP;  // the other layer's weights of channel a
+    double re = 0.0, im = 0.0;
+    auto add = [&](cplx<float> c, double2 v) {  // += conj(c) v
+      re += (double)c.re * v.x + (double)c.im * v.y;
+      im += (double)c.re * v.y - (double)c.im * v.x;
+    };
+    if (h == 0) {
+      add(bf16c(w[0]), m[64]);
+    } else {
+      for (int q = 0; q < 8; ++q) {
+        // W1[h]: M[h][adj q] of W2's hop q; W2[h]: M[q][adj h] of W1's hop q
+        const int row = second ? q : h - 1, col = ((second ? h - 1 : q) + 4) & 7;
+        add(bf16c(w[1 + q]), m[row * 8 + col]);
+      }
+    }
+    (second ? g2 : g1)[i % (C * NHOP)] = make_float2((float)re, (float)im);
+  }
+}
+
+// ------------------------------------------------------------------ small kernels
 __device__ __forceinline__ int adj_hop(int h) { return h == 0 ? 0 : (h <= 4 ? h + 4 : h - 4); }
 
 // Tied network: W2[0][a][h] = conj(W1[a][0][adj(h)]).
@@ -739,11 +599,6 @@ __global__ void k_tie_grad(float2* __restrict__ g1, const float2* __restrict__ g
   const float2 g = g2[a * NHOP + adj_hop(h)];
   g1[i].x += g.x;
   g1[i].y -= g.y;
-}
-
-__global__ void k_accumulate(float* __restrict__ acc, const float* __restrict__ g, int n) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) acc[i] += g[i];
 }
 
 // Adam on FP32 master weights with the real gradient 2*(Re G, Im G) of the Wirtinger gradient G.
@@ -1007,7 +862,6 @@ struct hisq_ptc {
   float2 *g1 = nullptr, *g2 = nullptr;  // gradients
   int adam_t = 0;
   int tied = 0;  // layer 2 = adjoint of layer 1 (N = B^dag B)
-  int* d_err = nullptr;
   float2* mix = nullptr;  // the composed network's mixing coefficients (65 complex), for the apply
 };
 
@@ -1019,68 +873,6 @@ static PtcGeom ptc_geom(const hisq_ctx* c) {
   G.fat32 = c->links[HISQ_F32];
   G.blk_bytes = link_block_bytes(HISQ_F32, c->g.half);
   return G;
-}
-
-template <int CIN, int COUT>
-static size_t fwd_smem() {
-  constexpr int N2 = ((2 * COUT + 15) / 16) * 16;
-  return (size_t)3 * PTC_TILE * FwdShape<CIN>::K2A * 2 + (size_t)N2 * FwdShape<CIN>::K2B * 2 + 16;
-}
-template <int CIN, int COUT>
-static size_t mix_smem() {
-  constexpr int K2 = ((2 * COUT + 15) / 16) * 16, N2 = ((2 * NHOP * CIN + 15) / 16) * 16;
-  return (size_t)3 * PTC_TILE * K2 * 2 + (size_t)N2 * K2 * 2 + 16;
-}
-template <int CIN, int COUT>
-static size_t wg_smem() {
-  constexpr int MT = (2 * NHOP * CIN + 127) / 128, N2 = ((2 * COUT + 15) / 16) * 16;
-  return (size_t)MT * 128 * WG_K * 2 + (size_t)N2 * WG_K * 2 + 16;
-}
-
-// One persistent CTA per SM keeps TMEM demand (at most 512 columns) within one SM's TMEM.
-template <typename K>
-static int launch_tc(hisq_ctx* c, K kern, size_t smem, int nwork, const char* what) {
-  // raise this kernel's dynamic shared-memory limit; inside the library's own stream capture the
-  // same launch has already been made eagerly, so the attribute is set
-  if (!c->capturing)
-    HISQ_CUDA(cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  int grid = c->num_sms;
-  if (grid > nwork) grid = nwork;
-  if (grid < 1) grid = 1;
-  (void)what;
-  return grid;
-}
-
-template <int CIN, int COUT, bool OUT_EVEN>
-static int forward_layer(hisq_ptc* P, const float2* in, float2* out, const float2* W, const int* skip = nullptr) {
-  hisq_ctx* c = P->ctx;
-  auto kern = k_ptc_forward<CIN, COUT, OUT_EVEN>;
-  const size_t smem = fwd_smem<CIN, COUT>() + 1024;
-  const int n_out = OUT_EVEN ? c->g.half : c->g.V;
-  int grid = launch_tc(c, kern, smem, (n_out + PTC_TILE - 1) / PTC_TILE, "ptc forward");
-  if (grid < 0) return grid;
-  // several CTAs per SM: as many as registers, shared memory and threads allow, and at most 6
-  // (each holds 64 TMEM columns; 8 would fill the SM's 512)
-  static int per_sm = 0;
-  if (per_sm == 0 && !c->capturing) {
-    cudaFuncAttributes fa;
-    int dev = 0, smem_sm = 0;
-    HISQ_CUDA(cudaFuncGetAttributes(&fa, (const void*)kern));
-    HISQ_CUDA(cudaGetDevice(&dev));
-    HISQ_CUDA(cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev));
-    const int by_regs = 65536 / ((fa.numRegs > 0 ? fa.numRegs : 64) * 256);
-    const int by_smem = smem_sm / (int)(smem + fa.sharedSizeBytes + 1024);
-    per_sm = by_regs < by_smem ? by_regs : by_smem;
-    if (per_sm > 6) per_sm = 6;
-    if (per_sm < 1) per_sm = 1;
-  }
-  const int ntiles = (n_out + PTC_TILE - 1) / PTC_TILE;
-  grid = c->num_sms * (per_sm > 0 ? per_sm : 1);
-  if (grid > ntiles) grid = ntiles;
-  kern<<<grid, 256, smem, c->stream>>>(ptc_geom(c), in, out, W, P->d_err, skip);
-  HISQ_CUDA(cudaGetLastError());
-  note_launch(c);
-  return HISQ_OK;
 }
 
 // z = N(r) for nvec even-site FP32 vectors (device), using workspaces of the context: the composed
@@ -1103,74 +895,20 @@ static int network_apply(hisq_ptc* P, float2* z, const float2* r, int nvec, __ha
   return HISQ_OK;
 }
 
-static int check_err(hisq_ptc* P) {
-  int e = 0;
-  HISQ_CUDA(cudaMemcpyAsync(&e, P->d_err, sizeof(int), cudaMemcpyDeviceToHost, P->ctx->stream));
-  HISQ_CUDA(cudaStreamSynchronize(P->ctx->stream));
-  if (e) {
-    cudaMemsetAsync(P->d_err, 0, sizeof(int), P->ctx->stream);
-    return set_error(HISQ_ETIMEOUT, "a tensor-core completion wait ran out");
-  }
-  return HISQ_OK;
-}
-
-template <int CIN, int COUT, bool G_EVEN>
-static int weight_grad(hisq_ptc* P, const float2* in, const float2* gout, float2* gW, float scale, float* part) {
+// Forward pass and gradient sums of NV pairs: d in dv, the blocks' partial sums in epart and gpart.
+template <int NV>
+static int train_group(hisq_ptc* P, const float2* b, const float2* x, float2* phi, float2* dv, double* epart,
+                       float2* gpart, int nblk) {
   hisq_ctx* c = P->ctx;
-  auto kern = k_ptc_wgrad<CIN, COUT, G_EVEN>;
-  const size_t smem = wg_smem<CIN, COUT>() + 1024;
-  const int n_g = G_EVEN ? c->g.half : c->g.V;
-  int grid = launch_tc(c, kern, smem, (n_g + WG_SITES - 1) / WG_SITES, "ptc wgrad");
-  if (grid < 0) return grid;
-  kern<<<grid, 128, smem, c->stream>>>(ptc_geom(c), in, gout, part, P->d_err);
-  HISQ_CUDA(cudaGetLastError());
-  k_ptc_wgrad_final<<<1, 128, 0, c->stream>>>(part, grid, CIN, COUT, scale, gW);
-  HISQ_CUDA(cudaGetLastError());
-  note_launch(c, 2);
+  const PtcGeom G = ptc_geom(c);
+  const size_t smem = (size_t)NV * 2 * PT_FIELD * sizeof(float2);
+  const float2* mix = P->mix;
+  HISQ_CUDA(launch_dependent(c, k_ptc_train_odd<NV>, nblk, 256, G, b, phi, mix));
+  HISQ_CUDA(launch_dependent(c, k_ptc_train_even<NV>, nblk, 256, G, b, (const float2*)phi, x, dv, mix, epart));
+  HISQ_CUDA(cudaFuncSetAttribute(k_ptc_grad<NV>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  HISQ_CUDA(launch_dependent_smem(c, k_ptc_grad<NV>, nblk, 256, smem, G, b, (const float2*)dv, gpart));
+  note_launch(c, 3);
   return HISQ_OK;
-}
-
-template <int CIN, int COUT, bool IN_EVEN>
-static int input_grad(hisq_ptc* P, const float2* gout, float2* m, float2* gin, const float2* W) {
-  hisq_ctx* c = P->ctx;
-  auto kern = k_ptc_bwd_mix<CIN, COUT, IN_EVEN>;
-  const size_t smem = mix_smem<CIN, COUT>() + 1024;
-  const int n_in = IN_EVEN ? c->g.half : c->g.V;
-  int grid = launch_tc(c, kern, smem, (n_in + PTC_TILE - 1) / PTC_TILE, "ptc mix");
-  if (grid < 0) return grid;
-  HISQ_CUDA(cudaMemsetAsync(m, 0, (size_t)CIN * NHOP * c->g.V * 3 * sizeof(float2), c->stream));
-  kern<<<grid, 128, smem, c->stream>>>(ptc_geom(c), gout, m, W, P->d_err);
-  HISQ_CUDA(cudaGetLastError());
-  k_ptc_bwd_gather<CIN><<<c->num_sms * 4, 128, 0, c->stream>>>(ptc_geom(c), m, gin);
-  HISQ_CUDA(cudaGetLastError());
-  note_launch(c, 2);
-  return HISQ_OK;
-}
-
-// e = (N(b) - x) / |x|^2 / npairs on even sites, and the loss terms (host reduction of a copy).
-__global__ void k_ptc_residual(const float2* __restrict__ z, const float2* __restrict__ x, float2* __restrict__ e,
-                               size_t n, float inv_nx, double* __restrict__ partials) {
-  double s = 0.0;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    const float2 a = z[i], b = x[i];
-    const float2 d = make_float2(a.x - b.x, a.y - b.y);
-    e[i] = make_float2(d.x * inv_nx, d.y * inv_nx);
-    s += (double)(d.x * d.x + d.y * d.y);
-  }
-  __shared__ double red[32];
-  double t = block_sum_dyn(s, red);
-  if (threadIdx.x == 0) partials[blockIdx.x] = t;
-}
-
-__global__ void k_sum_sq(const float2* __restrict__ x, size_t n, double* __restrict__ partials) {
-  double s = 0.0;
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    const float2 a = x[i];
-    s += (double)(a.x * a.x + a.y * a.y);
-  }
-  __shared__ double red[32];
-  double t = block_sum_dyn(s, red);
-  if (threadIdx.x == 0) partials[blockIdx.x] = t;
 }
 
 }  // namespace hisq
@@ -1194,8 +932,6 @@ int hisq_ptc_create(hisq_ptc** out, hisq_ctx* ctx, int channels) {
   if (e == cudaSuccess) e = cudaMalloc(&P->g2, nw * sizeof(float2));
   if (e == cudaSuccess) e = cudaMalloc(&P->m1, 4 * nw * 2 * sizeof(float));
   if (e == cudaSuccess) e = cudaMemset(P->m1, 0, 4 * nw * 2 * sizeof(float));
-  if (e == cudaSuccess) e = cudaMalloc(&P->d_err, sizeof(int));
-  if (e == cudaSuccess) e = cudaMemset(P->d_err, 0, sizeof(int));
   if (e == cudaSuccess) e = cudaMalloc(&P->mix, 65 * sizeof(float2));
   if (e != cudaSuccess) {
     hisq_ptc_destroy(P);
@@ -1217,7 +953,6 @@ int hisq_ptc_destroy(hisq_ptc* P) {
   cudaFree(P->g1);
   cudaFree(P->g2);
   cudaFree(P->m1);
-  cudaFree(P->d_err);
   cudaFree(P->mix);
   delete P;
   return HISQ_OK;
@@ -1275,7 +1010,7 @@ int hisq_ptc_apply(hisq_ptc* P, float* z, const float* r, int nvec) {
   hisq_ctx* c = P->ctx;
   __half2* phi = (__half2*)workspace(c, "ptc_phi", (size_t)8 * c->g.half * 3 * sizeof(__half2));
   if (!phi) return set_error(HISQ_ENOMEM, "ptc workspace");
-  // the composed apply has no tensor-core wait to report: asynchronous on the stream, like hisq_dslash
+  // asynchronous on the stream, like hisq_dslash
   return network_apply(P, (float2*)z, (const float2*)r, nvec, phi);
 }
 
@@ -1289,67 +1024,54 @@ int hisq_ptc_train_step(hisq_ptc* P, const float* b, const float* x, int npairs,
   if (!is_device_ptr(b) || !is_device_ptr(x)) return set_error(HISQ_EINVAL, "device vectors only");
   hisq_ctx* c = P->ctx;
   const int C = P->C;
-  const size_t V3 = (size_t)c->g.V * 3, nh = (size_t)c->g.half * 3;
-  float2* psi0 = (float2*)workspace(c, "ptc_psi0", V3 * sizeof(float2));
-  float2* psi1 = (float2*)workspace(c, "ptc_psi1", (size_t)C * V3 * sizeof(float2));
-  float2* z = (float2*)workspace(c, "ptc_z", nh * sizeof(float2));
-  float2* e = (float2*)workspace(c, "ptc_e", nh * sizeof(float2));
-  float2* m = (float2*)workspace(c, "ptc_m", (size_t)C * NHOP * V3 * sizeof(float2));
-  float2* gpsi1 = (float2*)workspace(c, "ptc_gpsi1", (size_t)C * V3 * sizeof(float2));
-  float2* gw = (float2*)workspace(c, "ptc_gw", 4 * (size_t)C * NHOP * sizeof(float2));
-  float* part = (float*)workspace(c, "ptc_part", (size_t)c->num_sms * 256 * 16 * sizeof(float));
-  double* red = (double*)workspace(c, "ptc_red", 2 * 1024 * sizeof(double));
-  if (!psi0 || !psi1 || !z || !e || !m || !gpsi1 || !gw || !part || !red) return set_error(HISQ_ENOMEM, "workspace");
-  float2* gw1 = gw;
-  float2* gw2 = gw + C * NHOP;
-  float2* acc1 = gw + 2 * C * NHOP;
-  float2* acc2 = gw + 3 * C * NHOP;
-  HISQ_CUDA(cudaMemsetAsync(acc1, 0, 2 * (size_t)C * NHOP * sizeof(float2), c->stream));
-  std::vector<double> hred(1024);
-  double loss = 0.0;
-  for (int q = 0; q < npairs; ++q) {
-    const float2* bq = (const float2*)b + q * nh;
-    const float2* xq = (const float2*)x + q * nh;
-    // |x|^2 (deterministic partials, summed on the host)
-    const int rg = 512;
-    k_sum_sq<<<rg, 256, 0, c->stream>>>(xq, nh, red);
-    HISQ_CUDA(cudaMemcpyAsync(hred.data(), red, rg * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-    HISQ_CUDA(cudaStreamSynchronize(c->stream));
-    double nx = 0;
-    for (int i = 0; i < rg; ++i) nx += hred[i];
-    // forward
-    k_embed_even<<<c->num_sms * 4, 256, 0, c->stream>>>(c->g, bq, psi0, nullptr);
-    int rc = forward_layer<1, 8, false>(P, psi0, psi1, P->w1);
-    if (rc == HISQ_OK) rc = forward_layer<8, 1, true>(P, psi1, z, P->w2);
-    if (rc != HISQ_OK) return rc;
-    // e = (z - x) / (|x|^2 npairs): dLoss/d(conj z)
-    k_ptc_residual<<<rg, 256, 0, c->stream>>>(z, xq, e, nh, (float)(1.0 / (nx * npairs)), red);
-    HISQ_CUDA(cudaMemcpyAsync(hred.data(), red, rg * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-    HISQ_CUDA(cudaStreamSynchronize(c->stream));
-    double ee = 0;
-    for (int i = 0; i < rg; ++i) ee += hred[i];
-    loss += ee / nx / npairs;
-    // backward: layer 2 weights and input gradient, then layer 1 weights
-    if ((rc = weight_grad<8, 1, true>(P, psi1, e, gw2, 1.f, part)) != HISQ_OK) return rc;
-    if ((rc = input_grad<8, 1, true>(P, e, m, gpsi1, P->w2)) != HISQ_OK) return rc;
-    if ((rc = weight_grad<1, 8, false>(P, psi0, gpsi1, gw1, 1.f, part)) != HISQ_OK) return rc;
-    note_launch(c, 4);
-    // accumulate over pairs
-    k_accumulate<<<1, 256, 0, c->stream>>>((float*)acc1, (const float*)gw1, 2 * C * NHOP);
-    k_accumulate<<<1, 256, 0, c->stream>>>((float*)acc2, (const float*)gw2, 2 * C * NHOP);
-    HISQ_CUDA(cudaGetLastError());
+  const size_t nh = (size_t)c->g.half * 3, nw = (size_t)C * NHOP;
+  const int nv_max = npairs >= 4 ? 4 : npairs >= 2 ? 2 : 1, chunk = npairs < PT_CHUNK ? npairs : PT_CHUNK;
+  // persistent grids of two resident blocks per SM
+  const int ntiles = (c->g.half + PT_SITES - 1) / PT_SITES;
+  const int nblk = ntiles < 2 * c->num_sms ? ntiles : 2 * c->num_sms;
+  float2* phi = (float2*)workspace(c, "ptc_phi32", nv_max * 8 * nh * sizeof(float2));
+  float2* dv = (float2*)workspace(c, "ptc_d", nv_max * nh * sizeof(float2));
+  double* epart = (double*)workspace(c, "ptc_epart", (size_t)chunk * nblk * PT_PART * sizeof(double));
+  float2* gpart = (float2*)workspace(c, "ptc_gpart", (size_t)chunk * nblk * 64 * sizeof(float2));
+  double2* tot = (double2*)workspace(c, "ptc_tot", (PT_CHUNK * PT_SPLIT + 1) * PT_TOT * sizeof(double2));
+  float2* gw = (float2*)workspace(c, "ptc_gw", (2 * nw + 1) * sizeof(float2));
+  if (!phi || !dv || !epart || !gpart || !tot || !gw) return set_error(HISQ_ENOMEM, "workspace");
+  float2 *acc1 = gw, *acc2 = gw + nw;
+  float* dloss = (float*)(gw + 2 * nw);
+  double2* msum = tot + PT_CHUNK * PT_SPLIT * PT_TOT;
+  int rc = HISQ_OK;
+  for (int q0 = 0; q0 < npairs; q0 += chunk) {
+    const int n = npairs - q0 < chunk ? npairs - q0 : chunk;
+    for (int q = 0; q < n;) {
+      const int nv = n - q >= 4 ? 4 : n - q >= 2 ? 2 : 1;
+      const float2 *bq = (const float2*)b + (q0 + q) * nh, *xq = (const float2*)x + (q0 + q) * nh;
+      double* ep = epart + (size_t)q * nblk * PT_PART;
+      float2* gp = gpart + (size_t)q * nblk * 64;
+      rc = nv == 4 ? train_group<4>(P, bq, xq, phi, dv, ep, gp, nblk)
+           : nv == 2 ? train_group<2>(P, bq, xq, phi, dv, ep, gp, nblk)
+                     : train_group<1>(P, bq, xq, phi, dv, ep, gp, nblk);
+      if (rc != HISQ_OK) return rc;
+      q += nv;
+    }
+    HISQ_CUDA(launch_dependent(c, k_ptc_train_sum, dim3(n, PT_SPLIT), 256, (const double*)epart, nblk,
+                               (const float2*)gpart, nblk, tot));
+    HISQ_CUDA(launch_dependent(c, k_ptc_train_final, 1, 544, (const double2*)tot, n, npairs, msum, (int)(q0 == 0),
+                               (int)(q0 + n == npairs), (const float2*)P->w1, (const float2*)P->w2, C, acc1, acc2, dloss));
     note_launch(c, 2);
   }
-  int rc = check_err(P);
-  if (rc != HISQ_OK) return rc;
   if (P->tied) {
     k_tie_grad<<<1, 128, 0, c->stream>>>(acc1, acc2, C);
     HISQ_CUDA(cudaGetLastError());
     note_launch(c);
   }
-  if (loss_out) *loss_out = (float)loss;
-  if (g1_out) HISQ_CUDA(cudaMemcpy(g1_out, acc1, (size_t)C * NHOP * sizeof(float2), cudaMemcpyDeviceToHost));
-  if (g2_out) HISQ_CUDA(cudaMemcpy(g2_out, acc2, (size_t)C * NHOP * sizeof(float2), cudaMemcpyDeviceToHost));
+  if (loss_out || g1_out || g2_out) {  // one read-back for all three
+    std::vector<float2> hg(2 * nw + 1);
+    HISQ_CUDA(cudaMemcpyAsync(hg.data(), gw, hg.size() * sizeof(float2), cudaMemcpyDeviceToHost, c->stream));
+    HISQ_CUDA(cudaStreamSynchronize(c->stream));
+    if (loss_out) *loss_out = hg[2 * nw].x;
+    if (g1_out) memcpy(g1_out, hg.data(), nw * sizeof(float2));
+    if (g2_out) memcpy(g2_out, hg.data() + nw, nw * sizeof(float2));
+  }
   if (lr > 0.f) {
     P->adam_t += 1;
     const float b1 = 0.9f, b2 = 0.999f;
@@ -1511,7 +1233,6 @@ int hisq_fcg(hisq_ctx* c, hisq_ptc* P, double* x_user, const double* b_user, dou
     }
   }
   cudaGraphExecDestroy(exec);
-  if ((rc = check_err(P)) != HISQ_OK) return rc;
   const double rel = h->bb > 0 ? sqrt(h->rr_true / h->bb) : sqrt(h->rr_true);
   if (stats) {
     stats->iters = h->iter;

@@ -1,6 +1,6 @@
-"""The PTC network on the GPU (tensor-core channel mixing, BF16 operands, FP32 accumulation) against the
-FP64 oracle: forward output, loss and weight gradients; flexible CG with the network as preconditioner
-judged by the oracle's true residual. Tolerances: BF16 forward <= 1e-2, gradients <= 2e-2 (relative)."""
+"""The PTC network on the GPU (weights rounded to BF16, FP32 arithmetic) against the FP64 oracle: forward
+output, loss and weight gradients; flexible CG with the network as preconditioner judged by the oracle's true
+residual. Tolerances with weights that BF16 rounds: forward <= 1e-2, gradients <= 2e-2 (relative)."""
 import numpy as np
 import pytest
 
@@ -238,3 +238,27 @@ def test_trained_network_gains_over_the_method_without_it(hisq):
     mixed = st["iters"]
     net.set_tied(False)
     assert trained <= 0.91 * min(identity, mixed), (trained, identity, mixed)
+
+
+@pytest.mark.parametrize("npairs", [1, 2, 3, 7, 17])
+@pytest.mark.parametrize("dims", [(6, 6, 6, 6), (4, 4, 4, 4), (4, 6, 8, 10)])
+def test_ptc_gradient_groups_and_tiles(hisq, dims, npairs):
+    """Loss and gradients of every grouping of the pairs (4, 2 and 1 per link read, chunks of 16) on lattices whose
+    sites fill the last tile of 32 or not (6^4: 648 = 20 * 32 + 8), with inputs far from unit scale. FP32
+    arithmetic on BF16-exact weights: transports and 8-term sums round by a few 2^-24, so 1e-5 leaves a factor
+    of more than ten for the cancellation in N(b) - x."""
+    import torch
+    fat, lng = hin.gen_links(dims, 77, 0.35, 0.1)
+    lat = hisq.Lattice(dims, precs=(0, 1)).load(fat, lng)
+    ff, _ = oracle.fold_links(dims, fat.reshape(-1, 4, 3, 3), lng.reshape(-1, 4, 3, 3))
+    net = hisq.Ptc(lat)
+    W = [torch.view_as_complex(torch.view_as_real(torch.from_numpy(w.astype(np.complex64))).to(torch.bfloat16).float())
+         .numpy() for w in optc.init_weights(78)]
+    net.set_weights(*W)
+    b = (3e6 * hin.gen_source(79, lat.half, npairs)).astype(np.complex64)
+    x = (3e6 * hin.gen_source(80, lat.half, npairs)).astype(np.complex64)
+    loss, g1, g2 = net.train_step(torch.from_numpy(b).cuda(), torch.from_numpy(x).cuda(), npairs, 0.0)
+    rl, r1, r2 = optc.loss_and_grads(dims, ff, *(w.astype(np.complex128) for w in W), list(b.astype(np.complex128)),
+                                     list(x.astype(np.complex128)))
+    assert abs(loss - rl) <= 1e-5 * rl
+    assert rel(g1, r1) <= 1e-5 and rel(g2, r2) <= 1e-5, (rel(g1, r1), rel(g2, r2))
