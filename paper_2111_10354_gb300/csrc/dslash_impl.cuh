@@ -125,11 +125,11 @@ __device__ __forceinline__ void dslash_site(const Geom& g, const char* links, si
 #pragma unroll
     for (int i = 0; i < 3; ++i) acc[r][i] = {A(0), A(0)};
 
-  // groups of 8 vectors keep the direction loop rolled: the fully unrolled body (16 hops x 8 vectors)
+  // groups of 5 to 8 vectors keep the direction loop rolled: the fully unrolled body (16 hops x 8 vectors)
   // outgrows the instruction cache and the warps stall on instruction fetch (48^3x12 FP32: 260 -> 245 us;
   // FP16: 204 -> 183 us); at 4 vectors the unrolled body is faster (156 vs 171 us)
   // double-float keeps it rolled as well (its hoisted link loads otherwise exceed the register budget)
-  constexpr int MU_UNROLL = (NR >= 8 || std::is_same<LR, df64>::value) ? 1 : 4;
+  constexpr int MU_UNROLL = (NR > 4 || std::is_same<LR, df64>::value) ? 1 : 4;
 #pragma unroll MU_UNROLL
   for (int mu = 0; mu < 4; ++mu) {
 #pragma unroll
@@ -220,9 +220,9 @@ __device__ __forceinline__ void dslash_site(const Geom& g, const char* links, si
 // bound by GB300's FP64 pipe, and a 64-register cap spills).
 template <typename LR, int NR>
 struct DslashBounds {
-  static constexpr int threads = NR == 1 ? (sizeof(LR) < 8 ? 256 : 512) : (NR == 2 ? 512 : (NR == 4 ? 256 : 128));
-  // FP32/16-bit: 64 registers for one vector, 128 for groups of 4 and 8 (enough warps in flight)
-  static constexpr int min_blocks = sizeof(LR) == 8 ? 1 : (NR == 1 ? 4 : (NR == 2 ? 1 : (NR == 4 ? 2 : (NR == 8 ? 4 : 1))));
+  static constexpr int threads = NR == 1 ? (sizeof(LR) < 8 ? 256 : 512) : (NR == 2 ? 512 : (NR <= 4 ? 256 : 128));
+  // FP32/16-bit: 64 registers for one vector, 128 for groups of 3 to 8 (enough warps in flight)
+  static constexpr int min_blocks = sizeof(LR) == 8 ? 1 : (NR == 1 ? 4 : (NR == 2 ? 1 : (NR <= 4 ? 2 : 4)));
 };
 // Double-float: 128 registers for one vector (a double-float link is 36 registers), all 255 for
 // groups, where fewer spill.

@@ -3,8 +3,9 @@
 // with the autotuner.
 #pragma once
 #include <string>
+#include <vector>
 
-#include "dslash_impl.cuh"
+#include "dslash_split.cuh"
 #include "tune.h"
 
 namespace hisq {
@@ -62,14 +63,67 @@ static TuneVariant dslash_variant(hisq_ctx* ctx, const DslashKArgs& a) {
                      }};
 }
 
-template <int N>
-static int launch_tuned(hisq_ctx* ctx, const char* key, const TuneVariant (&v)[N]) {
+// One launch form of dslash_split_kernel: ngrp groups of NR vectors, HS threads per (site, group).
+template <typename LR, typename SR, int NR, int EPI, int HS>
+static TuneVariant split_variant(hisq_ctx* ctx, const DslashKArgs& a, int ngrp = 1) {
+  return TuneVariant{(const void*)dslash_split_kernel<LR, SR, NR, EPI, HS>, [ctx, &a, ngrp](int block) -> cudaError_t {
+                       int grid = (int)(((size_t)ctx->g.half * HS + block - 1) / block);
+                       int cap = max_grid_blocks(ctx, block);
+                       if (EPI == EPI_AXPY && a.partials) {
+                         int per_sm = 0;
+                         cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+                             &per_sm, dslash_split_kernel<LR, SR, NR, EPI, HS>, block, 0);
+                         cap = ctx->num_sms * (per_sm > 0 ? per_sm : 1);
+                       }
+                       if (grid > cap) grid = cap;
+                       return launch_dependent(ctx, dslash_split_kernel<LR, SR, NR, EPI, HS>, dim3(grid, ngrp), block, a);
+                     }};
+}
+
+// The split forms are offered where the site count times the shares fills the GPU at most twice (1024 threads
+// per SM are one wave at 64 registers): beyond that one thread per site has warps enough and measured faster.
+inline bool split_fits(const hisq_ctx* ctx, int shares) {
+  return (double)ctx->g.half * shares <= 2.0 * ctx->num_sms * 1024;
+}
+
+static int launch_tuned(hisq_ctx* ctx, const char* key, const std::vector<TuneVariant>& v) {
   int vi = 0, block = 0;
-  int rc = tuned_variant(ctx, key, v, N, &vi, &block);
+  int rc = tuned_variant(ctx, key, v.data(), (int)v.size(), &vi, &block);
   if (rc != HISQ_OK) return rc;
   HISQ_CUDA(v[vi].run(block));
   note_launch(ctx);
   return HISQ_OK;
+}
+
+// The forms of a group of NR vectors in one thread per site, in cb order and (groups of 1 and 5 to 8) in the
+// tiled walk, and, with few sites and uncompressed links, the split forms.
+template <typename LR, typename SR, int NR, int EPI, bool COMP>
+static std::vector<TuneVariant> group_forms(hisq_ctx* ctx, const DslashKArgs& a) {
+  std::vector<TuneVariant> v = {dslash_variant<LR, SR, NR, EPI, COMP, 1>(ctx, a)};
+  if (NR == 2) v.push_back(dslash_variant<LR, SR, 1, EPI, COMP, 2>(ctx, a));
+  if (NR == 4) {
+    v.push_back(dslash_variant<LR, SR, 2, EPI, COMP, 2>(ctx, a));
+    v.push_back(dslash_variant<LR, SR, 1, EPI, COMP, 4>(ctx, a));
+  }
+  if constexpr (NR == 8) {
+    v.push_back(dslash_variant<LR, SR, 4, EPI, COMP, 2>(ctx, a));
+    v.push_back(dslash_variant<LR, SR, 2, EPI, COMP, 4>(ctx, a));
+    v.push_back(dslash_variant<LR, SR, 8, EPI, COMP, 1, true>(ctx, a));
+    v.push_back(dslash_variant<LR, SR, 4, EPI, COMP, 2, true>(ctx, a));
+    v.push_back(dslash_variant<LR, SR, 2, EPI, COMP, 4, true>(ctx, a));
+    v.push_back(dslash_variant<LR, SR, 8, EPI, COMP, 1, false, true>(ctx, a));
+    v.push_back(dslash_variant<LR, SR, 8, EPI, COMP, 1, true, true>(ctx, a));
+  }
+  if (NR == 1 || (NR > 4 && NR < 8)) v.push_back(dslash_variant<LR, SR, NR, EPI, COMP, 1, true>(ctx, a));
+  if constexpr (!COMP) {
+    if constexpr (NR == 1)
+      if (split_fits(ctx, 2)) v.push_back(split_variant<LR, SR, 1, EPI, 2>(ctx, a));
+    if constexpr (sizeof(LR) < 8 || NR == 1)
+      if (split_fits(ctx, 4)) v.push_back(split_variant<LR, SR, NR, EPI, 4>(ctx, a));
+    if constexpr (NR == 1)
+      if (split_fits(ctx, 8)) v.push_back(split_variant<LR, SR, 1, EPI, 8>(ctx, a));
+  }
+  return v;
 }
 
 // A group of nr vectors shares each link read. The launch forms differ in how the group is spread
@@ -78,56 +132,52 @@ template <typename LR, typename SR, int EPI, bool COMP>
 static int launch_nr(hisq_ctx* ctx, const DslashKArgs& a, int nr) {
   char key[64];
   snprintf(key, sizeof key, "dslash/l%d/s%d/nr%d/e%d/c%d", Real<LR>::prec, Real<SR>::prec, nr, EPI, (int)COMP);
+  if constexpr (sizeof(LR) == 8) {
+    if (nr > 1 && split_fits(ctx, 2 * nr)) {  // FP64 on few sites: each vector in its own row of blocks
+      snprintf(key, sizeof key, "dslash/l%d/s%d/ny%d/e%d", Real<LR>::prec, Real<SR>::prec, nr, EPI);
+      std::vector<TuneVariant> v = {split_variant<LR, SR, 1, EPI, 2>(ctx, a, nr)};
+      if (split_fits(ctx, 4 * nr)) v.push_back(split_variant<LR, SR, 1, EPI, 4>(ctx, a, nr));
+      if (split_fits(ctx, 8 * nr)) v.push_back(split_variant<LR, SR, 1, EPI, 8>(ctx, a, nr));
+      return launch_tuned(ctx, key, v);
+    }
+  }
   switch (nr) {
-    case 1: {
-      const TuneVariant v[] = {dslash_variant<LR, SR, 1, EPI, COMP, 1>(ctx, a),
-                               dslash_variant<LR, SR, 1, EPI, COMP, 1, true>(ctx, a)};
-      return launch_tuned(ctx, key, v);
+    case 1: return launch_tuned(ctx, key, group_forms<LR, SR, 1, EPI, COMP>(ctx, a));
+    case 2: return launch_tuned(ctx, key, group_forms<LR, SR, 2, EPI, COMP>(ctx, a));
+    case 3: return launch_tuned(ctx, key, group_forms<LR, SR, 3, EPI, COMP>(ctx, a));
+    case 4: return launch_tuned(ctx, key, group_forms<LR, SR, 4, EPI, COMP>(ctx, a));
+  }
+  if constexpr (sizeof(LR) < 8) {
+    switch (nr) {
+      case 5: return launch_tuned(ctx, key, group_forms<LR, SR, 5, EPI, COMP>(ctx, a));
+      case 6: return launch_tuned(ctx, key, group_forms<LR, SR, 6, EPI, COMP>(ctx, a));
+      case 7: return launch_tuned(ctx, key, group_forms<LR, SR, 7, EPI, COMP>(ctx, a));
+      case 8: return launch_tuned(ctx, key, group_forms<LR, SR, 8, EPI, COMP>(ctx, a));
     }
-    case 2: {
-      const TuneVariant v[] = {dslash_variant<LR, SR, 2, EPI, COMP, 1>(ctx, a),
-                               dslash_variant<LR, SR, 1, EPI, COMP, 2>(ctx, a)};
-      return launch_tuned(ctx, key, v);
-    }
-    case 4: {
-      const TuneVariant v[] = {dslash_variant<LR, SR, 4, EPI, COMP, 1>(ctx, a),
-                               dslash_variant<LR, SR, 2, EPI, COMP, 2>(ctx, a),
-                               dslash_variant<LR, SR, 1, EPI, COMP, 4>(ctx, a)};
-      return launch_tuned(ctx, key, v);
-    }
-    case 8:
-      if constexpr (sizeof(LR) < 8) {
-        const TuneVariant v[] = {dslash_variant<LR, SR, 8, EPI, COMP, 1>(ctx, a),
-                                 dslash_variant<LR, SR, 4, EPI, COMP, 2>(ctx, a),
-                                 dslash_variant<LR, SR, 2, EPI, COMP, 4>(ctx, a),
-                                 dslash_variant<LR, SR, 8, EPI, COMP, 1, true>(ctx, a),
-                                 dslash_variant<LR, SR, 4, EPI, COMP, 2, true>(ctx, a),
-                                 dslash_variant<LR, SR, 2, EPI, COMP, 4, true>(ctx, a),
-                                 dslash_variant<LR, SR, 8, EPI, COMP, 1, false, true>(ctx, a),
-                                 dslash_variant<LR, SR, 8, EPI, COMP, 1, true, true>(ctx, a)};
-        return launch_tuned(ctx, key, v);
-      }
-      break;
   }
   return set_error(HISQ_EINVAL, "unsupported rhs group %d", nr);
 }
 
-// Largest rhs group per launch (register budget): FP64 4, others 8 -- a group of 16 needs more
-// than the 255 registers a thread can hold and spills (measured 5x slower than two groups of 8).
+// Largest rhs group per launch: 8, because a group of 16 needs more than the 255 registers a thread can hold
+// and spills (measured 5x slower than two groups of 8). FP64 and double-float groups stop at 4, but where the
+// split forms fit they take as many vectors as fit.
 template <typename LR>
-static int max_group() {
-  return sizeof(LR) == 8 ? 4 : 8;
+static int max_group(const hisq_ctx* ctx) {
+  if (sizeof(LR) < 8) return 8;
+  int n = 8;
+  while (n > 4 && !split_fits(ctx, 2 * n)) --n;
+  return n;
 }
 
 template <typename LR, typename SR>
 int dslash_launch_t(hisq_ctx* ctx, const DslashCall& c) {
   const size_t site_bytes = 6 * sizeof(SR);
-  const int gmax = max_group<LR>();
+  const int gmax = max_group<LR>(ctx);
   int r0 = 0;
   while (r0 < c.nrhs) {
     const int left = c.nrhs - r0;
-    int nr = 1;
-    while (nr * 2 <= left && nr * 2 <= gmax) nr *= 2;
+    // groups of nearly equal size: the cost of a launch's link read is spread over all of them
+    const int ngrp = (left + gmax - 1) / gmax, nr = (left + ngrp - 1) / ngrp;
     DslashKArgs a;
     a.g = ctx->g;
     a.links = ctx->links[Real<LR>::prec];

@@ -80,13 +80,23 @@ inline int tuned_variant(hisq_ctx* ctx, const char* key, const TuneVariant* v, i
         cudaGetLastError();
         continue;
       }
-      cudaEventRecord(e0, ctx->stream);
-      for (int r = 0; r < 3; ++r) v[i].run(b);
-      note_launch(ctx, 4);
-      cudaEventRecord(e1, ctx->stream);
-      if (cudaEventSynchronize(e1) != cudaSuccess) break;
+      note_launch(ctx);
       float ms = 0;
-      cudaEventElapsedTime(&ms, e0, e1);
+      bool timed = true;
+      // three launches; where those take less than 60 us in all, twenty, so that the events' own cost and the
+      // launch of the first one do not decide between small kernels
+      for (int reps = 3; timed; reps = 20) {
+        cudaEventRecord(e0, ctx->stream);
+        for (int r = 0; r < reps; ++r) v[i].run(b);
+        note_launch(ctx, reps);
+        cudaEventRecord(e1, ctx->stream);
+        timed = cudaEventSynchronize(e1) == cudaSuccess;
+        if (!timed) break;
+        cudaEventElapsedTime(&ms, e0, e1);
+        ms /= (float)reps;
+        if (reps == 20 || ms >= 0.02f) break;
+      }
+      if (!timed) break;
       if (ms < best) {
         best = ms;
         best_v = i;

@@ -305,3 +305,62 @@ def test_every_launch_form_matches_oracle(hisq, prec):
             for r in range(nr):
                 ref = oracle.apply_A(L, ff, lf, 0.05, src[r])
                 assert rel_err(got[r], ref) <= 2 * TOL[prec], (prec, nr, vi, r)
+
+
+# the forms whose threads share a site's hops, as (rhs count, key, variants): appended to the forms above for
+# lattices with few sites; FP64 groups have keys of their own (a row of blocks per vector)
+def split_forms(prec):
+    if prec in (0, 4):
+        return [(1, "nr1", (2, 3, 4))] + [(n, "ny%d" % n, (0, 1, 2)) for n in (2, 5, 8)]
+    return [(1, "nr1", (2, 3, 4)), (2, "nr2", (2,)), (3, "nr3", (1,)), (4, "nr4", (3,)), (5, "nr5", (2,)),
+            (6, "nr6", (2,)), (7, "nr7", (2,)), (8, "nr8", (8,))]
+
+
+@pytest.mark.parametrize("L,block", [((4, 4, 4, 4), 64), ((4, 6, 8, 10), 160), ((6, 6, 10, 14), 256)])
+@pytest.mark.parametrize("prec", [0, 1, 2, 3, 4])
+def test_split_launch_forms_match_oracle(hisq, prec, L, block):
+    """Every launch form that shares a site's hops between threads, forced through loaded tune entries: the
+    Dslash to both parities and A, against the oracle, on the smallest lattice (fewer sites than threads), on
+    one whose hops alias, and on one with a ragged last block."""
+    lat, ff, lf = setup(hisq, L)
+    sp = 0 if prec == 4 else prec
+    dims = "%dx%dx%dx%d" % L
+    for nr, name, variants in split_forms(prec):
+        src = hin.gen_source(7100 + nr, lat.half, nr)
+        x = to_device(src, prec)
+        for vi in variants:
+            for epi in (0, 1):
+                key = "dslash/l%d/s%d/%s/e%d%s" % (prec, sp, name, epi, "/c0" if name[:2] == "nr" else "")
+                assert hisq.hisq_tune_load(lat.ctx, "%s %s -> %d\n" % (key, dims, vi * 10000 + block)) == 1
+            y = empty_like_prec((nr, lat.half, 3), prec)
+            for parity in (0, 1):
+                lat.dslash(parity, y, x, prec, nr)
+                got = from_device(y, prec)
+                for r in range(nr):
+                    assert rel_err(got[r], oracle.dslash(L, ff, lf, parity, src[r])) <= TOL[prec], (nr, vi, r, parity)
+            lat.apply_A(y, x, 0.05, prec, nr)
+            got = from_device(y, prec)
+            for r in range(nr):
+                assert rel_err(got[r], oracle.apply_A(L, ff, lf, 0.05, src[r])) <= 2 * TOL[prec], (nr, vi, r)
+            assert "%s %s -> %d" % (key, dims, vi * 10000 + block) in hisq.hisq_tune_report(lat.ctx)
+
+
+@pytest.mark.parametrize("prec", [0, 1, 2, 3, 4])
+def test_odd_vector_groups_match_oracle(hisq, prec):
+    """One launch for 3, 5, 6 and 7 vectors (every plain form), and counts that split into nearly equal groups."""
+    L = (8, 10, 12, 14)
+    lat, ff, lf = setup(hisq, L)
+    dims = "%dx%dx%dx%d" % L
+    sp = 0 if prec == 4 else prec
+    for nr in (3, 5, 6, 7, 9, 14):
+        src = hin.gen_source(7200 + nr, lat.half, nr)
+        x = to_device(src, prec)
+        y = empty_like_prec((nr, lat.half, 3), prec)
+        for vi in range(2 if nr in (5, 6, 7) else 1):
+            if nr <= 7 and prec not in (0, 4):
+                for epi in (0, 1):
+                    hisq.hisq_tune_load(lat.ctx, "dslash/l%d/s%d/nr%d/e%d/c0 %s -> %d\n" % (prec, sp, nr, epi, dims, vi * 10000 + 96))
+            lat.apply_A(y, x, 0.05, prec, nr)
+            got = from_device(y, prec)
+            for r in range(nr):
+                assert rel_err(got[r], oracle.apply_A(L, ff, lf, 0.05, src[r])) <= 2 * TOL[prec], (nr, vi, r)
