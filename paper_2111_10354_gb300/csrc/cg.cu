@@ -374,6 +374,10 @@ __device__ __forceinline__ void finish_iteration(SolverState* st, const double* 
 // The first KEEP chunks of r a thread updates stay in registers for phase 2; further chunks are read
 // again. Each thread handles its chunks in batches of KEEP whose loads are all issued before any store. Vector traffic: Ap, r read and r written, then p, x (and r beyond KEEP) read and p, x written:
 // seven vector passes where an x/r update launch and a separate p update launch take nine.
+// One thread per block forms alpha and beta (and one warp the sums behind them): a division by every thread is
+// some 20 FP64 operations of 16 cycles per warp, microseconds with 32 resident warps per SM. With that and the
+// pair sums (SumAcc) a launch went from 19.3 to 12.8 us for five FP16 vectors on 20x12x28x10 and from 9.7 to 8.8 us
+// on 8^4.
 template <typename S, typename X, int KEEP>
 __global__ void __launch_bounds__(256, 4) k_cg_update(X* __restrict__ x, S* __restrict__ r, S* __restrict__ p,
                                                    const S* __restrict__ Ap, size_t n, SolverState* st,
@@ -383,34 +387,47 @@ __global__ void __launch_bounds__(256, 4) k_cg_update(X* __restrict__ x, S* __re
   constexpr int K = Chunk<S>::K;
   __shared__ double red[32];
   __shared__ double s_tot[MAXR];
-  __shared__ int s_last;
+  __shared__ T s_a, s_beta;
+  __shared__ XT s_ax;
+  __shared__ int s_state;  // 0 frozen, 1 stopped (<p, Ap> not positive or not finite), 2 active
+  __shared__ int s_last, s_ok;
   if (st->done) return;  // uniform: only the last block at the barrier changes it
   const int rh = blockIdx.y;
   const size_t off = (size_t)rh * n;
-  const double pap = st->pAp[rh];
-  const bool frozen = st->rhs_done[rh] != 0;
-  const bool active = !frozen && pap > 0.0 && isfinite(pap);
-  const double rr_old = st->rr[rh];
-  const double alpha = active ? rr_old / pap : 0.0;
-  const T a = T(alpha);
-  const XT ax = XT(sizeof(X) == 8 ? alpha * st->scale[rh] : alpha);
   const size_t stride = (size_t)gridDim.x * blockDim.x * K;
   const size_t i0 = (blockIdx.x * (size_t)blockDim.x + threadIdx.x) * K;
-  const size_t nn = frozen ? 0 : n;  // a frozen rhs's vectors are not touched
-  cplx<T> keep[KEEP][K];
-  double v = 0.0;
-  // phase 1 in batches of KEEP chunks: every load of a batch is issued before any store (r is read and
-  // written, so a store would otherwise keep the next chunk's loads from being issued early)
-  auto phase1 = [&](size_t ib, cplx<T>(&rv)[KEEP][K]) {
-    cplx<T> av[KEEP][K];
+  cplx<T> keep[KEEP][K], a0[KEEP][K];
+  auto load_r_Ap = [&](size_t ib, cplx<T>(&rv)[KEEP][K], cplx<T>(&av)[KEEP][K]) {
 #pragma unroll
     for (int j = 0; j < KEEP; ++j) {
       const size_t i = ib + j * stride;
-      if (i < nn) {
+      if (i < n) {
         Chunk<S>::load(r, (off + i) / K, rv[j]);
-        if (active) Chunk<S>::load(Ap, (off + i) / K, av[j]);
+        Chunk<S>::load(Ap, (off + i) / K, av[j]);
       }
     }
+  };
+  load_r_Ap(i0, keep, a0);  // the first batch is in flight while alpha is formed
+  double rr_old = 1.0;      // thread 0
+  if (threadIdx.x == 0) {
+    const double pap = st->pAp[rh];
+    const int frozen = st->rhs_done[rh];
+    rr_old = st->rr[rh];
+    const bool act = !frozen && pap > 0.0 && isfinite(pap);
+    const double alpha = act ? rr_old / pap : 0.0;
+    s_a = T(alpha);
+    s_ax = XT(sizeof(X) == 8 ? alpha * st->scale[rh] : alpha);
+    s_state = frozen ? 0 : act ? 2 : 1;
+  }
+  __syncthreads();
+  const T a = s_a;
+  const XT ax = s_ax;
+  const bool active = s_state == 2;
+  const size_t nn = s_state == 0 ? 0 : n;  // a frozen rhs's vectors are not touched
+  SumAcc<T> v;
+  // phase 1 in batches of KEEP chunks: every load of a batch is issued before any store (r is read and
+  // written, so a store would otherwise keep the next chunk's loads from being issued early)
+  auto phase1 = [&](size_t ib, cplx<T>(&rv)[KEEP][K], const cplx<T>(&av)[KEEP][K]) {
 #pragma unroll
     for (int j = 0; j < KEEP; ++j) {
       const size_t i = ib + j * stride;
@@ -425,29 +442,59 @@ __global__ void __launch_bounds__(256, 4) k_cg_update(X* __restrict__ x, S* __re
           t += rv[j][c].re * rv[j][c].re + rv[j][c].im * rv[j][c].im;
         }
         if (active) Chunk<S>::store(r, (off + i) / K, rv[j]);
-        v += (double)t;
+        v.add(t);
       }
     }
   };
-  phase1(i0, keep);  // the first batch stays in registers for phase 2
+  phase1(i0, keep, a0);  // the first batch stays in registers for phase 2
   for (size_t ib = i0 + KEEP * stride; ib < nn; ib += KEEP * stride) {
-    cplx<T> rv[KEEP][K];
-    phase1(ib, rv);
+    cplx<T> rv[KEEP][K], av[KEEP][K];
+    load_r_Ap(ib, rv, av);
+    phase1(ib, rv, av);
+  }
+  // the first batch of p and x is requested before the barrier, whose wait then covers its latency
+  cplx<T> p0[KEEP][K];
+  cplx<XT> x0[KEEP][K];
+  auto load_p_x = [&](size_t ib, cplx<T>(&pv)[KEEP][K], cplx<XT>(&xv)[KEEP][K]) {
+#pragma unroll
+    for (int j = 0; j < KEEP; ++j) {
+      const size_t i = ib + j * stride;
+      if (i < nn) {
+        Chunk<S>::load(p, (off + i) / K, pv[j]);
+        load_k<X, K>(x, off + i, xv[j]);
+      }
+    }
+  };
+  if (active) load_p_x(i0, p0, x0);
+  const double bs = block_sum_acc(v, red);
+  if (threadIdx.x == 0) partials[(size_t)rh * gridDim.x + blockIdx.x] = bs;
+  unsigned gen;
+  bool last;
+  grid_arrive_release(bar, &gen, &last);
+  // warp 0 waits, sums its rhs's partials (the same order in every block, so every block forms the same beta) and
+  // forms beta; the block that arrived last also sums every rhs and commits the iteration
+  if (threadIdx.x < 32) {
+    const bool ok = grid_wait64_warp(bar, gen);
+    const double rr_new = warp_sum_partials(partials + (size_t)rh * gridDim.x, gridDim.x);
+    if (threadIdx.x == 0) {
+      s_tot[rh] = rr_new;
+      s_beta = T(rr_new / rr_old);
+      s_ok = ok ? 1 : 0;
+      s_last = last ? 1 : 0;
+    }
+  }
+  __syncthreads();
+  if (!s_ok) {
+    if (threadIdx.x == 0) {
+      st->timeout = 1;
+      st->done = 1;
+    }
+    return;
   }
   // phase 2 (x += alpha p, p = r + beta p), batch by batch: loads first, then the updates, then stores
-  auto update_p_x = [&](double rr_new) {
-    const T beta = T(rr_new / rr_old);
-    auto phase2 = [&](size_t ib, const cplx<T>(&rv)[KEEP][K]) {
-      cplx<T> pv[KEEP][K];
-      cplx<XT> xv[KEEP][K];
-#pragma unroll
-      for (int j = 0; j < KEEP; ++j) {
-        const size_t i = ib + j * stride;
-        if (i < nn) {
-          Chunk<S>::load(p, (off + i) / K, pv[j]);
-          load_k<X, K>(x, off + i, xv[j]);
-        }
-      }
+  if (active) {
+    const T beta = s_beta;
+    auto phase2 = [&](size_t ib, const cplx<T>(&rv)[KEEP][K], cplx<T>(&pv)[KEEP][K], cplx<XT>(&xv)[KEEP][K]) {
 #pragma unroll
       for (int j = 0; j < KEEP; ++j) {
         const size_t i = ib + j * stride;
@@ -464,43 +511,27 @@ __global__ void __launch_bounds__(256, 4) k_cg_update(X* __restrict__ x, S* __re
         }
       }
     };
-    phase2(i0, keep);
+    phase2(i0, keep, p0, x0);
     for (size_t ib = i0 + KEEP * stride; ib < nn; ib += KEEP * stride) {
-      cplx<T> rv[KEEP][K];
+      cplx<T> rv[KEEP][K], pv[KEEP][K];
+      cplx<XT> xv[KEEP][K];
 #pragma unroll
       for (int j = 0; j < KEEP; ++j) {
         const size_t i = ib + j * stride;
         if (i < nn) Chunk<S>::load(r, (off + i) / K, rv[j]);
       }
-      phase2(ib, rv);
+      load_p_x(ib, pv, xv);
+      phase2(ib, rv, pv, xv);
     }
-  };
-  const double bs = block_sum_dyn(v, red);
-  if (threadIdx.x == 0) partials[(size_t)rh * gridDim.x + blockIdx.x] = bs;
-  unsigned gen;
-  bool last;
-  grid_arrive_release(bar, &gen, &last);
-  if (!grid_wait64(bar, gen)) {
-    if (threadIdx.x == 0) {
-      st->timeout = 1;
-      st->done = 1;
-    }
-    return;
   }
-  // every block sums its rhs's partials itself (the same order in every block, so every block forms the
-  // same beta); the block that arrived last also sums every rhs and commits the iteration
-  if (threadIdx.x == 0) s_last = last ? 1 : 0;
-  const double rr_new = block_sum_partials(partials + (size_t)rh * gridDim.x, gridDim.x, red);
-  if (threadIdx.x == 0) s_tot[rh] = rr_new;
-  if (active) update_p_x(rr_new);
   // after its own vectors (the flag is read back from shared memory so that nothing of this tail stays
   // in registers through phase 2): the other rhs's sums and the commit, read by the next launches only
   if (*(volatile int*)&s_last) {
     const int nrhs = st->nrhs;
-    for (int q = 0; q < nrhs; ++q) {
+    for (int q = threadIdx.x >> 5; q < nrhs; q += (int)(blockDim.x >> 5)) {  // a warp per rhs
       if (q == (int)blockIdx.y) continue;
-      const double t = block_sum_partials(partials + (size_t)q * gridDim.x, gridDim.x, red);
-      if (threadIdx.x == 0) s_tot[q] = t;
+      const double t = warp_sum_partials(partials + (size_t)q * gridDim.x, gridDim.x);
+      if ((threadIdx.x & 31) == 0) s_tot[q] = t;
     }
     __syncthreads();
     if (threadIdx.x < 32) commit_iteration_warp(st, s_tot);
@@ -551,14 +582,22 @@ __global__ void __launch_bounds__(256) k_cg_update_il(float* __restrict__ e, flo
   __shared__ double s_tot[MAXR];
   if (st->done) return;  // uniform: only the last block at the barrier changes it
   const int q = threadIdx.x % P;
+  // one thread per rhs forms alpha (an FP64 division by every thread costs microseconds, see k_cg_update)
+  __shared__ float s_a[MAXR];
+  __shared__ int s_state[MAXR];  // 0 frozen, 1 stopped, 2 active
+  for (int rh = threadIdx.x; rh < 2 * P; rh += blockDim.x) {
+    const double pap = st->pAp[rh];
+    const bool fr = st->rhs_done[rh] != 0, act = !fr && pap > 0.0 && isfinite(pap);
+    s_a[rh] = act ? float(st->rr[rh] / pap) : 0.f;
+    s_state[rh] = fr ? 0 : act ? 2 : 1;
+  }
+  __syncthreads();
   bool active[2], frozen[2];
   float a[2];
   for (int k = 0; k < 2; ++k) {
-    const int rh = 2 * q + k;
-    const double pap = st->pAp[rh];
-    frozen[k] = st->rhs_done[rh] != 0;
-    active[k] = !frozen[k] && pap > 0.0 && isfinite(pap);
-    a[k] = active[k] ? float(st->rr[rh] / pap) : 0.f;
+    a[k] = s_a[2 * q + k];
+    frozen[k] = s_state[2 * q + k] == 0;
+    active[k] = s_state[2 * q + k] == 2;
   }
   const bool any = !frozen[0] || !frozen[1];
   const size_t w0 = blockIdx.x * (size_t)blockDim.x + threadIdx.x, stride = (size_t)gridDim.x * blockDim.x;
@@ -1227,9 +1266,12 @@ __global__ void k_ms_rupdate(S* __restrict__ r, const S* __restrict__ Ap, size_t
   using T = typename Real<S>::acc;
   constexpr int K = Chunk<S>::K;
   const double pap = st->pAp;
-  const double alpha = (pap > 0.0 && isfinite(pap)) ? st->rr / pap : 0.0;
+  __shared__ double s_alpha;  // one thread's division (see k_cg_update)
+  if (threadIdx.x == 0) s_alpha = (pap > 0.0 && isfinite(pap)) ? st->rr / pap : 0.0;
+  __syncthreads();
+  const double alpha = s_alpha;
   const T a = T(alpha);
-  double v = 0.0;
+  SumAcc<T> v;
   for (size_t i = (blockIdx.x * (size_t)blockDim.x + threadIdx.x) * K; i < n; i += (size_t)gridDim.x * blockDim.x * K) {
     cplx<T> rv[K], av[K];
     Chunk<S>::load(r, i / K, rv);
@@ -1242,11 +1284,11 @@ __global__ void k_ms_rupdate(S* __restrict__ r, const S* __restrict__ Ap, size_t
       t += rv[c].re * rv[c].re + rv[c].im * rv[c].im;
     }
     Chunk<S>::store(r, i / K, rv);
-    v += (double)t;
+    v.add(t);
   }
   __shared__ double red[32];
   __shared__ double s_tot;
-  double s = block_sum_dyn(v, red);
+  double s = block_sum_acc(v, red);
   if (threadIdx.x == 0) partials[blockIdx.x] = s;
   if (!last_block_done(counter)) return;
   double tot = sum_partials_dyn(partials, gridDim.x, red);
@@ -1260,6 +1302,7 @@ __global__ void k_ms_rupdate(S* __restrict__ r, const S* __restrict__ Ap, size_t
   __syncthreads();
   // the shifts' recurrences are independent: one thread each (GB300's FP64 divisions are slow in a
   // single thread's dependent chain)
+  if (threadIdx.x >= st->nshift) return;
   const double beta = s_tot / st->rr;
   const double s0 = st->sigma[st->base];
   for (int k = threadIdx.x; k < st->nshift; k += blockDim.x) {

@@ -49,6 +49,7 @@ struct DslashKArgs {
   size_t rhs_stride;  // sites between consecutive rhs vectors
   const void* y;      // EPI_AXPY
   double a[16];       // per-rhs diagonal coefficient 4m^2 + sigma_r
+  float af[16];       // the same rounded to FP32 (a conversion per thread would go through the FP64 pipe)
   double* partials;   // [NR][gridDim.x]
   double* dot_out;    // [NR]
   unsigned* counter;
@@ -61,6 +62,13 @@ struct DslashKArgs {
   int walk_chunk = 0;  // walk_zb * Lx Ly / 2: cb numbers per (tile, t) chunk
   unsigned long long walk_m_chunk = 0, walk_m_lt = 0;  // 2^64 / walk_chunk and 2^64 / Lt, rounded up
 };
+
+// Coefficient of vector r in the arithmetic of the axpy.
+template <typename EA>
+__device__ __forceinline__ EA axpy_coef(const DslashKArgs& k, int r) {
+  if constexpr (std::is_same<EA, float>::value) return k.af[r];
+  else return k.a[r];
+}
 
 // Output site of walk position w when the sites are walked in tiles of zb z-planes: tile by tile, and in
 // a tile t-slice by t-slice, each (tile, t) chunk being zb * Lx Ly / 2 consecutive cb numbers. In the
@@ -249,9 +257,7 @@ __global__ void __launch_bounds__(DslashBounds<LR, NR>::threads, DslashBounds<LR
   if (k.skip && *k.skip) return;  // uniform over the grid
   const Geom& g = k.g;
   const int p = k.out_parity;
-  double dot[NR];
-#pragma unroll
-  for (int r = 0; r < NR; ++r) dot[r] = 0.0;
+  SumAcc<SA> dot[NR];
   const int sub = TS == 1 ? 0 : (int)(threadIdx.x % TS);  // blockDim.x is a multiple of TS
   const int rbase = sub * NR;
   const size_t vbytes = (size_t)rbase * k.rhs_stride * 6 * sizeof(SR);
@@ -277,19 +283,18 @@ __global__ void __launch_bounds__(DslashBounds<LR, NR>::threads, DslashBounds<LR
         using EA = typename std::conditional<std::is_same<A, df64>::value, double, A>::type;
         cplx<SA> yv[3];
         VecIO<SR>::load(y, site, yv);
-        const EA a = EA(k.a[rbase + r]);
+        const EA a = axpy_coef<EA>(k, rbase + r);
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
           o[i].re = SA(fma(a, EA(yv[i].re), -EA(acc[r][i].re)));
           o[i].im = SA(fma(a, EA(yv[i].im), -EA(acc[r][i].im)));
         }
         if (k.partials) {
-          // the site's term in the arithmetic precision, summed over sites in FP64 (GB300's
-          // FP64 pipe is ~2 ops/clk/SM: one conversion and one add per site, not twelve)
+          // the site's term in the arithmetic precision, summed over sites to FP64 accuracy
           SA t = SA(0);
 #pragma unroll
           for (int i = 0; i < 3; ++i) t += yv[i].re * o[i].re + yv[i].im * o[i].im;
-          dot[r] += (double)t;
+          dot[r].add(t);
         }
       }
       VecIO<SR>::store(out, site, o);
@@ -301,8 +306,9 @@ __global__ void __launch_bounds__(DslashBounds<LR, NR>::threads, DslashBounds<LR
     __shared__ double red[32];
 #pragma unroll
     for (int R = 0; R < NR * TS; ++R) {
-      double s = block_sum_dyn(sub == R / NR ? dot[R % NR] : 0.0, red);
+      const double s = block_sum_acc(sub == R / NR ? dot[R % NR] : SumAcc<SA>(), red);
       if (threadIdx.x == 0) k.partials[(size_t)R * gridDim.x + blockIdx.x] = s;
+      __syncthreads();
     }
     if (last_block_done(k.counter)) {
       if constexpr (NR * TS == 1) {

@@ -187,7 +187,10 @@ int dslash_launch_t(hisq_ctx* ctx, const DslashCall& c) {
     a.in = (const char*)c.in + (size_t)r0 * c.rhs_stride * site_bytes;
     a.rhs_stride = c.rhs_stride;
     a.y = c.y ? (const char*)c.y + (size_t)r0 * c.rhs_stride * site_bytes : nullptr;
-    for (int r = 0; r < 16; ++r) a.a[r] = (c.a_rhs && r0 + r < c.nrhs) ? c.a_rhs[r0 + r] : c.a;
+    for (int r = 0; r < 16; ++r) {
+      a.a[r] = (c.a_rhs && r0 + r < c.nrhs) ? c.a_rhs[r0 + r] : c.a;
+      a.af[r] = (float)a.a[r];
+    }
     a.partials = c.partials ? c.partials + (size_t)r0 * partial_stride(ctx) : nullptr;
     a.dot_out = c.dot_out ? c.dot_out + r0 : nullptr;
     a.counter = c.counter;

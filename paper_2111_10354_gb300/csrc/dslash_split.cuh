@@ -64,9 +64,7 @@ __global__ void __launch_bounds__(SPLIT_MAX_BLOCK, sizeof(LR) < 8 && NR <= 2 ? 4
   const int spb = (int)blockDim.x / HS;  // sites per block
   const int r0 = blockIdx.y * NR;
   const char* in = (const char*)k.in + (size_t)r0 * k.rhs_stride * 6 * sizeof(SR);
-  double dot[NR];
-#pragma unroll
-  for (int r = 0; r < NR; ++r) dot[r] = 0.0;
+  SumAcc<SA> dot[NR];
 
   // all lanes of a warp stay in the loop together (the shares are combined by full-warp shuffles)
   for (int w0 = blockIdx.x * spb; w0 < g.half; w0 += gridDim.x * spb) {
@@ -132,22 +130,13 @@ __global__ void __launch_bounds__(SPLIT_MAX_BLOCK, sizeof(LR) < 8 && NR <= 2 ? 4
             o = SA(v[a]);
           } else {
             const SA yv = real_load((const SR*)k.y, base + 2 * a);
-            o = SA(fma(EA(k.a[r0 + r]), EA(yv), -EA(v[a])));
+            o = SA(fma(axpy_coef<EA>(k, r0 + r), EA(yv), -EA(v[a])));
             t += yv * o;
           }
           real_store((SR*)k.out, base + 2 * a, o);
         }
       }
-      if (EPI == EPI_AXPY && k.partials) {
-        // a site's term in the arithmetic precision; in FP32 summed over the shares first, so that a thread
-        // converts and adds one FP64 number per site as the other forms do
-        if constexpr (sizeof(SA) == 4) {
-#pragma unroll
-          for (int o = HS / 2; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-          if (j != 0) t = SA(0);
-        }
-        dot[r] += (double)t;
-      }
+      if (EPI == EPI_AXPY) dot[r].add(t);
     }
   }
 
@@ -156,8 +145,9 @@ __global__ void __launch_bounds__(SPLIT_MAX_BLOCK, sizeof(LR) < 8 && NR <= 2 ? 4
     __shared__ double red[32];
 #pragma unroll
     for (int r = 0; r < NR; ++r) {
-      const double s = block_sum_dyn(dot[r], red);
+      const double s = block_sum_acc(dot[r], red);
       if (threadIdx.x == 0) k.partials[(size_t)(r0 + r) * gridDim.x + blockIdx.x] = s;
+      __syncthreads();
     }
     if (last_block_done(k.counter)) {
       const int lane = threadIdx.x & 31, nw = blockDim.x >> 5, nr = NR * gridDim.y;

@@ -479,9 +479,10 @@ __device__ __forceinline__ double block_sum_dyn(double v, double* smem /* 32 */)
   if (l == 0) smem[w] = v;
   __syncthreads();
   double s = 0.0;
-  if (threadIdx.x == 0) {
-    const int nw = blockDim.x >> 5;
-    for (int k = 0; k < nw; ++k) s += smem[k];
+  if (threadIdx.x < 32) {  // a tree over the warps: FP64 adds are slow enough that a serial sum of 16 shows
+    s = l < (int)(blockDim.x >> 5) ? smem[l] : 0.0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
   }
   __syncthreads();
   return s;
@@ -492,9 +493,9 @@ __device__ __forceinline__ double block_sum_dyn(double v, double* smem /* 32 */)
 // reset by the last block so the next launch starts from zero.
 __device__ __forceinline__ bool last_block_done(unsigned* counter) {
   __shared__ bool is_last;
-  __threadfence();
   __syncthreads();
   if (threadIdx.x == 0) {
+    __threadfence();  // the block's writes, ordered before it by the barrier, before the count
     unsigned prev = atomicAdd(counter, 1u);
     is_last = (prev == gridDim.x * gridDim.y * gridDim.z - 1);
   }

@@ -1,52 +1,82 @@
-// Sums of per-block partial results by one warp or by a whole block, in a fixed order: shared by the
-// multi-RHS Dslash epilogues and the CG updates.
+// Reductions in a fixed order shared by the Dslash epilogues and the solvers' vector kernels: a thread's running
+// sum, its sum over a warp and a block, and sums of per-block partial results.
 #pragma once
 #include <cuda_runtime.h>
 
 namespace hisq {
+
+// A thread's running sum of terms in the arithmetic precision, kept to FP64 accuracy without FP64 instructions
+// where the terms are FP32: GB300's FP64 pipe takes a warp's operation in 16 cycles and is shared by the whole SM,
+// so a conversion and an add per term, five more per warp and a division per thread cost a streaming kernel
+// microseconds. FP32 terms go into an error-free pair (hi + lo, Knuth's two-sum: about 48 bits).
+template <typename T>
+struct SumAcc;
+template <>
+struct SumAcc<double> {
+  double v = 0.0;
+  __device__ __forceinline__ void add(double t) { v += t; }
+  // the sum over the warp, in every lane
+  __device__ __forceinline__ double warp_total() const {
+    double s = v;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    return s;
+  }
+};
+template <>
+struct SumAcc<float> {
+  float hi = 0.f, lo = 0.f;
+  __device__ __forceinline__ void add(float t) {
+    const float s = __fadd_rn(hi, t), b = __fsub_rn(s, hi);
+    lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(t, b)));
+    hi = s;
+  }
+  __device__ __forceinline__ double warp_total() const {
+    SumAcc<float> a = *this;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const float h = __shfl_xor_sync(0xffffffffu, a.hi, o), l = __shfl_xor_sync(0xffffffffu, a.lo, o);
+      a.add(h);
+      a.lo = __fadd_rn(a.lo, l);
+    }
+    // a sum beyond FP32's range (or a non-finite term) leaves hi non-finite and lo NaN: hi alone then says which
+    return isfinite(a.hi) ? (double)a.hi + (double)a.lo : (double)a.hi;
+  }
+};
+
+// Sum of every thread's a over the block (blockDim.x a multiple of 32); every lane of warp 0 gets it. smem: 32
+// doubles, free again after the caller's next __syncthreads.
+template <typename T>
+__device__ __forceinline__ double block_sum_acc(const SumAcc<T>& a, double* smem) {
+  const double w = a.warp_total();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (lane == 0) smem[warp] = w;
+  __syncthreads();
+  double s = 0.0;
+  if (warp == 0) {
+    s = lane < (int)(blockDim.x >> 5) ? smem[lane] : 0.0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  }
+  return s;
+}
 
 // Sum of partials[0..n) by the 32 lanes of one warp, in a fixed order: eight independent accumulators
 // per lane keep eight L2 loads in flight, then a fixed shuffle tree; every lane gets the total.
 __device__ __forceinline__ double warp_sum_partials(const double* partials, int n) {
   const int lane = threadIdx.x & 31;
   double s[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-  int i = lane;
-  for (; i + 7 * 32 < n; i += 8 * 32) {
+  for (int i = lane; i < n; i += 8 * 32) {
+    double v[8];
 #pragma unroll
-    for (int k = 0; k < 8; ++k) s[k] += __ldcg(partials + i + k * 32);
+    for (int k = 0; k < 8; ++k) v[k] = i + k * 32 < n ? __ldcg(partials + i + k * 32) : 0.0;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) s[k] += v[k];
   }
-  for (; i < n; i += 32) s[0] += __ldcg(partials + i);
   double t = ((s[0] + s[1]) + (s[2] + s[3])) + ((s[4] + s[5]) + (s[6] + s[7]));
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
   return t;
-}
-
-// Sum of partials[0..n) by a whole block (blockDim.x a multiple of 32), in a fixed order for a given n and
-// block size; every thread gets the total. Up to 4 blockDim.x partials every thread's loads are in flight
-// at once (one L2 round trip); beyond that warp 0 takes the loop above. red: blockDim.x / 32 doubles of
-// shared memory, free again on return.
-__device__ __forceinline__ double block_sum_partials(const double* partials, int n, double* red) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = blockDim.x >> 5, nb = blockDim.x;
-  const bool wide = n <= 4 * nb;
-  if (wide) {
-    double v[4];
-#pragma unroll
-    for (int k = 0; k < 4; ++k) v[k] = tid + k * nb < n ? __ldcg(partials + tid + k * nb) : 0.0;
-    double t = (v[0] + v[1]) + (v[2] + v[3]);
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
-    if (lane == 0) red[warp] = t;
-  } else if (warp == 0) {
-    const double t = warp_sum_partials(partials, n);
-    if (lane == 0) red[0] = t;
-  }
-  __syncthreads();
-  double s = red[0];
-  if (wide)
-    for (int w = 1; w < nw; ++w) s += red[w];
-  __syncthreads();
-  return s;
 }
 
 }  // namespace hisq

@@ -21,7 +21,7 @@ __global__ void k_selftest_wait(int* flag, uint32_t limit) {
 // One block waits at the fused CG update's grid barrier for a generation that nobody advances (the word
 // is zero and no block arrives), with the update's own bounded wait; when it gives up, the kernel records it.
 __global__ void k_selftest_grid_wait(int* flag, const unsigned* word, long limit) {
-  const bool passed = grid_wait64(word, 0u, limit);
+  const bool passed = grid_wait64_warp(word, 0u, limit);
   if (threadIdx.x == 0) *flag = passed ? 2 : 1;
 }
 

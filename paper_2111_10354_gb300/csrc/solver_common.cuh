@@ -169,9 +169,9 @@ __device__ __forceinline__ void grid_arrive_release(unsigned* bar, unsigned* gen
   __shared__ unsigned s_gen;
   __shared__ int s_last;
   unsigned long long* w = reinterpret_cast<unsigned long long*>(bar);
-  __threadfence();  // this block's partials become visible before its arrival
   __syncthreads();
   if (threadIdx.x == 0 && threadIdx.y == 0) {
+    __threadfence();  // the block's writes, ordered before it by the barrier, become visible before its arrival
     const unsigned nb = gridDim.x * gridDim.y * gridDim.z;
     const unsigned long long old = atomicAdd(w, 1ull);
     s_gen = (unsigned)(old >> 32);
@@ -183,13 +183,12 @@ __device__ __forceinline__ void grid_arrive_release(unsigned* bar, unsigned* gen
   *last = s_last != 0;
 }
 
-// Wait (bounded) until the generation in the high half has advanced past gen (acquire: every block's
-// partials are then visible). False on timeout.
-__device__ __forceinline__ bool grid_wait64(const unsigned* bar, unsigned gen, long limit = GRID_WAIT_POLLS) {
-  __shared__ int s_ok;
+// Wait (bounded) by one full warp until the generation in the high half has advanced past gen (acquire: every
+// block's partials are then visible): lane 0 polls, every lane gets the answer. False on timeout.
+__device__ __forceinline__ bool grid_wait64_warp(const unsigned* bar, unsigned gen, long limit = GRID_WAIT_POLLS) {
   const unsigned long long* w = reinterpret_cast<const unsigned long long*>(bar);
-  if (threadIdx.x == 0 && threadIdx.y == 0) {
-    int ok = 0;
+  int ok = 0;
+  if ((threadIdx.x & 31) == 0) {
     for (long it = 0; it < limit; ++it) {
       if ((unsigned)(ld_acquire_gpu64(w) >> 32) != gen) {
         ok = 1;
@@ -197,10 +196,8 @@ __device__ __forceinline__ bool grid_wait64(const unsigned* bar, unsigned gen, l
       }
       __nanosleep(32);
     }
-    s_ok = ok;
   }
-  __syncthreads();
-  return s_ok != 0;
+  return __shfl_sync(0xffffffffu, ok, 0) != 0;  // also orders the warp after lane 0's acquire
 }
 
 template <typename S>
