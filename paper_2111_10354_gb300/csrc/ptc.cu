@@ -15,6 +15,7 @@
 #include <math.h>
 #include <string.h>
 
+#include <algorithm>
 #include <chrono>
 #include <vector>
 
@@ -129,16 +130,51 @@ __global__ void __launch_bounds__(128, 7) k_ptc_apply_odd(const PtcGeom G, const
   }
 }
 
-// Pass 2, even sites x: z(x) = c0 r(x) + sum_h T_h phi_h (x).
+struct FcgState {
+  double pq;             // <p, A p> (real: A Hermitian positive)
+  double pr[2];          // <p, r>
+  double qz[2];          // <q, z>
+  double rr, rr_true, bb, tol2, scale;
+  int done, iter, cycle_iter, cycle_limit, conv, nonfinite, breakdown, pad;
+};
+
+// Sums of a complex quantity over the grid to FP64 accuracy: per-block partials, added in a fixed order by the last
+// block to finish; true in thread 0 of that block, with the totals in out. smem: 32 doubles.
+__device__ __forceinline__ bool grid_sum2(const SumAcc<float>& re, const SumAcc<float>& im, double* partials,
+                                          unsigned* counter, double* smem, double (&out)[2]) {
+  const double sr = block_sum_acc(re, smem);
+  __syncthreads();
+  const double si = block_sum_acc(im, smem);
+  if (threadIdx.x == 0) {
+    partials[blockIdx.x] = sr;
+    partials[gridDim.x + blockIdx.x] = si;
+  }
+  if (!last_block_done(counter)) return false;
+  if (threadIdx.x < 64) {
+    const double t = warp_sum_partials(partials + (threadIdx.x < 32 ? 0 : gridDim.x), gridDim.x);
+    if ((threadIdx.x & 31) == 0) smem[threadIdx.x >> 5] = t;
+  }
+  __syncthreads();
+  out[0] = smem[0];
+  out[1] = smem[1];
+  return threadIdx.x == 0;
+}
+
+// Pass 2, even sites x: z(x) = c0 r(x) + sum_h T_h phi_h (x). DOT: also st->qz = <q, z>, which saves the flexible
+// CG a launch and a read of z (12.5 us at 32^3x8).
+template <bool DOT>
 __global__ void __launch_bounds__(256) k_ptc_apply_even(const PtcGeom G, const float2* __restrict__ r,
                                                         const __half2* __restrict__ phi, float2* __restrict__ z,
-                                                        const float2* __restrict__ mix, const int* skip) {
+                                                        const float2* __restrict__ mix, const int* skip,
+                                                        const float2* __restrict__ q, FcgState* st, double* partials,
+                                                        unsigned* counter) {
   griddep_wait();  // a programmatic dependent launch (pdl.cuh): nothing is touched before this
   griddep_launch_dependents();
   if (skip && *skip) return;
   const Geom& g = G.g;
   const float2 m0 = __ldg(mix);
   const cplx<float> c0 = {m0.x, m0.y};
+  SumAcc<float> vr, vi;
   for (int cb = blockIdx.x * blockDim.x + threadIdx.x; cb < g.half; cb += gridDim.x * blockDim.x) {
     int c[4];
     site_coords(g, 0, cb, c);
@@ -172,6 +208,25 @@ __global__ void __launch_bounds__(256) k_ptc_apply_even(const PtcGeom G, const f
     }
 #pragma unroll
     for (int k = 0; k < 3; ++k) z[(size_t)cb * 3 + k] = make_float2(acc[k].re, acc[k].im);
+    if (DOT) {
+      float tr = 0.f, ti = 0.f;
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        const float2 w = __ldg(q + (size_t)cb * 3 + k);
+        tr += w.x * acc[k].re + w.y * acc[k].im;
+        ti += w.x * acc[k].im - w.y * acc[k].re;
+      }
+      vr.add(tr);
+      vi.add(ti);
+    }
+  }
+  if (DOT) {
+    __shared__ double red[32];
+    double t[2];
+    if (grid_sum2(vr, vi, partials, counter, red, t)) {
+      st->qz[0] = t[0];
+      st->qz[1] = t[1];
+    }
   }
 }
 
@@ -613,143 +668,87 @@ __global__ void k_adam(float* __restrict__ w, float* __restrict__ m, float* __re
 }
 
 // ------------------------------------------------------------------ flexible CG
-struct FcgState {
-  double pq;             // <p, A p> (real: A Hermitian positive)
-  double pr[2];          // <p, r>
-  double qz[2];          // <q, z>
-  double rr, rr_true, bb, tol2, scale;
-  int done, iter, cycle_iter, cycle_limit, conv, nonfinite, breakdown, pad;
-};
+// The updates take one 16-byte word (two complex entries) of every vector per thread; one thread per block forms the
+// complex quotients (see SumAcc on what FP64 costs). With a division by every thread and FP64 sums per site they
+// took 15.1 and 17.7 us a launch at 32^3x8 (ncu, caches flushed), now 11.8 and 13.2 us.
 
-__device__ __forceinline__ void load3(const float2* v, size_t site, float2 o[3]) {
-#pragma unroll
-  for (int k = 0; k < 3; ++k) o[k] = v[3 * site + k];
-}
-
-// alpha = <p, r> / <p, q>; e += alpha p; r -= alpha q; rr = |r|^2; inner convergence, cycle count.
-__global__ void k_fcg_update(float2* __restrict__ e, float2* __restrict__ r, const float2* __restrict__ p,
-                             const float2* __restrict__ q, int nsite, FcgState* st, double* partials,
-                             unsigned* counter) {
+// alpha = <p, r> / <p, q>; e += alpha p; r -= alpha q; rr = |r|^2; inner convergence, cycle count. nw: words.
+__global__ void __launch_bounds__(256) k_fcg_update(float4* __restrict__ e, float4* __restrict__ r,
+                                                    const float4* __restrict__ p, const float4* __restrict__ q, size_t nw,
+                                                    FcgState* st, double* partials, unsigned* counter) {
   if (st->done) return;
-  const double pq = st->pq;
-  const bool ok = pq > 0.0 && isfinite(pq);
-  const float ar = ok ? (float)(st->pr[0] / pq) : 0.f, ai = ok ? (float)(st->pr[1] / pq) : 0.f;
-  double v = 0.0;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nsite; i += gridDim.x * blockDim.x) {
-    float2 pv[3], qv[3], rv[3], ev[3];
-    load3(p, i, pv);
-    load3(q, i, qv);
-    load3(r, i, rv);
-    load3(e, i, ev);
-    float t = 0.f;
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      ev[k].x += ar * pv[k].x - ai * pv[k].y;
-      ev[k].y += ar * pv[k].y + ai * pv[k].x;
-      rv[k].x -= ar * qv[k].x - ai * qv[k].y;
-      rv[k].y -= ar * qv[k].y + ai * qv[k].x;
-      t += rv[k].x * rv[k].x + rv[k].y * rv[k].y;
-      e[3 * (size_t)i + k] = ev[k];
-      r[3 * (size_t)i + k] = rv[k];
-    }
-    v += (double)t;
-  }
   __shared__ double red[32];
-  const double s = block_sum_dyn(v, red);
+  __shared__ float s_ar, s_ai;
+  __shared__ int s_ok;
+  if (threadIdx.x == 0) {
+    const double pq = st->pq;
+    const bool ok = pq > 0.0 && isfinite(pq);
+    s_ar = ok ? (float)(st->pr[0] / pq) : 0.f;
+    s_ai = ok ? (float)(st->pr[1] / pq) : 0.f;
+    s_ok = ok;
+  }
+  __syncthreads();
+  const float ar = s_ar, ai = s_ai;
+  SumAcc<float> v;
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < nw; i += (size_t)gridDim.x * blockDim.x) {
+    const float4 pv = p[i], qv = q[i];
+    float4 rv = r[i], ev = e[i];
+    ev.x += ar * pv.x - ai * pv.y;
+    ev.y += ar * pv.y + ai * pv.x;
+    ev.z += ar * pv.z - ai * pv.w;
+    ev.w += ar * pv.w + ai * pv.z;
+    rv.x -= ar * qv.x - ai * qv.y;
+    rv.y -= ar * qv.y + ai * qv.x;
+    rv.z -= ar * qv.z - ai * qv.w;
+    rv.w -= ar * qv.w + ai * qv.z;
+    e[i] = ev;
+    r[i] = rv;
+    v.add((rv.x * rv.x + rv.y * rv.y) + (rv.z * rv.z + rv.w * rv.w));
+  }
+  const double s = block_sum_acc(v, red);
   if (threadIdx.x == 0) partials[blockIdx.x] = s;
-  if (!last_block_done(counter)) return;
-  const double tot = sum_partials_dyn(partials, gridDim.x, red);
+  if (!last_block_done(counter) || threadIdx.x >= 32) return;
+  const double tot = warp_sum_partials(partials, gridDim.x);
   if (threadIdx.x != 0) return;
   st->rr = tot;
-  if (!ok) st->breakdown = 1;
+  if (!s_ok) st->breakdown = 1;
   if (!isfinite(tot)) st->nonfinite = 1;
   st->iter += 1;
   st->cycle_iter += 1;
-  if (tot * st->scale * st->scale <= st->tol2 || st->cycle_iter >= st->cycle_limit || !ok || !isfinite(tot))
+  if (tot * st->scale * st->scale <= st->tol2 || st->cycle_iter >= st->cycle_limit || !s_ok || !isfinite(tot))
     st->done = 1;
 }
 
-// qz = <q, z> (complex, FP64 across sites)
-__global__ void k_fcg_qz(const float2* __restrict__ q, const float2* __restrict__ z, int nsite, FcgState* st,
-                         double* partials, unsigned* counter) {
+// p = z + beta p with beta = -<q, z> / <p, q> (restart: beta = 0); pr = <p, r>. nw: words.
+__global__ void __launch_bounds__(256) k_fcg_pupdate(float4* __restrict__ p, const float4* __restrict__ z,
+                                                     const float4* __restrict__ r, size_t nw, FcgState* st, int restart,
+                                                     double* partials, unsigned* counter) {
   if (st->done) return;
-  double vr = 0.0, vi = 0.0;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nsite; i += gridDim.x * blockDim.x) {
-    float2 qv[3], zv[3];
-    load3(q, i, qv);
-    load3(z, i, zv);
-    float tr = 0.f, ti = 0.f;
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      tr += qv[k].x * zv[k].x + qv[k].y * zv[k].y;
-      ti += qv[k].x * zv[k].y - qv[k].y * zv[k].x;
-    }
-    vr += (double)tr;
-    vi += (double)ti;
-  }
   __shared__ double red[32];
-  const double sr = block_sum_dyn(vr, red);
-  const double si = block_sum_dyn(vi, red);
+  __shared__ float s_br, s_bi;
   if (threadIdx.x == 0) {
-    partials[2 * blockIdx.x] = sr;
-    partials[2 * blockIdx.x + 1] = si;
+    s_br = restart ? 0.f : (float)(-st->qz[0] / st->pq);
+    s_bi = restart ? 0.f : (float)(-st->qz[1] / st->pq);
   }
-  if (!last_block_done(counter)) return;
-  double a = 0.0, b = 0.0;
-  for (int k = threadIdx.x; k < (int)gridDim.x; k += blockDim.x) {
-    a += __ldcg(partials + 2 * k);
-    b += __ldcg(partials + 2 * k + 1);
+  __syncthreads();
+  const float br = s_br, bi = s_bi;
+  SumAcc<float> vr, vi;
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < nw; i += (size_t)gridDim.x * blockDim.x) {
+    // a restart never reads p (it may hold stale data)
+    const float4 pv = restart ? make_float4(0.f, 0.f, 0.f, 0.f) : p[i], zv = z[i], rv = r[i];
+    float4 o;
+    o.x = zv.x + br * pv.x - bi * pv.y;
+    o.y = zv.y + br * pv.y + bi * pv.x;
+    o.z = zv.z + br * pv.z - bi * pv.w;
+    o.w = zv.w + br * pv.w + bi * pv.z;
+    p[i] = o;
+    vr.add((o.x * rv.x + o.y * rv.y) + (o.z * rv.z + o.w * rv.w));  // Re conj(p) r
+    vi.add((o.x * rv.y - o.y * rv.x) + (o.z * rv.w - o.w * rv.z));  // Im conj(p) r
   }
-  a = block_sum_dyn(a, red);
-  b = block_sum_dyn(b, red);
-  if (threadIdx.x == 0) {
-    st->qz[0] = a;
-    st->qz[1] = b;
-  }
-}
-
-// p = z + beta p with beta = -<q, z> / <p, q> (restart: beta = 0); pr = <p, r>.
-__global__ void k_fcg_pupdate(float2* __restrict__ p, const float2* __restrict__ z, const float2* __restrict__ r,
-                              int nsite, FcgState* st, int restart, double* partials, unsigned* counter) {
-  if (st->done) return;
-  const double pq = st->pq;
-  const float br = restart ? 0.f : (float)(-st->qz[0] / pq), bi = restart ? 0.f : (float)(-st->qz[1] / pq);
-  double vr = 0.0, vi = 0.0;
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nsite; i += gridDim.x * blockDim.x) {
-    float2 pv[3] = {}, zv[3], rv[3];
-    if (!restart) load3(p, i, pv);  // a restart never reads p (it may hold stale data)
-    load3(z, i, zv);
-    load3(r, i, rv);
-    float tr = 0.f, ti = 0.f;
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      const float nx = zv[k].x + br * pv[k].x - bi * pv[k].y;
-      const float ny = zv[k].y + br * pv[k].y + bi * pv[k].x;
-      p[3 * (size_t)i + k] = make_float2(nx, ny);
-      tr += nx * rv[k].x + ny * rv[k].y;  // Re conj(p) r
-      ti += nx * rv[k].y - ny * rv[k].x;  // Im conj(p) r
-    }
-    vr += (double)tr;
-    vi += (double)ti;
-  }
-  __shared__ double red[32];
-  const double sr = block_sum_dyn(vr, red);
-  const double si = block_sum_dyn(vi, red);
-  if (threadIdx.x == 0) {
-    partials[2 * blockIdx.x] = sr;
-    partials[2 * blockIdx.x + 1] = si;
-  }
-  if (!last_block_done(counter)) return;
-  double a = 0.0, b = 0.0;
-  for (int k = threadIdx.x; k < (int)gridDim.x; k += blockDim.x) {
-    a += __ldcg(partials + 2 * k);
-    b += __ldcg(partials + 2 * k + 1);
-  }
-  a = block_sum_dyn(a, red);
-  b = block_sum_dyn(b, red);
-  if (threadIdx.x == 0) {
-    st->pr[0] = a;
-    st->pr[1] = b;
+  double t[2];
+  if (grid_sum2(vr, vi, partials, counter, red, t)) {
+    st->pr[0] = t[0];
+    st->pr[1] = t[1];
   }
 }
 
@@ -878,18 +877,23 @@ static PtcGeom ptc_geom(const hisq_ctx* c) {
 // z = N(r) for nvec even-site FP32 vectors (device), using workspaces of the context: the composed
 // linear operator (mixing coefficients formed whenever the weights change, then one stencil pass over
 // odd and one over even sites); phi needs 8 * V/2 * 3 half2 of workspace.
-static int network_apply(hisq_ptc* P, float2* z, const float2* r, int nvec, __half2* phi, const int* skip = nullptr) {
+// With st: also st->qz = <q, z> (one vector).
+static int network_apply(hisq_ptc* P, float2* z, const float2* r, int nvec, __half2* phi, const int* skip = nullptr,
+                         const float2* q = nullptr, FcgState* st = nullptr, double* partials = nullptr) {
   hisq_ctx* c = P->ctx;
   const size_t nh = (size_t)c->g.half * 3;
   const PtcGeom G = ptc_geom(c);
   // one site per thread (the grid-stride loops then run once); the block scheduler balances the waves
-  const int grid_odd = (c->g.half + 127) / 128, grid_even = (c->g.half + 255) / 256;
+  const int grid_odd = (c->g.half + 127) / 128;
+  int grid_even = (c->g.half + 255) / 256;
+  if (st && grid_even > c->num_sms * 64) grid_even = c->num_sms * 64;  // the dot's partials: two per block
   for (int v = 0; v < nvec; ++v) {
     const float2* rv = r + v * nh;
     float2* zv = z + v * nh;
     const float2* mix = P->mix;
     HISQ_CUDA(launch_dependent(c, k_ptc_apply_odd, grid_odd, 128, G, rv, phi, mix, skip));
-    HISQ_CUDA(launch_dependent(c, k_ptc_apply_even, grid_even, 256, G, rv, (const __half2*)phi, zv, mix, skip));
+    HISQ_CUDA(launch_dependent(c, st ? k_ptc_apply_even<true> : k_ptc_apply_even<false>, grid_even, 256, G, rv,
+                               (const __half2*)phi, zv, mix, skip, q, st, partials, c->d_counters + 25));
     note_launch(c, 2);
   }
   return HISQ_OK;
@@ -1143,12 +1147,16 @@ int hisq_fcg(hisq_ctx* c, hisq_ptc* P, double* x_user, const double* b_user, dou
   h->tol2 = rel_tol * rel_tol * h->bb;
   HISQ_CUDA(cudaMemcpyAsync(&st->tol2, &h->tol2, sizeof(double), cudaMemcpyHostToDevice, c->stream));
   const int gb = c->num_sms * 4;
+  // the updates: a 16-byte word (two complex entries) per thread, at most one wave of six blocks per SM
+  const size_t nw = n / 2;
+  const int gu = (int)std::min<size_t>((nw + 255) / 256, (size_t)c->num_sms * 6);
   auto restart = [&]() -> int {
     k_fcg_reliable<<<gb, 256, 0, c->stream>>>(rh, r, n, st, c->d_counters + 21);
     HISQ_CUDA(cudaGetLastError());
     int r2 = network_apply(P, z, r, 1, phi, &st->done);
     if (r2 != HISQ_OK) return r2;
-    k_fcg_pupdate<<<gb, 256, 0, c->stream>>>(p, z, r, half, st, 1, red, c->d_counters + 22);
+    k_fcg_pupdate<<<gu, 256, 0, c->stream>>>((float4*)p, (const float4*)z, (const float4*)r, nw, st, 1, red,
+                                             c->d_counters + 22);
     HISQ_CUDA(cudaGetLastError());
     note_launch(c, 2);
     return HISQ_OK;
@@ -1179,13 +1187,14 @@ int hisq_fcg(hisq_ctx* c, hisq_ptc* P, double* x_user, const double* b_user, dou
     int r2 = dslash_launch(c, HISQ_F32, HISQ_F32, c1);
     if (r2 == HISQ_OK) r2 = dslash_launch(c, HISQ_F32, HISQ_F32, c2);
     if (r2 != HISQ_OK) return r2;
-    k_fcg_update<<<gb, 256, 0, c->stream>>>(e, r, p, q, half, st, red, c->d_counters + 24);
+    k_fcg_update<<<gu, 256, 0, c->stream>>>((float4*)e, (float4*)r, (const float4*)p, (const float4*)q, nw, st, red,
+                                            c->d_counters + 24);
     HISQ_CUDA(cudaGetLastError());
-    if ((r2 = network_apply(P, z, r, 1, phi, &st->done)) != HISQ_OK) return r2;
-    k_fcg_qz<<<gb, 256, 0, c->stream>>>(q, z, half, st, red, c->d_counters + 25);
-    k_fcg_pupdate<<<gb, 256, 0, c->stream>>>(p, z, r, half, st, 0, red, c->d_counters + 22);
+    if ((r2 = network_apply(P, z, r, 1, phi, &st->done, q, st, red)) != HISQ_OK) return r2;
+    k_fcg_pupdate<<<gu, 256, 0, c->stream>>>((float4*)p, (const float4*)z, (const float4*)r, nw, st, 0, red,
+                                             c->d_counters + 22);
     HISQ_CUDA(cudaGetLastError());
-    note_launch(c, 3);
+    note_launch(c, 2);
     return HISQ_OK;
   };
   // one graph = one reliable cycle
