@@ -17,6 +17,7 @@
 
 #include <algorithm>
 #include <chrono>
+#include <string>
 #include <vector>
 
 #include "internal.cuh"
@@ -1197,27 +1198,43 @@ int hisq_fcg(hisq_ctx* c, hisq_ptc* P, double* x_user, const double* b_user, dou
     note_launch(c, 2);
     return HISQ_OK;
   };
-  // one graph = one reliable cycle
-  cudaGraph_t graph;
-  cudaGraphExec_t exec = nullptr;
-  HISQ_CUDA(cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
-  c->capturing = true;
-  int crc = HISQ_OK;
-  for (int i = 0; i < o.reliable_period && crc == HISQ_OK; ++i) crc = iteration();
-  if (crc == HISQ_OK) {
-    k_fcg_fold<<<gb, 256, 0, c->stream>>>(x, e, n, st);
-    crc = fcg_true_residual(c, x, b, rh, Ax, t64, st, a, 0, red);
+  // one graph = the iterations of one reliable cycle, kept in the context for the next solves: it touches the
+  // context's workspaces, links and the network's mixing coefficients only (the caller's x and b enter in the
+  // launches after it)
+  std::string key = "fcg/" + std::to_string(o.reliable_period);
+  char buf[64];
+  for (const void* ptr : {(const void*)r, (const void*)p, (const void*)q, (const void*)t, (const void*)z, (const void*)e,
+                          (const void*)phi, (const void*)st, (const void*)partials, (const void*)P->mix}) {
+    snprintf(buf, sizeof buf, "/%p", ptr);
+    key += buf;
   }
-  if (crc == HISQ_OK) crc = restart();
-  c->capturing = false;
-  cudaError_t ce = cudaStreamEndCapture(c->stream, &graph);
-  if (crc != HISQ_OK) return crc;
-  HISQ_CUDA(ce);
-  size_t nodes = 0;
-  cudaGraphGetNodes(graph, nullptr, &nodes);
-  ce = cudaGraphInstantiate(&exec, graph, 0);
-  cudaGraphDestroy(graph);
-  HISQ_CUDA(ce);
+  snprintf(buf, sizeof buf, "/%a", a);
+  key += buf;
+  cudaGraphExec_t exec = nullptr;
+  long long nodes = 0;
+  auto cached = c->graphs.find(key);
+  if (cached != c->graphs.end()) {
+    exec = cached->second.first;
+    nodes = cached->second.second;
+  } else {
+    cudaGraph_t graph;
+    HISQ_CUDA(cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
+    c->capturing = true;
+    int crc = HISQ_OK;
+    for (int i = 0; i < o.reliable_period && crc == HISQ_OK; ++i) crc = iteration();
+    c->capturing = false;
+    cudaError_t ce = cudaStreamEndCapture(c->stream, &graph);
+    if (crc != HISQ_OK) return crc;
+    HISQ_CUDA(ce);
+    size_t gn = 0;
+    cudaGraphGetNodes(graph, nullptr, &gn);
+    nodes = (long long)gn;
+    ce = cudaGraphInstantiate(&exec, graph, 0);
+    cudaGraphDestroy(graph);
+    HISQ_CUDA(ce);
+    if (c->graphs.size() >= 32) release_graphs(c);  // bound the cache
+    c->graphs[key] = {exec, nodes};
+  }
   int status = HISQ_OK;
   int reliable = 0;
   HISQ_CUDA(cudaMemcpyAsync(h, st, sizeof(FcgState), cudaMemcpyDeviceToHost, c->stream));
@@ -1228,7 +1245,13 @@ int hisq_fcg(hisq_ctx* c, hisq_ptc* P, double* x_user, const double* b_user, dou
       break;
     }
     HISQ_CUDA(cudaGraphLaunch(exec, c->stream));
-    c->launches += (long long)nodes;
+    c->launches += nodes;
+    // the reliable update: fold the correction into x, true residual in FP64, restart
+    k_fcg_fold<<<gb, 256, 0, c->stream>>>(x, e, n, st);
+    HISQ_CUDA(cudaGetLastError());
+    note_launch(c);
+    if ((rc = fcg_true_residual(c, x, b, rh, Ax, t64, st, a, 0, red)) != HISQ_OK) return rc;
+    if ((rc = restart()) != HISQ_OK) return rc;
     ++reliable;
     HISQ_CUDA(cudaMemcpyAsync(h, st, sizeof(FcgState), cudaMemcpyDeviceToHost, c->stream));
     HISQ_CUDA(cudaStreamSynchronize(c->stream));
@@ -1241,7 +1264,6 @@ int hisq_fcg(hisq_ctx* c, hisq_ptc* P, double* x_user, const double* b_user, dou
       break;
     }
   }
-  cudaGraphExecDestroy(exec);
   const double rel = h->bb > 0 ? sqrt(h->rr_true / h->bb) : sqrt(h->rr_true);
   if (stats) {
     stats->iters = h->iter;
