@@ -262,9 +262,9 @@ int hisq_multishift_cg(hisq_ctx* ctx, double* x, const double* b, int nshift, co
 /*
  * A batch of independent lattices of (possibly) different sizes, solved together: every
  * step of the batched CG is one persistent launch over a tile table that covers all
- * lattices, and one CUDA graph holds a whole reliable cycle (inner iterations, fold, FP64
- * residual, reliable update). This is the many-small-lattices form of the paper's CG
- * (Sec. 2, Sec. 3); the paper itself batches right-hand sides, not lattices.
+ * lattices, and one CUDA graph holds the inner iterations of a reliable cycle. This is the
+ * many-small-lattices form of the paper's CG (Sec. 2, Sec. 3); the paper itself batches
+ * right-hand sides, not lattices.
  * dims: nlat x 4 extents (each even and >= 4), nlat <= 256. FP64 and FP32 links are always
  * resident. Vectors of the batch: the even-site vectors of all lattices back to back,
  * complex128 [lattice][V_l/2][3]; hisq_batch_vector_offset gives lattice l's first complex

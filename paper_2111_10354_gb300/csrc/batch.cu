@@ -1,15 +1,17 @@
 // Batched mixed-precision CG over many independent lattices of uneven sizes.
 //
-// Every step of the solve is one launch for all lattices: a persistent grid walks a table of
-// tiles (a tile = blockDim consecutive output sites of one lattice), so small and large
-// lattices share the GPU without one launch per lattice. Lattices that have met their inner
-// tolerance skip their tiles. Reductions are per lattice and deterministic: each tile writes
-// its partial, and the CTA that completes a lattice's last tile sums that lattice's partials
-// in tile order. One CUDA graph holds a whole reliable cycle -- reliable_period inner
-// iterations (FP32 links and spinors, FP32 correction e), the fold x += s e, the FP64 true
-// residual and the reliable update -- and the host only replays it and polls once per cycle.
-// Tile size (the block size of the batched Dslash) is chosen by the autotuner.
+// Every step of the solve is one launch for all lattices: a persistent grid walks the tiles (consecutive output
+// sites of one lattice) of the lattices that still iterate, so small and large lattices share the GPU without one
+// launch per lattice. Each block lists those lattices when it starts, from flags that no block of the launch changes
+// (they are committed by the last block of the grid to finish), so all blocks walk the same tiles; with a table of
+// all tiles, blocks spent a launch's last microseconds looking up tiles of finished lattices. Reductions are per
+// lattice and deterministic: each block writes its part, and the last block of a lattice's to do so sums them
+// in tile order. One CUDA graph, kept for the next solves, holds the reliable_period inner iterations of a
+// cycle (FP32 links and spinors, FP32 correction e); the fold x += s e, the FP64 true residual and the reliable
+// update follow it, and the host polls once per cycle.
+// The Dslash tile (its block size) is chosen by the autotuner.
 #include <math.h>
+#include <stdio.h>
 #include <string.h>
 
 #include <chrono>
@@ -30,90 +32,163 @@ constexpr int MAXB = 256;  // lattices per batch
 
 struct BatchState {
   double rr[MAXB], rr_new[MAXB], pAp[MAXB], bb[MAXB], tol2[MAXB], scale[MAXB], rr_true[MAXB], a[MAXB];
+  double alpha[MAXB], beta[MAXB];           // formed once per lattice (an FP64 division per thread costs microseconds)
+  float af[MAXB], alphaf[MAXB], betaf[MAXB];  // a, alpha and beta rounded to FP32
   int done[MAXB];   // frozen for the rest of the cycle (inner tolerance met, or verified)
   int conv[MAXB];   // true FP64 residual verified below tolerance
   int iters[MAXB];  // inner iterations per lattice
   unsigned cnt[6][MAXB];  // per-lattice tile counters, one row per reduction kernel
   unsigned grid_cnt[6];   // per-kernel CTA counters (last CTA does global bookkeeping)
-  int nlat, cycle_done, cycle_iter, cycle_limit, breakdown, nonfinite, all_conv, pad;
+  int nlat, cycle_done, cycle_iter, cycle_limit, breakdown, nonfinite, all_conv, x_nonzero;
 };
 
-// Device tables describing the batch for one tile size.
+// First tile of every lattice in a numbering of all tiles of one size (where the tiles' partials go).
 struct TileTable {
-  int block = 0;
   int ntiles = 0;
-  int* tile_lat = nullptr;   // [ntiles]
-  int* tile_cb0 = nullptr;   // [ntiles]
   int* lat_tile0 = nullptr;  // [nlat + 1]
 };
 
 struct BatchArgs {
-  const Geom* geoms;        // [nlat]
+  const Geom* geoms;         // [nlat]
   const char* const* links;  // [nlat] link storage of one precision
   const size_t* blk_bytes;   // [nlat]
   const size_t* site_off;    // [nlat] offset of lattice l's vectors, in sites
-  const int* tile_lat;
-  const int* tile_cb0;
   const int* lat_tile0;
-  int ntiles;
+  int tile;                  // sites per tile
   int nlat;
 };
 
-// ------------------------------------------------------------------ reduction helpers
-// Tile partial -> per-lattice total by the CTA completing the lattice's last tile.
-// Returns true (in all threads) in that CTA; thread 0 then holds the total in *total.
-__device__ __forceinline__ bool lattice_reduce(double v, int t, int l, const BatchArgs& a, double* partials,
-                                               unsigned* cnt, double* red, double* total) {
-  __shared__ bool last;
-  double s = block_sum_dyn(v, red);
-  if (threadIdx.x == 0) partials[t] = s;
-  __threadfence();
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    const unsigned n = (unsigned)(a.lat_tile0[l + 1] - a.lat_tile0[l]);
-    last = atomicAdd(&cnt[l], 1u) == n - 1;
+// ------------------------------------------------------------------ the lattices a launch works on
+struct ActiveTiles {
+  int n;               // lattices listed
+  int lat[MAXB];
+  int tile0[MAXB + 1];  // first tile of each in the launch's numbering; [n]: all tiles
+};
+
+// Lists the lattices whose skip flag is 0 (every thread of the block calls it).
+__device__ __forceinline__ void list_active(ActiveTiles& A, const BatchArgs& a, const int* skip) {
+  if (threadIdx.x < 32) {
+    const int lane = threadIdx.x;
+    int n = 0, tiles = 0;
+    for (int l0 = 0; l0 < a.nlat; l0 += 32) {
+      const int l = l0 + lane;
+      const bool on = l < a.nlat && !skip[l];
+      const int cnt = on ? (a.geoms[l].half + a.tile - 1) / a.tile : 0;
+      int incl = cnt;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int up = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += up;
+      }
+      const unsigned m = __ballot_sync(0xffffffffu, on);
+      if (on) {
+        const int k = n + __popc(m & ((1u << lane) - 1));
+        A.lat[k] = l;
+        A.tile0[k] = tiles + incl - cnt;
+      }
+      n += __popc(m);
+      tiles += __shfl_sync(0xffffffffu, incl, 31);
+    }
+    if (lane == 0) {
+      A.n = n;
+      A.tile0[n] = tiles;
+    }
   }
   __syncthreads();
-  if (!last) return false;
-  __threadfence();
-  double tot = sum_partials_dyn(partials + a.lat_tile0[l], a.lat_tile0[l + 1] - a.lat_tile0[l], red);
-  if (threadIdx.x == 0) {
-    cnt[l] = 0u;
-    *total = tot;
-  }
-  return true;
 }
 
-// True in thread 0 of the last CTA of the grid to reach this point.
+// The list number of tile t's lattice (binary search); *local: the tile's number within it.
+__device__ __forceinline__ int tile_lattice(const ActiveTiles& A, int t, int* local) {
+  int lo = 0, hi = A.n - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (A.tile0[mid] <= t) lo = mid;
+    else hi = mid - 1;
+  }
+  *local = t - A.tile0[lo];
+  return lo;
+}
+
+// ------------------------------------------------------------------ reduction helpers
+// The reducing launches give every block one contiguous range of the launch's tiles, [tile_begin(b), tile_begin(b+1)),
+// so that a block reduces once per lattice it meets (mostly one) instead of once per tile. With fewer tiles than
+// blocks the first blocks get one each and the others none.
+__device__ __forceinline__ unsigned tile_blocks(const ActiveTiles& A) { return min((unsigned)A.tile0[A.n], gridDim.x); }
+__device__ __forceinline__ int tile_begin(const ActiveTiles& A, unsigned b) {
+  const unsigned nb = tile_blocks(A);
+  return b >= nb ? A.tile0[A.n] : (int)((unsigned long long)A.tile0[A.n] * b / nb);
+}
+__device__ __forceinline__ int tile_owner(const ActiveTiles& A, int t) {  // the block whose range holds tile t
+  const unsigned nb = tile_blocks(A);
+  unsigned b = (unsigned)((unsigned long long)t * nb / (unsigned)A.tile0[A.n]);
+  while (b + 1 < nb && tile_begin(A, b + 1) <= t) ++b;
+  while (tile_begin(A, b) > t) --b;
+  return (int)b;
+}
+
+// This block's part of lattice number k (of the list)'s sum -> the total by the CTA that is last to bring its part.
+// Returns true in thread 0 of that CTA, with the total in *total.
+template <typename T>
+__device__ __forceinline__ bool lattice_reduce(const SumAcc<T>& v, const ActiveTiles& A, int k, const BatchArgs& a,
+                                               double* partials, unsigned* cnt, double* red, double* total) {
+  __shared__ bool last;
+  const double s = block_sum_acc(v, red);
+  const int l = A.lat[k], p0 = a.lat_tile0[l];
+  int n = 0;
+  if (threadIdx.x < 32) {  // the blocks that share this lattice
+    const int b0 = tile_owner(A, A.tile0[k]);
+    n = tile_owner(A, A.tile0[k + 1] - 1) - b0 + 1;
+    if (threadIdx.x == 0) {
+      partials[p0 + blockIdx.x - b0] = s;
+      __threadfence();
+      last = atomicAdd(&cnt[l], 1u) == (unsigned)n - 1;
+    }
+  }
+  __syncthreads();
+  if (!last || threadIdx.x >= 32) return false;
+  __threadfence();
+  *total = warp_sum_partials(partials + p0, n);
+  if (threadIdx.x == 0) cnt[l] = 0u;
+  return threadIdx.x == 0;
+}
+
+// True in every thread of the last CTA of the grid to reach this point.
 __device__ __forceinline__ bool grid_last(unsigned* c) {
   __shared__ bool last;
-  __threadfence();
   __syncthreads();
-  if (threadIdx.x == 0) last = atomicAdd(c, 1u) == gridDim.x - 1;
-  __syncthreads();
-  if (last && threadIdx.x == 0) {
+  if (threadIdx.x == 0) {
     __threadfence();
-    *c = 0u;
+    last = atomicAdd(c, 1u) == gridDim.x - 1;
+    if (last) {
+      __threadfence();
+      *c = 0u;
+    }
   }
-  return last && threadIdx.x == 0;
+  __syncthreads();
+  return last;
 }
 
 // ------------------------------------------------------------------ batched Dslash
-// out_l = D in_l (EPI_PLAIN) or out_l = a_l y_l - D in_l with pAp_l = Re<y_l, out_l> (EPI_AXPY),
-// for every lattice l whose skip[l] is 0.
+// out_l = D in_l (EPI_PLAIN) or out_l = a_l y_l - D in_l with pAp_l = Re<y_l, out_l> and alpha_l = rr_l / pAp_l
+// (EPI_AXPY), for every lattice l whose skip[l] is 0. FP32 is held to 64 registers like the single-lattice form.
 template <typename LR, typename SR, int EPI>
-__global__ void __launch_bounds__(256) k_bdslash(const BatchArgs a, int p, void* out, const void* in, const void* y,
-                                                 const int* skip, BatchState* st, double* partials, int red_row) {
+__global__ void __launch_bounds__(256, sizeof(LR) == 4 ? 4 : 2) k_bdslash(const BatchArgs a, int p, void* out, const void* in,
+                                                                         const void* y, const int* skip, BatchState* st,
+                                                                         double* partials, int red_row) {
   using A = typename Real<LR>::acc;
   using SA = typename Real<SR>::acc;
   __shared__ double red[32];
-  for (int t = blockIdx.x; t < a.ntiles; t += gridDim.x) {
-    const int l = a.tile_lat[t];
-    if (skip[l]) continue;  // uniform over the CTA
+  __shared__ ActiveTiles act;
+  list_active(act, a, skip);
+  constexpr bool RED = EPI == EPI_AXPY;
+  const int t1 = RED ? tile_begin(act, blockIdx.x + 1) : act.tile0[act.n];
+  SumAcc<SA> dot;
+  for (int t = RED ? tile_begin(act, blockIdx.x) : (int)blockIdx.x; t < t1; t += RED ? 1 : (int)gridDim.x) {
+    int local;
+    const int kl = tile_lattice(act, t, &local), l = act.lat[kl];
     const Geom g = a.geoms[l];
-    const int cb = a.tile_cb0[t] + threadIdx.x;
+    const int cb = local * a.tile + threadIdx.x;  // blockDim.x == a.tile
     const size_t base = a.site_off[l];
-    double dot = 0.0;
     if (cb < g.half) {
       cplx<A> acc[1][3];
       const char* in_l = (const char*)in + base * 6 * sizeof(SR);
@@ -125,7 +200,9 @@ __global__ void __launch_bounds__(256) k_bdslash(const BatchArgs a, int p, void*
       } else {
         cplx<SA> yv[3];
         VecIO<SR>::load(y, base + cb, yv);
-        const A al = A(st->a[l]);
+        A al;
+        if constexpr (std::is_same<A, float>::value) al = st->af[l];
+        else al = st->a[l];
         SA tt = SA(0);
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
@@ -133,113 +210,155 @@ __global__ void __launch_bounds__(256) k_bdslash(const BatchArgs a, int p, void*
           o[i].im = SA(fma(al, A(yv[i].im), -acc[0][i].im));
           tt += yv[i].re * o[i].re + yv[i].im * o[i].im;
         }
-        dot = (double)tt;
+        dot.add(tt);
       }
       VecIO<SR>::store(out, base + cb, o);
     }
-    if (EPI == EPI_AXPY) {
+    if (RED && (t + 1 == t1 || t + 1 == act.tile0[kl + 1])) {  // the block's last tile of this lattice
       double tot;
-      if (lattice_reduce(dot, t, l, a, partials, st->cnt[red_row], red, &tot) && threadIdx.x == 0) st->pAp[l] = tot;
+      if (lattice_reduce(dot, act, kl, a, partials, st->cnt[red_row], red, &tot)) {
+        st->pAp[l] = tot;
+        const double alpha = tot > 0.0 && isfinite(tot) ? st->rr[l] / tot : 0.0;
+        st->alpha[l] = alpha;
+        st->alphaf[l] = (float)alpha;
+      }
+      dot = SumAcc<SA>();
     }
   }
 }
 
 // ------------------------------------------------------------------ batched BLAS-1
-// e_l += alpha_l p_l; r_l -= alpha_l Ap_l; rr_new_l = |r_l|^2 (alpha_l = rr_l / pAp_l).
-template <typename S, typename X>
-__global__ void __launch_bounds__(256) k_bupdate(const BatchArgs a, X* e, S* r, const S* p, const S* Ap,
-                                                 BatchState* st, double* partials) {
+// Tiles of BLAS_TILE sites, whose 16-byte words (two complex FP32 entries, one FP64) a block of 256 takes three
+// (six) at a time, all loads before the first store.
+constexpr int BLAS_TILE = 512;
+template <typename S>
+struct Word;
+template <>
+struct Word<float> {
+  using V = float4;
+  static constexpr int PER_TILE = BLAS_TILE * 3 / 2, J = PER_TILE / 256;
+  __device__ __forceinline__ static V axpy(float a, V x, V y) {  // a x + y
+    return make_float4(fmaf(a, x.x, y.x), fmaf(a, x.y, y.y), fmaf(a, x.z, y.z), fmaf(a, x.w, y.w));
+  }
+  __device__ __forceinline__ static float norm2(V x) { return (x.x * x.x + x.y * x.y) + (x.z * x.z + x.w * x.w); }
+};
+template <>
+struct Word<double> {
+  using V = double2;
+  static constexpr int PER_TILE = BLAS_TILE * 3, J = PER_TILE / 256;
+  __device__ __forceinline__ static V axpy(double a, V x, V y) { return make_double2(fma(a, x.x, y.x), fma(a, x.y, y.y)); }
+  __device__ __forceinline__ static double norm2(V x) { return x.x * x.x + x.y * x.y; }
+};
+
+// e_l += alpha_l p_l; r_l -= alpha_l Ap_l; rr_new_l = |r_l|^2, beta_l = rr_new_l / rr_l. S = double: e is the FP64
+// solution itself (true units, scale_l); S = float: inner units, k_bfold scales.
+template <typename S>
+__global__ void __launch_bounds__(256) k_bupdate(const BatchArgs a, S* e, S* r, const S* p, const S* Ap, BatchState* st,
+                                                 double* partials) {
   if (st->cycle_done) return;
-  using T = typename Real<S>::acc;
-  using XT = typename Real<X>::acc;
+  using W = Word<S>;
+  using V = typename W::V;
+  constexpr bool F = std::is_same<S, float>::value;
   __shared__ double red[32];
-  for (int t = blockIdx.x; t < a.ntiles; t += gridDim.x) {
-    const int l = a.tile_lat[t];
-    if (st->done[l]) continue;
-    const int half = a.geoms[l].half;
-    const int cb = a.tile_cb0[t] + threadIdx.x;
-    const size_t site = a.site_off[l] + cb;
-    const double pap = st->pAp[l];
-    const bool ok = pap > 0.0 && isfinite(pap);
-    const double alpha = ok ? st->rr[l] / pap : 0.0;
-    double v = 0.0;
-    if (cb < half) {
-      cplx<T> pv[3], rv[3], av[3];
-      cplx<XT> xv[3];
-      VecIO<S>::load(p, site, pv);
-      VecIO<S>::load(r, site, rv);
-      VecIO<S>::load(Ap, site, av);
-      VecIO<X>::load(e, site, xv);
-      const T al = T(alpha);
-      // X = double: e is the FP64 solution itself (true units); X = float: inner units, k_bfold scales
-      const XT ax = XT(sizeof(X) == 8 ? alpha * st->scale[l] : alpha);
-      T tt = T(0);
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        xv[c].re = fma(ax, XT(pv[c].re), xv[c].re);
-        xv[c].im = fma(ax, XT(pv[c].im), xv[c].im);
-        rv[c].re = fma(-al, av[c].re, rv[c].re);
-        rv[c].im = fma(-al, av[c].im, rv[c].im);
-        tt += rv[c].re * rv[c].re + rv[c].im * rv[c].im;
-      }
-      VecIO<X>::store(e, site, xv);
-      VecIO<S>::store(r, site, rv);
-      v = (double)tt;
+  __shared__ ActiveTiles act;
+  list_active(act, a, st->done);
+  const int t1 = tile_begin(act, blockIdx.x + 1);
+  SumAcc<S> v;
+  for (int t = tile_begin(act, blockIdx.x); t < t1; ++t) {
+    int local;
+    const int kl = tile_lattice(act, t, &local), l = act.lat[kl];
+    const int nw = a.geoms[l].half * (W::PER_TILE / (BLAS_TILE / 2)) / 2;  // words of the lattice
+    const size_t off = a.site_off[l] * (W::PER_TILE / (BLAS_TILE / 2)) / 2;
+    const int w0 = local * W::PER_TILE + threadIdx.x;
+    S al, ax;
+    if constexpr (F) {
+      al = ax = st->alphaf[l];
+    } else {
+      al = st->alpha[l];
+      ax = al * st->scale[l];
     }
+    V rv[W::J], av[W::J], pv[W::J], xv[W::J];
+#pragma unroll
+    for (int j = 0; j < W::J; ++j) {
+      const int w = w0 + j * 256;
+      if (w < nw) {
+        rv[j] = reinterpret_cast<const V*>(r)[off + w];
+        av[j] = reinterpret_cast<const V*>(Ap)[off + w];
+        pv[j] = reinterpret_cast<const V*>(p)[off + w];
+        xv[j] = reinterpret_cast<const V*>(e)[off + w];
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < W::J; ++j) {
+      const int w = w0 + j * 256;
+      if (w < nw) {
+        rv[j] = W::axpy(-al, av[j], rv[j]);
+        reinterpret_cast<V*>(r)[off + w] = rv[j];
+        reinterpret_cast<V*>(e)[off + w] = W::axpy(ax, pv[j], xv[j]);
+        v.add(W::norm2(rv[j]));
+      }
+    }
+    if (t + 1 != t1 && t + 1 != act.tile0[kl + 1]) continue;
     double tot;
-    if (lattice_reduce(v, t, l, a, partials, st->cnt[1], red, &tot) && threadIdx.x == 0) {
+    if (lattice_reduce(v, act, kl, a, partials, st->cnt[1], red, &tot)) {
       st->rr_new[l] = tot;
-      if (!ok) st->breakdown = 1;
+      const double beta = tot / st->rr[l];
+      st->beta[l] = beta;
+      st->betaf[l] = (float)beta;
+      const double pap = st->pAp[l];
+      if (!(pap > 0.0 && isfinite(pap))) st->breakdown = 1;
       if (!isfinite(tot)) st->nonfinite = 1;
     }
+    v = SumAcc<S>();
   }
 }
 
-// p_l = r_l + beta_l p_l; per lattice (last tile): commit rr, count the iteration, inner
-// convergence; last CTA: end of cycle when every lattice is frozen or the cycle is full.
+// p_l = r_l + beta_l p_l; last CTA of the grid: per lattice commit rr, count the iteration, inner convergence; end
+// of cycle when every lattice is frozen or the cycle is full.
 template <typename S>
 __global__ void __launch_bounds__(256) k_bpupdate(const BatchArgs a, const S* r, S* p, BatchState* st) {
   if (st->cycle_done) return;
-  using T = typename Real<S>::acc;
-  __shared__ bool last;
-  for (int t = blockIdx.x; t < a.ntiles; t += gridDim.x) {
-    const int l = a.tile_lat[t];
-    if (st->done[l]) continue;
-    const int half = a.geoms[l].half;
-    const int cb = a.tile_cb0[t] + threadIdx.x;
-    if (cb < half) {
-      const size_t site = a.site_off[l] + cb;
-      const T beta = T(st->rr_new[l] / st->rr[l]);
-      cplx<T> pv[3], rv[3];
-      VecIO<S>::load(p, site, pv);
-      VecIO<S>::load(r, site, rv);
+  using W = Word<S>;
+  using V = typename W::V;
+  __shared__ ActiveTiles act;
+  list_active(act, a, st->done);
+  for (int t = blockIdx.x; t < act.tile0[act.n]; t += gridDim.x) {
+    int local;
+    const int l = act.lat[tile_lattice(act, t, &local)];
+    const int nw = a.geoms[l].half * (W::PER_TILE / (BLAS_TILE / 2)) / 2;
+    const size_t off = a.site_off[l] * (W::PER_TILE / (BLAS_TILE / 2)) / 2;
+    const int w0 = local * W::PER_TILE + threadIdx.x;
+    S beta;
+    if constexpr (std::is_same<S, float>::value) beta = st->betaf[l];
+    else beta = st->beta[l];
+    V rv[W::J], pv[W::J];
 #pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        pv[c].re = fma(beta, pv[c].re, rv[c].re);
-        pv[c].im = fma(beta, pv[c].im, rv[c].im);
+    for (int j = 0; j < W::J; ++j) {
+      const int w = w0 + j * 256;
+      if (w < nw) {
+        rv[j] = reinterpret_cast<const V*>(r)[off + w];
+        pv[j] = reinterpret_cast<const V*>(p)[off + w];
       }
-      VecIO<S>::store(p, site, pv);
     }
-    __threadfence();
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      const unsigned n = (unsigned)(a.lat_tile0[l + 1] - a.lat_tile0[l]);
-      last = atomicAdd(&st->cnt[2][l], 1u) == n - 1;
+#pragma unroll
+    for (int j = 0; j < W::J; ++j) {
+      const int w = w0 + j * 256;
+      if (w < nw) reinterpret_cast<V*>(p)[off + w] = W::axpy(beta, pv[j], rv[j]);
     }
-    __syncthreads();
-    if (last && threadIdx.x == 0) {
-      __threadfence();
-      st->cnt[2][l] = 0u;
-      st->rr[l] = st->rr_new[l];
-      st->iters[l] += 1;
-      const double s = st->scale[l];
-      if (st->rr[l] * s * s <= st->tol2[l]) st->done[l] = 1;
-    }
-    __syncthreads();
   }
-  if (grid_last(&st->grid_cnt[2])) {
-    bool all = true;
-    for (int l = 0; l < st->nlat; ++l) all = all && st->done[l];
+  if (!grid_last(&st->grid_cnt[2])) return;
+  bool all = true;
+  for (int l = threadIdx.x; l < st->nlat; l += blockDim.x) {
+    if (!st->done[l]) {
+      const double rr = st->rr_new[l], s = st->scale[l];
+      st->rr[l] = rr;
+      st->iters[l] += 1;
+      if (rr * s * s <= st->tol2[l]) st->done[l] = 1;
+      else all = false;
+    }
+  }
+  all = __syncthreads_and(all);
+  if (threadIdx.x == 0) {
     st->cycle_iter += 1;
     if (all || st->cycle_iter >= st->cycle_limit || st->breakdown || st->nonfinite) st->cycle_done = 1;
   }
@@ -247,106 +366,114 @@ __global__ void __launch_bounds__(256) k_bpupdate(const BatchArgs a, const S* r,
 
 // x_l += scale_l e_l; e_l = 0 (all lattices not yet verified).
 __global__ void __launch_bounds__(256) k_bfold(const BatchArgs a, double2* x, float* e, BatchState* st) {
-  for (int t = blockIdx.x; t < a.ntiles; t += gridDim.x) {
-    const int l = a.tile_lat[t];
-    if (st->conv[l]) continue;
-    const int cb = a.tile_cb0[t] + threadIdx.x;
-    if (cb >= a.geoms[l].half) continue;
-    const size_t site = a.site_off[l] + cb;
+  __shared__ ActiveTiles act;
+  list_active(act, a, st->conv);
+  for (int t = blockIdx.x; t < act.tile0[act.n]; t += gridDim.x) {
+    int local;
+    const int l = act.lat[tile_lattice(act, t, &local)];
+    const int n = a.geoms[l].half * 3;
+    const size_t off = a.site_off[l] * 3;
     const double s = st->scale[l];
-    float2* ep = reinterpret_cast<float2*>(e) + 3 * site;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const float2 ev = ep[c];
-      double2 xv = x[3 * site + c];
+    for (int i = local * BLAS_TILE * 3 + threadIdx.x; i < n && i < (local + 1) * BLAS_TILE * 3; i += 256) {
+      float2* ep = reinterpret_cast<float2*>(e) + off + i;
+      const float2 ev = *ep;
+      double2 xv = x[off + i];
       xv.x += s * (double)ev.x;
       xv.y += s * (double)ev.y;
-      x[3 * site + c] = xv;
-      ep[c] = make_float2(0.f, 0.f);
+      x[off + i] = xv;
+      *ep = make_float2(0.f, 0.f);
     }
   }
 }
 
-// r_hi = b - Ax (FP64); rr_true and (init) bb per lattice.
+// Sets st->x_nonzero if any of the n entries of the initial guess is not zero.
+__global__ void k_bnonzero(const double2* __restrict__ x, size_t n, BatchState* st) {
+  bool nz = false;
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+    const double2 v = x[i];
+    nz = nz || v.x != 0.0 || v.y != 0.0;
+  }
+  if (nz) st->x_nonzero = 1;
+}
+
+// r_hi = b - Ax (FP64; Ax null: a zero guess, r_hi = b); rr_true and (init) bb per lattice.
 __global__ void __launch_bounds__(256) k_bresidual(const BatchArgs a, const double2* b, const double2* Ax, double2* rh,
-                                                   BatchState* st, double* partials, int init) {
+                                                   BatchState* st, double* partials, size_t pstride, int init) {
   __shared__ double red[32];
-  for (int t = blockIdx.x; t < a.ntiles; t += gridDim.x) {
-    const int l = a.tile_lat[t];
-    if (st->conv[l]) continue;
-    const int cb = a.tile_cb0[t] + threadIdx.x;
-    double v0 = 0.0, v1 = 0.0;
-    if (cb < a.geoms[l].half) {
-      const size_t site = a.site_off[l] + cb;
-#pragma unroll
-      for (int c = 0; c < 3; ++c) {
-        const double2 bv = b[3 * site + c], av = Ax[3 * site + c];
-        const double2 rv = make_double2(bv.x - av.x, bv.y - av.y);
-        rh[3 * site + c] = rv;
-        v0 += rv.x * rv.x + rv.y * rv.y;
-        v1 += bv.x * bv.x + bv.y * bv.y;
-      }
+  __shared__ ActiveTiles act;
+  list_active(act, a, st->conv);
+  const int t1 = tile_begin(act, blockIdx.x + 1);
+  SumAcc<double> v0, v1;
+  for (int t = tile_begin(act, blockIdx.x); t < t1; ++t) {
+    int local;
+    const int kl = tile_lattice(act, t, &local), l = act.lat[kl];
+    const int n = a.geoms[l].half * 3;
+    const size_t off = a.site_off[l] * 3;
+    for (int i = local * BLAS_TILE * 3 + threadIdx.x; i < n && i < (local + 1) * BLAS_TILE * 3; i += 256) {
+      const double2 bv = b[off + i], av = Ax ? Ax[off + i] : make_double2(0.0, 0.0);
+      const double2 rv = make_double2(bv.x - av.x, bv.y - av.y);
+      rh[off + i] = rv;
+      v0.add(rv.x * rv.x + rv.y * rv.y);
+      if (init) v1.add(bv.x * bv.x + bv.y * bv.y);
     }
+    if (t + 1 != t1 && t + 1 != act.tile0[kl + 1]) continue;
     double tot;
-    if (lattice_reduce(v0, t, l, a, partials, st->cnt[3], red, &tot) && threadIdx.x == 0) {
+    if (lattice_reduce(v0, act, kl, a, partials, st->cnt[3], red, &tot)) {
       st->rr_true[l] = tot;
       if (!isfinite(tot)) st->nonfinite = 1;
     }
-    if (init) {
-      if (lattice_reduce(v1, t, l, a, partials + a.ntiles, st->cnt[4], red, &tot) && threadIdx.x == 0)
-        st->bb[l] = tot;
-    }
+    __syncthreads();
+    if (init && lattice_reduce(v1, act, kl, a, partials + pstride, st->cnt[4], red, &tot)) st->bb[l] = tot;
+    __syncthreads();
+    v0 = v1 = SumAcc<double>();
   }
 }
 
-// Reliable update per lattice not yet verified: r_lo = r_hi / s, p = r_lo, rr = rr_true / s^2;
-// verified lattices are frozen for good. Last CTA: new cycle, or all verified.
+// Reliable update per lattice not yet verified: r_lo = r_hi / s, p = r_lo, rr = rr_true / s^2; verified lattices
+// are frozen for good. Last CTA: the per-lattice bookkeeping; new cycle, or all verified.
 template <typename S>
 __global__ void __launch_bounds__(256) k_breliable(const BatchArgs a, const double2* rh, S* r, S* p, BatchState* st) {
-  __shared__ bool last;
-  for (int t = blockIdx.x; t < a.ntiles; t += gridDim.x) {
-    const int l = a.tile_lat[t];
-    if (st->conv[l]) continue;
-    const int half = a.geoms[l].half;
-    const int cb = a.tile_cb0[t] + threadIdx.x;
-    const double n = 3.0 * half;
-    const bool c = st->rr_true[l] <= st->tol2[l];
-    const double s = sqrt(st->rr_true[l] / n);
-    if (!c && s > 0.0 && cb < half) {
-      const size_t site = a.site_off[l] + cb;
-      const double inv = 1.0 / s;
-      using T = typename Real<S>::acc;
-      cplx<T> v[3];
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        const double2 w = rh[3 * site + k];
-        v[k] = {T(w.x * inv), T(w.y * inv)};
-      }
-      VecIO<S>::store(r, site, v);
-      VecIO<S>::store(p, site, v);
-    }
-    __threadfence();
+  __shared__ ActiveTiles act;
+  __shared__ double s_inv;
+  list_active(act, a, st->conv);
+  for (int t = blockIdx.x; t < act.tile0[act.n]; t += gridDim.x) {
+    int local;
+    const int l = act.lat[tile_lattice(act, t, &local)];
+    const int n = a.geoms[l].half * 3;
+    const size_t off = a.site_off[l] * 3;
     __syncthreads();
     if (threadIdx.x == 0) {
-      const unsigned nt = (unsigned)(a.lat_tile0[l + 1] - a.lat_tile0[l]);
-      last = atomicAdd(&st->cnt[5][l], 1u) == nt - 1;
+      const double s = sqrt(st->rr_true[l] / (double)n);
+      s_inv = !(st->rr_true[l] <= st->tol2[l]) && s > 0.0 ? 1.0 / s : 0.0;
     }
     __syncthreads();
-    if (last && threadIdx.x == 0) {
-      __threadfence();
-      st->cnt[5][l] = 0u;
-      st->conv[l] = c;
-      st->done[l] = c;
-      if (!c && s > 0.0) {
-        st->scale[l] = s;
-        st->rr[l] = st->rr_true[l] / (s * s);
-      }
+    const double inv = s_inv;
+    if (inv == 0.0) continue;  // verified now: frozen (uniform over the block)
+    for (int i = local * BLAS_TILE * 3 + threadIdx.x; i < n && i < (local + 1) * BLAS_TILE * 3; i += 256) {
+      const double2 w = rh[off + i];
+      const S re = S(w.x * inv), im = S(w.y * inv);
+      r[2 * (off + i)] = re;
+      r[2 * (off + i) + 1] = im;
+      p[2 * (off + i)] = re;
+      p[2 * (off + i) + 1] = im;
     }
-    __syncthreads();
   }
-  if (grid_last(&st->grid_cnt[5])) {
-    bool all = true;
-    for (int l = 0; l < st->nlat; ++l) all = all && st->conv[l];
+  if (!grid_last(&st->grid_cnt[5])) return;
+  bool all = true;
+  for (int l = threadIdx.x; l < st->nlat; l += blockDim.x) {
+    if (st->conv[l]) continue;
+    const bool c = st->rr_true[l] <= st->tol2[l];
+    const double s = sqrt(st->rr_true[l] / (3.0 * a.geoms[l].half));
+    st->conv[l] = c;
+    st->done[l] = c;
+    if (!c && s > 0.0) {
+      st->scale[l] = s;
+      st->rr[l] = st->rr_true[l] / (s * s);
+    }
+    all = all && c;
+  }
+  all = __syncthreads_and(all);
+  if (threadIdx.x == 0) {
     st->all_conv = all;
     st->cycle_done = all ? 1 : 0;
     st->cycle_iter = 0;
@@ -374,9 +501,16 @@ struct hisq_batch {
   std::map<std::string, DevBuf> ws;
   void* pinned = nullptr;
   long long launches = 0;
+  // instantiated iteration graphs, keyed by what their kernels capture
+  std::map<std::string, std::pair<cudaGraphExec_t, long long>> graphs;
 };
 
 namespace hisq {
+
+static void release_batch_graphs(hisq_batch* B) {
+  for (auto& kv : B->graphs) cudaGraphExecDestroy(kv.second.first);
+  B->graphs.clear();
+}
 
 static void* bws(hisq_batch* B, const char* name, size_t bytes) {
   DevBuf& b = B->ws[name];
@@ -396,46 +530,31 @@ static void* bws(hisq_batch* B, const char* name, size_t bytes) {
   return b.ptr;
 }
 
-static int tile_table(hisq_batch* B, int block, TileTable** out) {
-  auto it = B->tiles.find(block);
+static int tile_table(hisq_batch* B, int tile, TileTable** out) {
+  auto it = B->tiles.find(tile);
   if (it != B->tiles.end()) {
     *out = &it->second;
     return HISQ_OK;
   }
-  std::vector<int> tl, tc, l0;
-  for (int l = 0; l < B->nlat; ++l) {
-    l0.push_back((int)tl.size());
-    const int half = B->lat[l]->g.half;
-    for (int cb = 0; cb < half; cb += block) {
-      tl.push_back(l);
-      tc.push_back(cb);
-    }
-  }
-  l0.push_back((int)tl.size());
+  std::vector<int> l0 = {0};
+  for (int l = 0; l < B->nlat; ++l) l0.push_back(l0.back() + (B->lat[l]->g.half + tile - 1) / tile);
   TileTable T;
-  T.block = block;
-  T.ntiles = (int)tl.size();
-  HISQ_CUDA(cudaMalloc(&T.tile_lat, tl.size() * sizeof(int)));
-  HISQ_CUDA(cudaMalloc(&T.tile_cb0, tc.size() * sizeof(int)));
+  T.ntiles = l0.back();
   HISQ_CUDA(cudaMalloc(&T.lat_tile0, l0.size() * sizeof(int)));
-  HISQ_CUDA(cudaMemcpy(T.tile_lat, tl.data(), tl.size() * sizeof(int), cudaMemcpyHostToDevice));
-  HISQ_CUDA(cudaMemcpy(T.tile_cb0, tc.data(), tc.size() * sizeof(int), cudaMemcpyHostToDevice));
   HISQ_CUDA(cudaMemcpy(T.lat_tile0, l0.data(), l0.size() * sizeof(int), cudaMemcpyHostToDevice));
-  B->tiles[block] = T;
-  *out = &B->tiles[block];
+  B->tiles[tile] = T;
+  *out = &B->tiles[tile];
   return HISQ_OK;
 }
 
-static BatchArgs batch_args(hisq_batch* B, int prec, const TileTable& T) {
+static BatchArgs batch_args(hisq_batch* B, int prec, int tile, const TileTable& T) {
   BatchArgs a;
   a.geoms = B->d_geoms;
   a.links = B->d_links[prec];
   a.blk_bytes = B->d_blk[prec];
   a.site_off = B->d_site_off;
-  a.tile_lat = T.tile_lat;
-  a.tile_cb0 = T.tile_cb0;
   a.lat_tile0 = T.lat_tile0;
-  a.ntiles = T.ntiles;
+  a.tile = tile;
   a.nlat = B->nlat;
   return a;
 }
@@ -454,6 +573,7 @@ struct BatchBufs {
   void *r, *p, *Ap, *t, *e;
   BatchState* st;
   double* partials;
+  size_t pstride;  // doubles per row of partials
 };
 
 // Launch the batched Dslash in link/spinor type LR/SR with the tuned tile size.
@@ -482,7 +602,7 @@ static int bdslash(hisq_batch* B, int p, void* out, const void* in, const void* 
       TileTable* T;
       int rc = tile_table(B, c, &T);
       if (rc != HISQ_OK) return rc;
-      const BatchArgs a = batch_args(B, Real<LR>::prec, *T);
+      const BatchArgs a = batch_args(B, Real<LR>::prec, c, *T);
       const int grid = persistent_grid(B, (const void*)kern, c);
       kern<<<grid, c, 0, B->stream>>>(a, p, out, in, y, skip, st, partials, red_row);
       cudaEventRecord(e0, B->stream);
@@ -504,7 +624,7 @@ static int bdslash(hisq_batch* B, int p, void* out, const void* in, const void* 
   TileTable* T;
   int rc = tile_table(B, block, &T);
   if (rc != HISQ_OK) return rc;
-  const BatchArgs a = batch_args(B, Real<LR>::prec, *T);
+  const BatchArgs a = batch_args(B, Real<LR>::prec, block, *T);
   kern<<<persistent_grid(B, (const void*)kern, block), block, 0, B->stream>>>(a, p, out, in, y, skip, st, partials,
                                                                             red_row);
   HISQ_CUDA(cudaGetLastError());
@@ -512,28 +632,33 @@ static int bdslash(hisq_batch* B, int p, void* out, const void* in, const void* 
   return HISQ_OK;
 }
 
-template <typename S>
-static int blas_args(hisq_batch* B, BatchArgs* a, int* grid) {
+// Arguments of the BLAS kernels and their grid: one wave of resident blocks, or a block per tile if those are fewer.
+static int blas_args(hisq_batch* B, const void* func, BatchArgs* a, int* grid) {
   TileTable* T;
-  int rc = tile_table(B, 256, &T);
+  int rc = tile_table(B, BLAS_TILE, &T);
   if (rc != HISQ_OK) return rc;
-  *a = batch_args(B, HISQ_F64, *T);
-  *grid = B->num_sms * 8;
+  *a = batch_args(B, HISQ_F64, BLAS_TILE, *T);
+  *grid = persistent_grid(B, func, 256);
+  if (*grid > T->ntiles) *grid = T->ntiles;
   return HISQ_OK;
 }
 
-// r_hi = b - A_64 x for every lattice not yet verified.
-static int b_true_residual(hisq_batch* B, const BatchBufs& U, int init) {
-  int rc = bdslash<double, double, EPI_PLAIN>(B, 1, U.t64, U.x, nullptr, U.st->conv, U.st, U.partials, 0);
-  if (rc != HISQ_OK) return rc;
-  // the FP64 A uses a_l from the state and writes pAp, which the inner loop recomputes anyway
-  rc = bdslash<double, double, EPI_AXPY>(B, 0, U.Ax, U.t64, U.x, U.st->conv, U.st, U.partials, 0);
-  if (rc != HISQ_OK) return rc;
+// r_hi = b - A_64 x for every lattice not yet verified (zero: x is zero and A x need not be formed).
+static int b_true_residual(hisq_batch* B, const BatchBufs& U, int init, bool zero = false) {
+  int rc;
+  if (!zero) {
+    rc = bdslash<double, double, EPI_PLAIN>(B, 1, U.t64, U.x, nullptr, U.st->conv, U.st, U.partials, 0);
+    if (rc != HISQ_OK) return rc;
+    // the FP64 A uses a_l from the state and writes pAp and alpha, which the inner loop recomputes anyway
+    rc = bdslash<double, double, EPI_AXPY>(B, 0, U.Ax, U.t64, U.x, U.st->conv, U.st, U.partials, 0);
+    if (rc != HISQ_OK) return rc;
+  }
   BatchArgs a;
   int grid;
-  if ((rc = blas_args<double>(B, &a, &grid)) != HISQ_OK) return rc;
-  k_bresidual<<<grid, 256, 0, B->stream>>>(a, U.b, U.Ax, U.rh, U.st, U.partials, init);
+  if ((rc = blas_args(B, (const void*)k_bresidual, &a, &grid)) != HISQ_OK) return rc;
+  k_bresidual<<<grid, 256, 0, B->stream>>>(a, U.b, zero ? nullptr : U.Ax, U.rh, U.st, U.partials, U.pstride, init);
   HISQ_CUDA(cudaGetLastError());
+  B->launches += 1;
   return HISQ_OK;
 }
 
@@ -541,16 +666,16 @@ template <typename S>
 static int b_reliable(hisq_batch* B, const BatchBufs& U) {
   BatchArgs a;
   int grid;
-  int rc = blas_args<S>(B, &a, &grid);
+  int rc = blas_args(B, (const void*)k_breliable<S>, &a, &grid);
   if (rc != HISQ_OK) return rc;
   k_breliable<S><<<grid, 256, 0, B->stream>>>(a, U.rh, (S*)U.r, (S*)U.p, U.st);
   HISQ_CUDA(cudaGetLastError());
+  B->launches += 1;
   return HISQ_OK;
 }
 
 template <typename S>
 static int b_iteration(hisq_batch* B, const BatchBufs& U, int lp) {
-  using X = typename std::conditional<sizeof(S) == 8, double, float>::type;
   int rc;
   if (lp == HISQ_F64) {
     rc = bdslash<double, double, EPI_PLAIN>(B, 1, U.t, U.p, nullptr, U.st->done, U.st, U.partials, 0);
@@ -563,9 +688,10 @@ static int b_iteration(hisq_batch* B, const BatchBufs& U, int lp) {
   if (rc != HISQ_OK) return rc;
   BatchArgs a;
   int grid;
-  if ((rc = blas_args<S>(B, &a, &grid)) != HISQ_OK) return rc;
-  k_bupdate<S, X><<<grid, 256, 0, B->stream>>>(a, (X*)U.e, (S*)U.r, (const S*)U.p, (const S*)U.Ap, U.st,
-                                                U.partials + 2 * (size_t)a.ntiles);
+  if ((rc = blas_args(B, (const void*)k_bupdate<S>, &a, &grid)) != HISQ_OK) return rc;
+  k_bupdate<S><<<grid, 256, 0, B->stream>>>(a, (S*)U.e, (S*)U.r, (const S*)U.p, (const S*)U.Ap, U.st,
+                                            U.partials + 2 * U.pstride);
+  if ((rc = blas_args(B, (const void*)k_bpupdate<S>, &a, &grid)) != HISQ_OK) return rc;
   k_bpupdate<S><<<grid, 256, 0, B->stream>>>(a, (const S*)U.r, (S*)U.p, U.st);
   HISQ_CUDA(cudaGetLastError());
   return HISQ_OK;
@@ -594,6 +720,7 @@ static int run_batch(hisq_batch* B, double2* x, const double2* b, const double* 
   size_t max_tiles = 0;
   for (int l = 0; l < B->nlat; ++l) max_tiles += (B->lat[l]->g.half + 63) / 64;
   U.partials = (double*)bws(B, "partials", 4 * max_tiles * sizeof(double));
+  U.pstride = max_tiles;
   if (!U.rh || !U.Ax || !U.t64 || !U.r || !U.p || !U.Ap || !U.t || !U.e || !U.st || !U.partials)
     return set_error(HISQ_ENOMEM, "batch workspace");
   BatchState* h = (BatchState*)B->pinned;
@@ -603,10 +730,17 @@ static int run_batch(hisq_batch* B, double2* x, const double2* b, const double* 
   for (int l = 0; l < B->nlat; ++l) {
     h->scale[l] = 1.0;
     h->a[l] = 4.0 * mass[l] * mass[l];
+    h->af[l] = (float)h->a[l];
   }
   HISQ_CUDA(cudaMemcpyAsync(U.st, h, sizeof(BatchState), cudaMemcpyHostToDevice, B->stream));
   if (mixed) HISQ_CUDA(cudaMemsetAsync(U.e, 0, n * 2 * sizeof(float), B->stream));
-  int rc = b_true_residual(B, U, 1);
+  // a zero initial guess (the usual start) needs no A x: its residual is b
+  k_bnonzero<<<B->num_sms * 8, 256, 0, B->stream>>>(x, n, U.st);
+  HISQ_CUDA(cudaGetLastError());
+  B->launches += 1;
+  HISQ_CUDA(cudaMemcpyAsync(&h->x_nonzero, &U.st->x_nonzero, sizeof(int), cudaMemcpyDeviceToHost, B->stream));
+  HISQ_CUDA(cudaStreamSynchronize(B->stream));
+  int rc = b_true_residual(B, U, 1, h->x_nonzero == 0);
   if (rc != HISQ_OK) return rc;
   HISQ_CUDA(cudaMemcpyAsync(h, U.st, sizeof(BatchState), cudaMemcpyDeviceToHost, B->stream));
   HISQ_CUDA(cudaStreamSynchronize(B->stream));
@@ -628,29 +762,53 @@ static int run_batch(hisq_batch* B, double2* x, const double2* b, const double* 
   }
   if (rc != HISQ_OK) return rc;
 
-  // one graph = one reliable cycle: inner iterations, fold, FP64 residual, reliable update
+  // one graph = the inner iterations of one reliable cycle, kept in the batch for the next solves: it touches the
+  // batch's own buffers only, except that FP64 solves accumulate in the caller's x (which is then in the key); x
+  // and b enter in the launches after it
   const int cycle = h->cycle_limit;
-  cudaGraph_t graph;
-  cudaGraphExec_t exec = nullptr;
-  HISQ_CUDA(cudaStreamBeginCapture(B->stream, cudaStreamCaptureModeThreadLocal));
-  int crc = HISQ_OK;
-  for (int i = 0; i < cycle && crc == HISQ_OK; ++i) crc = b_iteration<S>(B, U, lp);
-  if (crc == HISQ_OK && mixed) {
-    BatchArgs a;
-    int grid;
-    crc = blas_args<S>(B, &a, &grid);
-    if (crc == HISQ_OK) k_bfold<<<grid, 256, 0, B->stream>>>(a, U.x, (float*)U.e, U.st);
+  std::string key = "b/" + std::to_string(lp) + "/" + std::to_string(cycle);
+  char buf[64];
+  for (const void* ptr : {(const void*)U.r, (const void*)U.p, (const void*)U.Ap, (const void*)U.t, (const void*)U.e,
+                          (const void*)U.st, (const void*)U.partials}) {
+    snprintf(buf, sizeof buf, "/%p", ptr);
+    key += buf;
   }
-  if (crc == HISQ_OK) crc = b_true_residual(B, U, 0);
-  if (crc == HISQ_OK) crc = b_reliable<S>(B, U);
-  cudaError_t ce = cudaStreamEndCapture(B->stream, &graph);
-  if (crc != HISQ_OK) return crc;
-  HISQ_CUDA(ce);
-  size_t nodes = 0;
-  cudaGraphGetNodes(graph, nullptr, &nodes);
-  ce = cudaGraphInstantiate(&exec, graph, 0);
-  cudaGraphDestroy(graph);
-  HISQ_CUDA(ce);
+  cudaGraphExec_t exec = nullptr;
+  long long nodes = 0;
+  auto cached = B->graphs.find(key);
+  if (cached != B->graphs.end()) {
+    exec = cached->second.first;
+    nodes = cached->second.second;
+  } else {
+    cudaGraph_t graph;
+    HISQ_CUDA(cudaStreamBeginCapture(B->stream, cudaStreamCaptureModeThreadLocal));
+    int crc = HISQ_OK;
+    for (int i = 0; i < cycle && crc == HISQ_OK; ++i) crc = b_iteration<S>(B, U, lp);
+    cudaError_t ce = cudaStreamEndCapture(B->stream, &graph);
+    if (crc != HISQ_OK) return crc;
+    HISQ_CUDA(ce);
+    size_t gn = 0;
+    cudaGraphGetNodes(graph, nullptr, &gn);
+    nodes = (long long)gn;
+    ce = cudaGraphInstantiate(&exec, graph, 0);
+    cudaGraphDestroy(graph);
+    HISQ_CUDA(ce);
+    if (B->graphs.size() >= 8) release_batch_graphs(B);  // bound the cache
+    B->graphs[key] = {exec, nodes};
+  }
+  auto reliable_update = [&]() -> int {
+    int r2;
+    if (mixed) {
+      BatchArgs a;
+      int grid;
+      if ((r2 = blas_args(B, (const void*)k_bfold, &a, &grid)) != HISQ_OK) return r2;
+      k_bfold<<<grid, 256, 0, B->stream>>>(a, U.x, (float*)U.e, U.st);
+      HISQ_CUDA(cudaGetLastError());
+      B->launches += 1;
+    }
+    if ((r2 = b_true_residual(B, U, 0)) != HISQ_OK) return r2;
+    return b_reliable<S>(B, U);
+  };
 
   int status = HISQ_OK;
   int cycles = 0;
@@ -664,7 +822,8 @@ static int run_batch(hisq_batch* B, double2* x, const double2* b, const double* 
       break;
     }
     HISQ_CUDA(cudaGraphLaunch(exec, B->stream));
-    B->launches += (long long)nodes;
+    B->launches += nodes;
+    if ((rc = reliable_update()) != HISQ_OK) return rc;
     ++cycles;
     HISQ_CUDA(cudaMemcpyAsync(h, U.st, sizeof(BatchState), cudaMemcpyDeviceToHost, B->stream));
     HISQ_CUDA(cudaStreamSynchronize(B->stream));
@@ -677,7 +836,6 @@ static int run_batch(hisq_batch* B, double2* x, const double2* b, const double* 
       break;
     }
   }
-  cudaGraphExecDestroy(exec);
   double worst = 0.0;
   int total_it = 0;
   for (int l = 0; l < B->nlat; ++l) {
@@ -772,6 +930,7 @@ int hisq_batch_create(hisq_batch** out, int nlat, const int* dims, unsigned prec
 int hisq_batch_destroy(hisq_batch* B) {
   if (!B) return HISQ_OK;
   if (B->stream) cudaStreamSynchronize(B->stream);
+  release_batch_graphs(B);
   for (auto* c : B->lat) hisq_destroy(c);
   cudaFree(B->d_geoms);
   cudaFree(B->d_site_off);
@@ -779,11 +938,7 @@ int hisq_batch_destroy(hisq_batch* B) {
     cudaFree(B->d_links[p]);
     cudaFree(B->d_blk[p]);
   }
-  for (auto& kv : B->tiles) {
-    cudaFree(kv.second.tile_lat);
-    cudaFree(kv.second.tile_cb0);
-    cudaFree(kv.second.lat_tile0);
-  }
+  for (auto& kv : B->tiles) cudaFree(kv.second.lat_tile0);
   for (auto& kv : B->ws) cudaFree(kv.second.ptr);
   if (B->pinned) cudaFreeHost(B->pinned);
   if (B->own_stream) cudaStreamDestroy(B->stream);
