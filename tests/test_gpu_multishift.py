@@ -98,3 +98,29 @@ def test_rational_apply(hisq, inner):
     assert st["converged"] == 1
     ref = oracle.rational_apply(L, ff, lf, mass, b, a0, coeffs, shifts, tol=1e-13)
     assert np.linalg.norm(out.cpu().numpy() - ref) / np.linalg.norm(ref) < 1e-8
+
+
+@pytest.mark.parametrize("inner", [0, 1])
+def test_multishift_group_lengths_bitwise(hisq, inner):
+    """The other shifts' updates are applied once per group of up to 8 iterations, whose length follows from the poll
+    interval: 1 (every iteration, as the recurrence is written), 7 (one short group), 8, 9 (8 and 1) and 25 give
+    the same bits, shifts that converge inside a group and the one group that the solve leaves unfinished
+    included. The tolerance is one that FP32 meets, so no refinement follows that could hide a difference."""
+    import torch
+    L = (8, 10, 12, 14)
+    fat, lng = hin.gen_links(L, 1234, 0.3, 0.1)
+    lat = hisq.Lattice(L, precs=(0, 1)).load(fat, lng)
+    b = torch.from_numpy(hin.gen_source(4321, lat.half, 1)).cuda()
+    shifts = np.array([0.02, 1e-3, 0.3, 1e-3, 2.0])  # unsorted, one repeated
+    outs, its = [], []
+    for poll in (1, 7, 8, 9, 25):
+        x = torch.zeros((len(shifts), lat.half, 3), dtype=torch.complex128, device="cuda")
+        rc, st = hisq.hisq_multishift_cg(lat.ctx, x, b, shifts, 0.05, 1e-4, 4000,
+                                         hisq.make_opts(inner_prec=inner, poll_every=poll, reliable_period=4000))
+        assert rc == 0
+        outs.append(x.clone())
+        its.append(st["shift_iters"])
+    assert all(i == its[0] for i in its), its
+    assert min(its[0]) < max(its[0])
+    for o in outs[1:]:
+        assert torch.equal(o, outs[0])
