@@ -126,25 +126,15 @@ __device__ __forceinline__ void store_m(typename FieldIO<T>::S* f, size_t V, int
   for (int k = 0; k < 9; ++k) FieldIO<T>::st(f + (size_t)k * V + s, m.e[k]);
 }
 
-// m = a * f0[s] + b * (f1[s] + f2[s]); f2 may be null (m = a f0 + b f1), and f1 too (m = a f0)
+// m = f0[s] + b f1[s] (f1 may be null: m = f0)
 template <typename T>
-__device__ __forceinline__ void load_comb(M3<T>& m, const typename FieldIO<T>::S* f0, T a,
-                                          const typename FieldIO<T>::S* f1, const typename FieldIO<T>::S* f2, T b,
-                                          size_t V, int s) {
-  const T z = FieldIO<T>::zero();
+__device__ __forceinline__ void load_sum(M3<T>& m, const typename FieldIO<T>::S* f0, const typename FieldIO<T>::S* f1, T b,
+                                         size_t V, int s) {
 #pragma unroll
   for (int k = 0; k < 9; ++k) {
-    const cplx<T> u = FieldIO<T>::ld(f0 + (size_t)k * V + s);
-    cplx<T> r;
-    r.re = fma(a, u.re, z);
-    r.im = fma(a, u.im, z);
+    cplx<T> r = FieldIO<T>::ld(f0 + (size_t)k * V + s);
     if (f1) {
-      cplx<T> w = FieldIO<T>::ld(f1 + (size_t)k * V + s);
-      if (f2) {
-        const cplx<T> w2 = FieldIO<T>::ld(f2 + (size_t)k * V + s);
-        w.re = w.re + w2.re;
-        w.im = w.im + w2.im;
-      }
+      const cplx<T> w = FieldIO<T>::ld(f1 + (size_t)k * V + s);
       r.re = fma(b, w.re, r.re);
       r.im = fma(b, w.im, r.im);
     }
@@ -384,7 +374,7 @@ __global__ void __launch_bounds__(SMEAR_MAX_BLOCK, MINB) k_smear_fat(const typen
   int c[4];
   lex_coords(g, s, c);
   const S* Umu = U + (size_t)mu * 9 * V;
-  const T one = FieldIO<T>::coef(1.0), tL = FieldIO<T>::coef(cL), tN = FieldIO<T>::coef(cN);
+  const T tL = FieldIO<T>::coef(cL), tN = FieldIO<T>::coef(cN);
   const int s_mu = step(g, s, c[mu], mu, 1);
   M3<T> f;
   load_m(f, Umu, V, s, false);
@@ -404,8 +394,8 @@ __global__ void __launch_bounds__(SMEAR_MAX_BLOCK, MINB) k_smear_fat(const typen
       Ua = U + (size_t)a * 9 * V;
       y0 = bwd ? step(g, s, c[a], a, -1) : s;
       sc = step(g, y0, c[mu], mu, 1);
-      load_comb(z, Y + (size_t)ai * 9 * V, one, cL != 0.0 ? St + (size_t)it * 9 * V : (const S*)nullptr,
-                (const S*)nullptr, tL, V, bwd ? y0 : step(g, s, c[a], a, 1));
+      load_sum(z, Y + (size_t)ai * 9 * V, cL != 0.0 ? St + (size_t)it * 9 * V : (const S*)nullptr, tL, V,
+               bwd ? y0 : step(g, s, c[a], a, 1));
     } else {
       store_link(fat, s, mu, f);
       zero_m(f);
@@ -413,7 +403,8 @@ __global__ void __launch_bounds__(SMEAR_MAX_BLOCK, MINB) k_smear_fat(const typen
       Ua = Umu;
       y0 = s;
       sc = step(g, s_mu, c[mu] + 1 < g.L[mu] ? c[mu] + 1 : 0, mu, 1);
-      load_comb(z, Umu, tN, (const S*)nullptr, (const S*)nullptr, tN, V, s_mu);
+      load_m(z, Umu, V, s_mu, false);
+      scale_m(z, tN);
     }
     load_m(u, Ua, V, y0, bwd);
     mul_nn(p, u, z);
