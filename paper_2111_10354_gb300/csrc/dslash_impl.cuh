@@ -303,13 +303,10 @@ __global__ void __launch_bounds__(DslashBounds<LR, NR>::threads, DslashBounds<LR
 
   if (EPI == EPI_AXPY) {
     if (k.partials == nullptr) return;  // uniform over the grid
-    __shared__ double red[32];
-#pragma unroll
-    for (int R = 0; R < NR * TS; ++R) {
-      const double s = block_sum_acc(sub == R / NR ? dot[R % NR] : SumAcc<SA>(), red);
-      if (threadIdx.x == 0) k.partials[(size_t)R * gridDim.x + blockIdx.x] = s;
-      __syncthreads();
-    }
+    __shared__ double red[NR * TS > 2 ? NR * TS * 16 : 32];
+    block_sums_acc<NR * TS>(
+        red, [&](int R) { return sub == R / NR ? dot[R % NR] : SumAcc<SA>(); },
+        [&](int R, double s) { k.partials[(size_t)R * gridDim.x + blockIdx.x] = s; });
     if (last_block_done(k.counter)) {
       if constexpr (NR * TS == 1) {
         double s = sum_partials_dyn(k.partials, gridDim.x, red);

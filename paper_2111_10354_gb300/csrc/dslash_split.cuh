@@ -142,13 +142,10 @@ __global__ void __launch_bounds__(SPLIT_MAX_BLOCK, sizeof(LR) < 8 && NR <= 2 ? 4
 
   if (EPI == EPI_AXPY) {
     if (k.partials == nullptr) return;  // uniform over the grid
-    __shared__ double red[32];
-#pragma unroll
-    for (int r = 0; r < NR; ++r) {
-      const double s = block_sum_acc(dot[r], red);
-      if (threadIdx.x == 0) k.partials[(size_t)(r0 + r) * gridDim.x + blockIdx.x] = s;
-      __syncthreads();
-    }
+    __shared__ double red[NR > 2 ? NR * 16 : 32];
+    block_sums_acc<NR>(
+        red, [&](int r) { return dot[r]; },
+        [&](int r, double s) { k.partials[(size_t)(r0 + r) * gridDim.x + blockIdx.x] = s; });
     if (last_block_done(k.counter)) {
       const int lane = threadIdx.x & 31, nw = blockDim.x >> 5, nr = NR * gridDim.y;
       if (nr == 1) {

@@ -61,6 +61,25 @@ __device__ __forceinline__ double block_sum_acc(const SumAcc<T>& a, double* smem
   return s;
 }
 
+// Sums of several quantities over the block with one barrier: get(q) is this thread's running sum of quantity q < N;
+// put(q, s) is called by one lane with each total. smem: N * 16 doubles (blocks of at most 512 threads).
+template <int N, typename Get, typename Put>
+__device__ __forceinline__ void block_sums_acc(double* smem, Get get, Put put) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+#pragma unroll
+  for (int q = 0; q < N; ++q) {
+    const double w = get(q).warp_total();
+    if (lane == 0) smem[q * 16 + warp] = w;
+  }
+  __syncthreads();
+  for (int q = warp; q < N; q += nw) {  // a warp per quantity
+    double s = lane < nw ? smem[q * 16 + lane] : 0.0;
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) put(q, s);
+  }
+}
+
 // Sum of partials[0..n) by the 32 lanes of one warp, in a fixed order: eight independent accumulators
 // per lane keep eight L2 loads in flight, then a fixed shuffle tree; every lane gets the total.
 __device__ __forceinline__ double warp_sum_partials(const double* partials, int n) {
