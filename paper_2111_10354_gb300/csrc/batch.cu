@@ -61,6 +61,7 @@ struct BatchArgs {
 // ------------------------------------------------------------------ the lattices a launch works on
 struct ActiveTiles {
   int n;               // lattices listed
+  unsigned nb, q, rem;  // blocks that get tiles in the reducing launches; tiles / nb and tiles % nb
   int lat[MAXB];
   int tile0[MAXB + 1];  // first tile of each in the launch's numbering; [n]: all tiles
 };
@@ -72,8 +73,10 @@ __device__ __forceinline__ void list_active(ActiveTiles& A, const BatchArgs& a, 
     int n = 0, tiles = 0;
     for (int l0 = 0; l0 < a.nlat; l0 += 32) {
       const int l = l0 + lane;
-      const bool on = l < a.nlat && !skip[l];
-      const int cnt = on ? (a.geoms[l].half + a.tile - 1) / a.tile : 0;
+      // flag and tile count in flight together
+      const int sk = l < a.nlat ? skip[l] : 1, t0 = a.lat_tile0[min(l, a.nlat)], t1 = a.lat_tile0[min(l + 1, a.nlat)];
+      const bool on = sk == 0;
+      const int cnt = on ? t1 - t0 : 0;
       int incl = cnt;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
@@ -92,6 +95,9 @@ __device__ __forceinline__ void list_active(ActiveTiles& A, const BatchArgs& a, 
     if (lane == 0) {
       A.n = n;
       A.tile0[n] = tiles;
+      A.nb = min((unsigned)tiles, gridDim.x);
+      A.q = A.nb ? tiles / A.nb : 0;
+      A.rem = tiles - A.q * A.nb;
     }
   }
   __syncthreads();
@@ -113,17 +119,12 @@ __device__ __forceinline__ int tile_lattice(const ActiveTiles& A, int t, int* lo
 // The reducing launches give every block one contiguous range of the launch's tiles, [tile_begin(b), tile_begin(b+1)),
 // so that a block reduces once per lattice it meets (mostly one) instead of once per tile. With fewer tiles than
 // blocks the first blocks get one each and the others none.
-__device__ __forceinline__ unsigned tile_blocks(const ActiveTiles& A) { return min((unsigned)A.tile0[A.n], gridDim.x); }
 __device__ __forceinline__ int tile_begin(const ActiveTiles& A, unsigned b) {
-  const unsigned nb = tile_blocks(A);
-  return b >= nb ? A.tile0[A.n] : (int)((unsigned long long)A.tile0[A.n] * b / nb);
+  return b >= A.nb ? A.tile0[A.n] : (int)(b * A.q + min(b, A.rem));
 }
 __device__ __forceinline__ int tile_owner(const ActiveTiles& A, int t) {  // the block whose range holds tile t
-  const unsigned nb = tile_blocks(A);
-  unsigned b = (unsigned)((unsigned long long)t * nb / (unsigned)A.tile0[A.n]);
-  while (b + 1 < nb && tile_begin(A, b + 1) <= t) ++b;
-  while (tile_begin(A, b) > t) --b;
-  return (int)b;
+  const unsigned big = A.rem * (A.q + 1);  // the first rem blocks have a tile more
+  return (unsigned)t < big ? (int)((unsigned)t / (A.q + 1)) : (int)(A.rem + ((unsigned)t - big) / A.q);
 }
 
 // This block's part of lattice number k (of the list)'s sum -> the total by the CTA that is last to bring its part.
@@ -170,9 +171,10 @@ __device__ __forceinline__ bool grid_last(unsigned* c) {
 
 // ------------------------------------------------------------------ batched Dslash
 // out_l = D in_l (EPI_PLAIN) or out_l = a_l y_l - D in_l with pAp_l = Re<y_l, out_l> and alpha_l = rr_l / pAp_l
-// (EPI_AXPY), for every lattice l whose skip[l] is 0. FP32 is held to 64 registers like the single-lattice form.
+// (EPI_AXPY), for every lattice l whose skip[l] is 0. FP32 takes 80 registers (three blocks of 256 per SM): at 64, like
+// the single-lattice form, the tile walk spills (16 lattices, all active: 174 and 196 us against 164 and 181 us).
 template <typename LR, typename SR, int EPI>
-__global__ void __launch_bounds__(256, sizeof(LR) == 4 ? 4 : 2) k_bdslash(const BatchArgs a, int p, void* out, const void* in,
+__global__ void __launch_bounds__(256, sizeof(LR) == 4 ? 3 : 2) k_bdslash(const BatchArgs a, int p, void* out, const void* in,
                                                                          const void* y, const int* skip, BatchState* st,
                                                                          double* partials, int red_row) {
   using A = typename Real<LR>::acc;
@@ -228,15 +230,15 @@ __global__ void __launch_bounds__(256, sizeof(LR) == 4 ? 4 : 2) k_bdslash(const 
 }
 
 // ------------------------------------------------------------------ batched BLAS-1
-// Tiles of BLAS_TILE sites, whose 16-byte words (two complex FP32 entries, one FP64) a block of 256 takes three
-// (six) at a time, all loads before the first store.
-constexpr int BLAS_TILE = 512;
+// Tiles of BLAS_TILE sites, whose 16-byte words (two complex FP32 entries, one FP64) a block of BLAS_BLOCK takes one
+// (two) per thread, all loads before the first store. Larger tiles leave SMs idle in small batches.
+constexpr int BLAS_TILE = 128, BLAS_BLOCK = BLAS_TILE * 3 / 2;
 template <typename S>
 struct Word;
 template <>
 struct Word<float> {
   using V = float4;
-  static constexpr int PER_TILE = BLAS_TILE * 3 / 2, J = PER_TILE / 256;
+  static constexpr int PER_TILE = BLAS_TILE * 3 / 2, J = PER_TILE / BLAS_BLOCK;
   __device__ __forceinline__ static V axpy(float a, V x, V y) {  // a x + y
     return make_float4(fmaf(a, x.x, y.x), fmaf(a, x.y, y.y), fmaf(a, x.z, y.z), fmaf(a, x.w, y.w));
   }
@@ -245,7 +247,7 @@ struct Word<float> {
 template <>
 struct Word<double> {
   using V = double2;
-  static constexpr int PER_TILE = BLAS_TILE * 3, J = PER_TILE / 256;
+  static constexpr int PER_TILE = BLAS_TILE * 3, J = PER_TILE / BLAS_BLOCK;
   __device__ __forceinline__ static V axpy(double a, V x, V y) { return make_double2(fma(a, x.x, y.x), fma(a, x.y, y.y)); }
   __device__ __forceinline__ static double norm2(V x) { return x.x * x.x + x.y * x.y; }
 };
@@ -253,7 +255,7 @@ struct Word<double> {
 // e_l += alpha_l p_l; r_l -= alpha_l Ap_l; rr_new_l = |r_l|^2, beta_l = rr_new_l / rr_l. S = double: e is the FP64
 // solution itself (true units, scale_l); S = float: inner units, k_bfold scales.
 template <typename S>
-__global__ void __launch_bounds__(256) k_bupdate(const BatchArgs a, S* e, S* r, const S* p, const S* Ap, BatchState* st,
+__global__ void __launch_bounds__(BLAS_BLOCK) k_bupdate(const BatchArgs a, S* e, S* r, const S* p, const S* Ap, BatchState* st,
                                                  double* partials) {
   if (st->cycle_done) return;
   using W = Word<S>;
@@ -280,7 +282,7 @@ __global__ void __launch_bounds__(256) k_bupdate(const BatchArgs a, S* e, S* r, 
     V rv[W::J], av[W::J], pv[W::J], xv[W::J];
 #pragma unroll
     for (int j = 0; j < W::J; ++j) {
-      const int w = w0 + j * 256;
+      const int w = w0 + j * BLAS_BLOCK;
       if (w < nw) {
         rv[j] = reinterpret_cast<const V*>(r)[off + w];
         av[j] = reinterpret_cast<const V*>(Ap)[off + w];
@@ -290,7 +292,7 @@ __global__ void __launch_bounds__(256) k_bupdate(const BatchArgs a, S* e, S* r, 
     }
 #pragma unroll
     for (int j = 0; j < W::J; ++j) {
-      const int w = w0 + j * 256;
+      const int w = w0 + j * BLAS_BLOCK;
       if (w < nw) {
         rv[j] = W::axpy(-al, av[j], rv[j]);
         reinterpret_cast<V*>(r)[off + w] = rv[j];
@@ -316,7 +318,7 @@ __global__ void __launch_bounds__(256) k_bupdate(const BatchArgs a, S* e, S* r, 
 // p_l = r_l + beta_l p_l; last CTA of the grid: per lattice commit rr, count the iteration, inner convergence; end
 // of cycle when every lattice is frozen or the cycle is full.
 template <typename S>
-__global__ void __launch_bounds__(256) k_bpupdate(const BatchArgs a, const S* r, S* p, BatchState* st) {
+__global__ void __launch_bounds__(BLAS_BLOCK) k_bpupdate(const BatchArgs a, const S* r, S* p, BatchState* st) {
   if (st->cycle_done) return;
   using W = Word<S>;
   using V = typename W::V;
@@ -334,7 +336,7 @@ __global__ void __launch_bounds__(256) k_bpupdate(const BatchArgs a, const S* r,
     V rv[W::J], pv[W::J];
 #pragma unroll
     for (int j = 0; j < W::J; ++j) {
-      const int w = w0 + j * 256;
+      const int w = w0 + j * BLAS_BLOCK;
       if (w < nw) {
         rv[j] = reinterpret_cast<const V*>(r)[off + w];
         pv[j] = reinterpret_cast<const V*>(p)[off + w];
@@ -342,7 +344,7 @@ __global__ void __launch_bounds__(256) k_bpupdate(const BatchArgs a, const S* r,
     }
 #pragma unroll
     for (int j = 0; j < W::J; ++j) {
-      const int w = w0 + j * 256;
+      const int w = w0 + j * BLAS_BLOCK;
       if (w < nw) reinterpret_cast<V*>(p)[off + w] = W::axpy(beta, pv[j], rv[j]);
     }
   }
@@ -365,7 +367,7 @@ __global__ void __launch_bounds__(256) k_bpupdate(const BatchArgs a, const S* r,
 }
 
 // x_l += scale_l e_l; e_l = 0 (all lattices not yet verified).
-__global__ void __launch_bounds__(256) k_bfold(const BatchArgs a, double2* x, float* e, BatchState* st) {
+__global__ void __launch_bounds__(BLAS_BLOCK) k_bfold(const BatchArgs a, double2* x, float* e, BatchState* st) {
   __shared__ ActiveTiles act;
   list_active(act, a, st->conv);
   for (int t = blockIdx.x; t < act.tile0[act.n]; t += gridDim.x) {
@@ -374,7 +376,7 @@ __global__ void __launch_bounds__(256) k_bfold(const BatchArgs a, double2* x, fl
     const int n = a.geoms[l].half * 3;
     const size_t off = a.site_off[l] * 3;
     const double s = st->scale[l];
-    for (int i = local * BLAS_TILE * 3 + threadIdx.x; i < n && i < (local + 1) * BLAS_TILE * 3; i += 256) {
+    for (int i = local * BLAS_TILE * 3 + threadIdx.x; i < n && i < (local + 1) * BLAS_TILE * 3; i += BLAS_BLOCK) {
       float2* ep = reinterpret_cast<float2*>(e) + off + i;
       const float2 ev = *ep;
       double2 xv = x[off + i];
@@ -397,7 +399,7 @@ __global__ void k_bnonzero(const double2* __restrict__ x, size_t n, BatchState* 
 }
 
 // r_hi = b - Ax (FP64; Ax null: a zero guess, r_hi = b); rr_true and (init) bb per lattice.
-__global__ void __launch_bounds__(256) k_bresidual(const BatchArgs a, const double2* b, const double2* Ax, double2* rh,
+__global__ void __launch_bounds__(BLAS_BLOCK) k_bresidual(const BatchArgs a, const double2* b, const double2* Ax, double2* rh,
                                                    BatchState* st, double* partials, size_t pstride, int init) {
   __shared__ double red[32];
   __shared__ ActiveTiles act;
@@ -409,7 +411,7 @@ __global__ void __launch_bounds__(256) k_bresidual(const BatchArgs a, const doub
     const int kl = tile_lattice(act, t, &local), l = act.lat[kl];
     const int n = a.geoms[l].half * 3;
     const size_t off = a.site_off[l] * 3;
-    for (int i = local * BLAS_TILE * 3 + threadIdx.x; i < n && i < (local + 1) * BLAS_TILE * 3; i += 256) {
+    for (int i = local * BLAS_TILE * 3 + threadIdx.x; i < n && i < (local + 1) * BLAS_TILE * 3; i += BLAS_BLOCK) {
       const double2 bv = b[off + i], av = Ax ? Ax[off + i] : make_double2(0.0, 0.0);
       const double2 rv = make_double2(bv.x - av.x, bv.y - av.y);
       rh[off + i] = rv;
@@ -432,7 +434,7 @@ __global__ void __launch_bounds__(256) k_bresidual(const BatchArgs a, const doub
 // Reliable update per lattice not yet verified: r_lo = r_hi / s, p = r_lo, rr = rr_true / s^2; verified lattices
 // are frozen for good. Last CTA: the per-lattice bookkeeping; new cycle, or all verified.
 template <typename S>
-__global__ void __launch_bounds__(256) k_breliable(const BatchArgs a, const double2* rh, S* r, S* p, BatchState* st) {
+__global__ void __launch_bounds__(BLAS_BLOCK) k_breliable(const BatchArgs a, const double2* rh, S* r, S* p, BatchState* st) {
   __shared__ ActiveTiles act;
   __shared__ double s_inv;
   list_active(act, a, st->conv);
@@ -449,7 +451,7 @@ __global__ void __launch_bounds__(256) k_breliable(const BatchArgs a, const doub
     __syncthreads();
     const double inv = s_inv;
     if (inv == 0.0) continue;  // verified now: frozen (uniform over the block)
-    for (int i = local * BLAS_TILE * 3 + threadIdx.x; i < n && i < (local + 1) * BLAS_TILE * 3; i += 256) {
+    for (int i = local * BLAS_TILE * 3 + threadIdx.x; i < n && i < (local + 1) * BLAS_TILE * 3; i += BLAS_BLOCK) {
       const double2 w = rh[off + i];
       const S re = S(w.x * inv), im = S(w.y * inv);
       r[2 * (off + i)] = re;
@@ -592,8 +594,9 @@ static int bdslash(hisq_batch* B, int p, void* out, const void* in, const void* 
   } else if (cap != cudaStreamCaptureStatusNone) {
     block = 128;
   } else {
-    // autotune the tile size: time each candidate (the launch is idempotent)
-    static const int cands[] = {64, 128, 256};
+    // autotune the tile size: time each candidate (the launch is idempotent). 224 rather than 256: a 16^4 lattice's
+    // 32,768 sites are then 147 tiles for 152 SMs, and FP64 tiles are bound by their SM's FP64 pipe
+    static const int cands[] = {64, 128, 224};
     cudaEvent_t e0, e1;
     HISQ_CUDA(cudaEventCreate(&e0));
     HISQ_CUDA(cudaEventCreate(&e1));
@@ -638,7 +641,7 @@ static int blas_args(hisq_batch* B, const void* func, BatchArgs* a, int* grid) {
   int rc = tile_table(B, BLAS_TILE, &T);
   if (rc != HISQ_OK) return rc;
   *a = batch_args(B, HISQ_F64, BLAS_TILE, *T);
-  *grid = persistent_grid(B, func, 256);
+  *grid = persistent_grid(B, func, BLAS_BLOCK);
   if (*grid > T->ntiles) *grid = T->ntiles;
   return HISQ_OK;
 }
@@ -656,7 +659,7 @@ static int b_true_residual(hisq_batch* B, const BatchBufs& U, int init, bool zer
   BatchArgs a;
   int grid;
   if ((rc = blas_args(B, (const void*)k_bresidual, &a, &grid)) != HISQ_OK) return rc;
-  k_bresidual<<<grid, 256, 0, B->stream>>>(a, U.b, zero ? nullptr : U.Ax, U.rh, U.st, U.partials, U.pstride, init);
+  k_bresidual<<<grid, BLAS_BLOCK, 0, B->stream>>>(a, U.b, zero ? nullptr : U.Ax, U.rh, U.st, U.partials, U.pstride, init);
   HISQ_CUDA(cudaGetLastError());
   B->launches += 1;
   return HISQ_OK;
@@ -668,7 +671,7 @@ static int b_reliable(hisq_batch* B, const BatchBufs& U) {
   int grid;
   int rc = blas_args(B, (const void*)k_breliable<S>, &a, &grid);
   if (rc != HISQ_OK) return rc;
-  k_breliable<S><<<grid, 256, 0, B->stream>>>(a, U.rh, (S*)U.r, (S*)U.p, U.st);
+  k_breliable<S><<<grid, BLAS_BLOCK, 0, B->stream>>>(a, U.rh, (S*)U.r, (S*)U.p, U.st);
   HISQ_CUDA(cudaGetLastError());
   B->launches += 1;
   return HISQ_OK;
@@ -689,10 +692,10 @@ static int b_iteration(hisq_batch* B, const BatchBufs& U, int lp) {
   BatchArgs a;
   int grid;
   if ((rc = blas_args(B, (const void*)k_bupdate<S>, &a, &grid)) != HISQ_OK) return rc;
-  k_bupdate<S><<<grid, 256, 0, B->stream>>>(a, (S*)U.e, (S*)U.r, (const S*)U.p, (const S*)U.Ap, U.st,
+  k_bupdate<S><<<grid, BLAS_BLOCK, 0, B->stream>>>(a, (S*)U.e, (S*)U.r, (const S*)U.p, (const S*)U.Ap, U.st,
                                             U.partials + 2 * U.pstride);
   if ((rc = blas_args(B, (const void*)k_bpupdate<S>, &a, &grid)) != HISQ_OK) return rc;
-  k_bpupdate<S><<<grid, 256, 0, B->stream>>>(a, (const S*)U.r, (S*)U.p, U.st);
+  k_bpupdate<S><<<grid, BLAS_BLOCK, 0, B->stream>>>(a, (const S*)U.r, (S*)U.p, U.st);
   HISQ_CUDA(cudaGetLastError());
   return HISQ_OK;
 }
@@ -802,7 +805,7 @@ static int run_batch(hisq_batch* B, double2* x, const double2* b, const double* 
       BatchArgs a;
       int grid;
       if ((r2 = blas_args(B, (const void*)k_bfold, &a, &grid)) != HISQ_OK) return r2;
-      k_bfold<<<grid, 256, 0, B->stream>>>(a, U.x, (float*)U.e, U.st);
+      k_bfold<<<grid, BLAS_BLOCK, 0, B->stream>>>(a, U.x, (float*)U.e, U.st);
       HISQ_CUDA(cudaGetLastError());
       B->launches += 1;
     }
