@@ -174,7 +174,7 @@ __device__ __forceinline__ bool grid_last(unsigned* c) {
 // (EPI_AXPY), for every lattice l whose skip[l] is 0. FP32 takes 80 registers (three blocks of 256 per SM): at 64, like
 // the single-lattice form, the tile walk spills (16 lattices, all active: 174 and 196 us against 164 and 181 us).
 template <typename LR, typename SR, int EPI>
-__global__ void __launch_bounds__(256, sizeof(LR) == 4 ? 3 : 2) k_bdslash(const BatchArgs a, int p, void* out, const void* in,
+__global__ void __launch_bounds__(256, sizeof(LR) == 4 ? 3 : 0) k_bdslash(const BatchArgs a, int p, void* out, const void* in,
                                                                          const void* y, const int* skip, BatchState* st,
                                                                          double* partials, int red_row) {
   using A = typename Real<LR>::acc;
