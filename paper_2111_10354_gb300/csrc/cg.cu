@@ -1567,11 +1567,6 @@ static int run_multishift(hisq_ctx* ctx, double2* x, const double2* b, int ns, c
   const int lp = o.inner_prec;
   const int sp = sizeof(S) == 8 ? HISQ_F64 : HISQ_F32;
   const size_t n = (size_t)ctx->g.half * 3;
-  // the residuals of a group of iterations; where memory does not allow that many, shorter groups
-  int slots = ns > 1 ? MS_SLOTS : 1;
-  S* r = nullptr;
-  for (; slots >= 1 && !r; slots /= 2) r = (S*)workspace(ctx, "ms_r", slots * n * 2 * sizeof(S));
-  slots = slots >= 1 ? slots * 2 : 1;
   S* Ap = (S*)workspace(ctx, "ms_Ap", n * 2 * sizeof(S));
   S* t = (S*)workspace(ctx, "ms_t", n * 2 * sizeof(S));
   S* p = (S*)workspace(ctx, "ms_p", (size_t)ns * n * 2 * sizeof(S));
@@ -1580,6 +1575,17 @@ static int run_multishift(hisq_ctx* ctx, double2* x, const double2* b, int ns, c
   X* xacc = sizeof(S) == 8 ? (X*)x : (X*)workspace(ctx, "ms_e", (size_t)ns * n * 2 * sizeof(float));
   MsState* st = (MsState*)workspace(ctx, "ms_state", sizeof(MsState));
   double* partials = (double*)workspace(ctx, "ms_partials", 2 * MAXR * partial_stride(ctx) * sizeof(double));
+  // the residuals of a group of iterations, taken last; shorter groups where more would not leave the
+  // verification its room (at most 112 bytes an entry and shift)
+  int slots = ns > 1 ? MS_SLOTS : 1;
+  if (slots > 1 && ctx->ws["ms_r"].bytes < slots * n * 2 * sizeof(S)) {
+    size_t free_b = 0, total_b = 0;
+    HISQ_CUDA(cudaMemGetInfo(&free_b, &total_b));
+    while (slots > 1 && slots * n * 2 * sizeof(S) + (size_t)ns * n * 128 > free_b) slots /= 2;
+  }
+  S* r = nullptr;
+  for (; slots >= 1 && !r; slots /= 2) r = (S*)workspace(ctx, "ms_r", slots * n * 2 * sizeof(S));
+  slots = slots >= 1 ? slots * 2 : 1;
   if (!r || !Ap || !t || !p || !xacc || !st || !partials) return set_error(HISQ_ENOMEM, "multi-shift workspace");
   MsState* h = (MsState*)ctx->pinned;
   int base = 0;
