@@ -364,8 +364,8 @@ __device__ __forceinline__ void finish_iteration(SolverState* st, const double* 
 
 // One CG iteration's vector updates in one launch on the blocked layout [rhs][cb][color] (grid: x
 // chunks of a rhs, y = rhs; a cooperative launch of one wave):
-//   phase 1: r -= alpha Ap (alpha = rr / pAp), rr_new = |r|^2 (per-chunk terms in the arithmetic
-//            precision, FP64 over chunks);
+//   phase 1: r -= alpha Ap (alpha = rr / pAp), rr_new = |r|^2 (terms in the arithmetic precision,
+//            added error-free over a thread's chunks and the warp, then in FP64);
 //   barrier: one atomic per block; the last block to arrive releases the others at once, then every
 //            block sums its rhs's partials (same order everywhere) into rr_new and beta, and the last
 //            block also commits the iteration (counts, flags, Lanczos record);
