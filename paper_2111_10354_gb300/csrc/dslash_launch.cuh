@@ -138,6 +138,12 @@ static int launch_nr(hisq_ctx* ctx, const DslashKArgs& a, int nr) {
       std::vector<TuneVariant> v = {split_variant<LR, SR, 1, EPI, 2>(ctx, a, nr)};
       if (split_fits(ctx, 4 * nr)) v.push_back(split_variant<LR, SR, 1, EPI, 4>(ctx, a, nr));
       if (split_fits(ctx, 8 * nr)) v.push_back(split_variant<LR, SR, 1, EPI, 8>(ctx, a, nr));
+      // near the line the thread-per-site forms fill the FP64 pipe as well and read each link once for all the
+      // vectors (8x10x14x34: two vectors 38.0 us, 38.8 split, four 74.0 and 75.3; 8^4: two vectors 21.2 and 7.2)
+      auto add = [&v](const std::vector<TuneVariant>& g) { v.insert(v.end(), g.begin(), g.end()); };
+      if (nr == 2) add(group_forms<LR, SR, 2, EPI, COMP>(ctx, a));
+      if (nr == 3) add(group_forms<LR, SR, 3, EPI, COMP>(ctx, a));
+      if (nr == 4) add(group_forms<LR, SR, 4, EPI, COMP>(ctx, a));
       return launch_tuned(ctx, key, v);
     }
   }

@@ -311,7 +311,8 @@ def test_every_launch_form_matches_oracle(hisq, prec):
 # lattices with few sites; FP64 groups have keys of their own (a row of blocks per vector)
 def split_forms(prec):
     if prec in (0, 4):
-        return [(1, "nr1", (2, 3, 4))] + [(n, "ny%d" % n, (0, 1, 2)) for n in (2, 5, 8)]
+        return [(1, "nr1", (2, 3, 4)), (2, "ny2", (0, 1, 2, 3, 4)), (3, "ny3", (3,)), (4, "ny4", (3, 4, 5)),
+                (5, "ny5", (0, 1, 2)), (8, "ny8", (0, 1, 2))]
     return [(1, "nr1", (2, 3, 4)), (2, "nr2", (2,)), (3, "nr3", (1,)), (4, "nr4", (3,)), (5, "nr5", (2,)),
             (6, "nr6", (2,)), (7, "nr7", (2,)), (8, "nr8", (8,))]
 
@@ -319,9 +320,9 @@ def split_forms(prec):
 @pytest.mark.parametrize("L,block", [((4, 4, 4, 4), 64), ((4, 6, 8, 10), 160), ((6, 6, 10, 14), 256)])
 @pytest.mark.parametrize("prec", [0, 1, 2, 3, 4])
 def test_split_launch_forms_match_oracle(hisq, prec, L, block):
-    """Every launch form that shares a site's hops between threads, forced through loaded tune entries: the
-    Dslash to both parities and A, against the oracle, on the smallest lattice (fewer sites than threads), on
-    one whose hops alias, and on one with a ragged last block."""
+    """Every launch form that shares a site's hops between threads, and the thread-per-site forms FP64 tunes beside
+    them, forced through loaded tune entries: the Dslash to both parities and A, against the oracle, on the smallest
+    lattice (fewer sites than threads), on one whose hops alias, and on one with a ragged last block."""
     lat, ff, lf = setup(hisq, L)
     sp = 0 if prec == 4 else prec
     dims = "%dx%dx%dx%d" % L
@@ -329,9 +330,10 @@ def test_split_launch_forms_match_oracle(hisq, prec, L, block):
         src = hin.gen_source(7100 + nr, lat.half, nr)
         x = to_device(src, prec)
         for vi in variants:
+            blk = 64 if name[:2] == "ny" and vi > 2 else block  # thread-per-site forms: fewer threads may fit a block
             for epi in (0, 1):
                 key = "dslash/l%d/s%d/%s/e%d%s" % (prec, sp, name, epi, "/c0" if name[:2] == "nr" else "")
-                assert hisq.hisq_tune_load(lat.ctx, "%s %s -> %d\n" % (key, dims, vi * 10000 + block)) == 1
+                assert hisq.hisq_tune_load(lat.ctx, "%s %s -> %d\n" % (key, dims, vi * 10000 + blk)) == 1
             y = empty_like_prec((nr, lat.half, 3), prec)
             for parity in (0, 1):
                 lat.dslash(parity, y, x, prec, nr)
@@ -342,7 +344,7 @@ def test_split_launch_forms_match_oracle(hisq, prec, L, block):
             got = from_device(y, prec)
             for r in range(nr):
                 assert rel_err(got[r], oracle.apply_A(L, ff, lf, 0.05, src[r])) <= 2 * TOL[prec], (nr, vi, r)
-            assert "%s %s -> %d" % (key, dims, vi * 10000 + block) in hisq.hisq_tune_report(lat.ctx)
+            assert "%s %s -> %d" % (key, dims, vi * 10000 + blk) in hisq.hisq_tune_report(lat.ctx)
 
 
 @pytest.mark.parametrize("prec", [0, 1, 2, 3, 4])
