@@ -467,6 +467,14 @@ int hisq_set_pdl(hisq_ctx* ctx, int enable);
  */
 int hisq_selftest_bounded_wait(hisq_ctx* ctx);
 
+/*
+ * Self-test of the solvers' sums: the sum of n FP32 terms (device) as the fused CG update forms its residual norm --
+ * running sums per thread and block, a grid barrier, every block adding the blocks' shares -- `repeats` times over in
+ * one launch. *total (host): the sum. Errors: HISQ_EINVAL, HISQ_ENOMEM, HISQ_ETIMEOUT (a barrier wait ran out),
+ * HISQ_ECUDA (two blocks or two repetitions differ). The paper has no counterpart.
+ */
+int hisq_selftest_sum(hisq_ctx* ctx, const float* terms, long long n, int repeats, double* total);
+
 #ifdef __cplusplus
 }
 #endif

@@ -118,6 +118,7 @@ def _load():
     lib.hisq_tune_report.argtypes = [vp, ctypes.c_char_p, ctypes.c_size_t]
     lib.hisq_tune_load.argtypes = [vp, ctypes.c_char_p, ctypes.POINTER(ctypes.c_int)]
     lib.hisq_selftest_bounded_wait.argtypes = [vp]
+    lib.hisq_selftest_sum.argtypes = [vp, vp, ctypes.c_longlong, ip, ctypes.POINTER(dp)]
     lib.hisq_release_workspaces.argtypes = [vp]
     cp = ctypes.POINTER(hisq_smear_coeffs)
     lib.hisq_smear.argtypes = [vp, vp, vp, vp, cp, ip]
@@ -382,6 +383,13 @@ def hisq_release_workspaces(ctx):
 def hisq_selftest_bounded_wait(ctx) -> int:
     """Status of the bounded-wait self-test (HISQ_ETIMEOUT when the wait gave up as intended)."""
     return _load().hisq_selftest_bounded_wait(ctx)
+
+
+def hisq_selftest_sum(ctx, terms, repeats: int = 1) -> float:
+    """Sum of a device FP32 tensor as the fused CG update forms its residual norm, `repeats` times in one launch."""
+    total = ctypes.c_double()
+    _check(_load().hisq_selftest_sum(ctx, _ptr(terms), terms.numel(), repeats, ctypes.byref(total)), "hisq_selftest_sum")
+    return total.value
 
 
 def hisq_batch_create(dims_list, prec_mask: int = HISQ_PREC_BIT(HISQ_F64) | HISQ_PREC_BIT(HISQ_F32), stream=None):

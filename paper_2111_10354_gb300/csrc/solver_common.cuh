@@ -183,8 +183,9 @@ __device__ __forceinline__ void grid_arrive_release(unsigned* bar, unsigned* gen
   *last = s_last != 0;
 }
 
-// Wait (bounded) by one full warp until the generation in the high half has advanced past gen (acquire: every
-// block's partials are then visible): lane 0 polls, every lane gets the answer. False on timeout.
+// Wait (bounded) by one full warp until the generation in the high half has advanced past gen: lane 0 polls with
+// acquire loads, and the warp barrier after its last poll orders every lane's later reads after it (a shuffle alone
+// orders no memory), so every lane may read every block's partials. Every lane gets the answer. False on timeout.
 __device__ __forceinline__ bool grid_wait64_warp(const unsigned* bar, unsigned gen, long limit = GRID_WAIT_POLLS) {
   const unsigned long long* w = reinterpret_cast<const unsigned long long*>(bar);
   int ok = 0;
@@ -197,7 +198,8 @@ __device__ __forceinline__ bool grid_wait64_warp(const unsigned* bar, unsigned g
       __nanosleep(32);
     }
   }
-  return __shfl_sync(0xffffffffu, ok, 0) != 0;  // also orders the warp after lane 0's acquire
+  __syncwarp();
+  return __shfl_sync(0xffffffffu, ok, 0) != 0;
 }
 
 template <typename S>

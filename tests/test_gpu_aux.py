@@ -1,5 +1,7 @@
 """Auxiliary subsystems on the GPU: the failure path of the bounded device waits (made to run out on
 purpose, without a fault or a hang) and the persistence of the autotuner's cache."""
+import math
+
 import numpy as np
 import pytest
 
@@ -23,6 +25,18 @@ def test_bounded_wait_gives_up_and_context_survives(hisq):
     y = torch.empty((1, lat.half, 3), dtype=torch.complex128, device="cuda")
     lat.dslash(0, y, torch.from_numpy(src).cuda(), 0)
     assert rel_err(y.cpu().numpy()[0], oracle.dslash(L, ff, lf, 0, src[0])) <= 1e-12
+
+
+@pytest.mark.parametrize("n", [1, 152 * 256 - 1, 10 ** 6 + 3])
+def test_grid_sum_is_the_same_in_every_block_and_repetition(hisq, n):
+    """The fused CG update's sum over the grid, 300 times in one launch: every block reads the shares of the others
+    behind the barrier, and none may see a share of an earlier repetition. n positive FP32 terms: a thread's pair of
+    FP32 sums and the FP64 tree over them round far below 1e-13 of the total."""
+    import torch
+    lat = hisq.Lattice((4, 4, 4, 4), precs=(0,))
+    terms = np.random.default_rng(n).random(n, dtype=np.float32)
+    got = hisq.hisq_selftest_sum(lat.ctx, torch.from_numpy(terms).cuda(), repeats=300)
+    assert abs(got - math.fsum(terms.tolist())) <= 1e-13 * math.fsum(terms.tolist())
 
 
 def test_tune_cache_report_and_load(hisq):
