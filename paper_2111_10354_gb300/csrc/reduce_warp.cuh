@@ -8,7 +8,9 @@ namespace hisq {
 // A thread's running sum of terms in the arithmetic precision, kept to FP64 accuracy without FP64 instructions
 // where the terms are FP32: GB300's FP64 pipe takes a warp's operation in 16 cycles and is shared by the whole SM,
 // so a conversion and an add per term, five more per warp and a division per thread cost a streaming kernel
-// microseconds. FP32 terms go into an error-free pair (hi + lo, Knuth's two-sum: about 48 bits).
+// microseconds. FP32 terms go into an error-free pair (hi + lo, Knuth's two-sum: about 48 bits). The pair's range is
+// FP32's, so a thread's own terms (one to some tens) have to add up to less than 3.4e38; sums over the warp and
+// beyond are not bound by it.
 template <typename T>
 struct SumAcc;
 template <>
@@ -39,8 +41,15 @@ struct SumAcc<float> {
       a.add(h);
       a.lo = __fadd_rn(a.lo, l);
     }
-    // a sum beyond FP32's range (or a non-finite term) leaves hi non-finite and lo NaN: hi alone then says which
-    return isfinite(a.hi) ? (double)a.hi + (double)a.lo : (double)a.hi;
+    // Beyond FP32's range (or with a non-finite term) the pair has lost the sum, though each lane's own may be
+    // finite: once more in FP64. hi is the same in every lane, so the whole warp takes the branch.
+    if (!isfinite(a.hi)) {
+      double s = isfinite(hi) ? (double)hi + (double)lo : (double)hi;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+      return s;
+    }
+    return (double)a.hi + (double)a.lo;
   }
 };
 

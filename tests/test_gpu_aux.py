@@ -39,6 +39,31 @@ def test_grid_sum_is_the_same_in_every_block_and_repetition(hisq, n):
     assert abs(got - math.fsum(terms.tolist())) <= 1e-13 * math.fsum(terms.tolist())
 
 
+def test_grid_sum_range_cancellation_and_nonfinite_terms(hisq):
+    """The FP32-pair sums at their edges: a total beyond FP32's range, terms that cancel to a 1e-9 of their size,
+    subnormal terms, and non-finite ones. A pair keeps some 48 bits: 2^-46 of the sum of the terms' sizes."""
+    import torch
+    lat = hisq.Lattice((4, 4, 4, 4), precs=(0,))
+    r = np.random.default_rng(5)
+
+    def total(t):
+        return hisq.hisq_selftest_sum(lat.ctx, torch.from_numpy(t).cuda())
+
+    big = (3e37 * (1 + r.random(150000))).astype(np.float32)  # 4 or fewer terms a thread, 100 times FP32's range a warp
+    pair = (1e6 * r.random(100000)).astype(np.float32)
+    cancel = np.concatenate([pair, [np.float32(1.25e-3)], -pair[::-1]])
+    tiny = np.full(100003, 3e-45, np.float32)
+    for t in (big, -big, cancel, tiny):
+        exact = math.fsum(t.tolist())
+        assert abs(total(t) - exact) <= 2.0 ** -46 * math.fsum(abs(t).tolist())
+    for bad in (np.inf, -np.inf, np.nan):
+        t = pair.copy()
+        t[77777] = bad
+        assert total(t) == bad or (np.isnan(bad) and np.isnan(total(t)))
+    t[3] = np.inf
+    assert np.isnan(total(np.concatenate([t, [np.float32(-np.inf)]])))
+
+
 def test_tune_cache_report_and_load(hisq):
     import torch
     L = (8, 10, 12, 14)

@@ -269,3 +269,19 @@ def test_cg_16bit_spinor_storage_errors(hisq):
     with pytest.raises(hisq.HisqError) as e:
         lat.multishift_cg(xs, b[:1], [0.0, 0.1], 0.1, [1e-9, 1e-9], 100, inner_prec=2, spinor_prec=2)
     assert e.value.code == hisq.HISQ_EINVAL
+
+
+@pytest.mark.parametrize("inner,nrhs", [(1, 1), (1, 2), (2, 3)])
+def test_cg_with_a_mass_whose_products_leave_fp32s_range(hisq, inner, nrhs):
+    """A mass of 1.5e18: every site's term of <p, A p> is a finite FP32 number, a warp's sum of them is not. A is
+    4 m^2 to 1e-35, so x = b / (4 m^2)."""
+    import torch
+    L, mass = (8, 8, 8, 8), 1.5e18
+    fat, lng = hin.gen_links(L, 1234, 0.3, 0.1)
+    lat = hisq.Lattice(L, precs=(0, inner)).load(fat, lng)
+    hisq.hisq_set_autotune(lat.ctx, False)  # one thread per site: 32 sites' terms in a warp
+    b = hin.gen_source(99, lat.half, nrhs)
+    x = torch.zeros((nrhs, lat.half, 3), dtype=torch.complex128, device="cuda")
+    rc, st = lat.cg(x, torch.from_numpy(b).cuda(), mass, 1e-10, 200, nrhs=nrhs, inner_prec=inner)
+    assert rc == 0 and st["converged"] == 1
+    assert np.linalg.norm(4 * mass * mass * x.cpu().numpy() - b) <= 1e-10 * np.linalg.norm(b)
