@@ -283,8 +283,9 @@ __device__ __forceinline__ void ptc_tile_put(float2* field, const cplx<float> (&
 }
 
 // Pass 1 of training, odd sites: phi_h = sum_h' C[h][h'] T_h' b for NV vectors, FP32 planes
-// [vector][h][colour][cb] (training's inputs may have any scale, so no FP16 here). The next tile's link and
-// vectors are loaded while this tile is mixed.
+// [vector][h][colour][cb] (no FP16 here: training takes inputs of any scale whose squares and products, summed over a
+// block's sites in FP32, are FP32 numbers: 1e-18 to 1e16 up to 144^3x36). The next tile's link and vectors are loaded
+// while this tile is mixed.
 template <int NV>
 __global__ void __launch_bounds__(256, 2) k_ptc_train_odd(const PtcGeom G, const float2* __restrict__ b,
                                                           float2* __restrict__ phi, const float2* __restrict__ mix) {
@@ -346,7 +347,8 @@ __global__ void __launch_bounds__(256, 2) k_ptc_train_odd(const PtcGeom G, const
 }
 
 // Pass 2 of training, even sites: d = N(b) - x for NV vectors, planes [vector][colour][cb], and this block's
-// sums of |d|^2, |x|^2 and conj(b) d (FP32 over a thread's few sites, FP64 over the block).
+// sums of |d|^2, |x|^2 and conj(b) d: FP32 terms, summed over a thread's sites (14 at 32^3x8, growing with the lattice)
+// and its warp to FP64 accuracy (SumAcc; plain FP32 sums were off by 6e-7 at 32^3x24), FP64 over the block.
 template <int NV>
 __global__ void __launch_bounds__(256, 2) k_ptc_train_even(const PtcGeom G, const float2* __restrict__ b,
                                                            const float2* __restrict__ phi, const float2* __restrict__ x,
@@ -361,7 +363,7 @@ __global__ void __launch_bounds__(256, 2) k_ptc_train_even(const PtcGeom G, cons
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const float2 m0 = __ldg(mix);
   constexpr int ITEMS = (NV * 3 + 7) / 8;  // (vector, colour) pairs per warp
-  float s[ITEMS][PT_PART] = {};
+  SumAcc<float> s[ITEMS][PT_PART];
   const int ntiles = (g.half + PT_SITES - 1) / PT_SITES;
   cplx<float> U[9], v[NV][3];
   auto load = [&](int cb) {
@@ -400,10 +402,10 @@ __global__ void __launch_bounds__(256, 2) k_ptc_train_even(const PtcGeom G, cons
         }
         const float dx = z.re - xv.x, dy = z.im - xv.y;
         d[((size_t)f * 3 + col) * half + cb] = make_float2(dx, dy);
-        s[j][0] += dx * dx + dy * dy;
-        s[j][1] += xv.x * xv.x + xv.y * xv.y;
-        s[j][2] += bv.x * dx + bv.y * dy;
-        s[j][3] += bv.x * dy - bv.y * dx;
+        s[j][0].add(dx * dx + dy * dy);
+        s[j][1].add(xv.x * xv.x + xv.y * xv.y);
+        s[j][2].add(bv.x * dx + bv.y * dy);
+        s[j][3].add(bv.x * dy - bv.y * dx);
       }
     }
     __syncthreads();
@@ -412,9 +414,7 @@ __global__ void __launch_bounds__(256, 2) k_ptc_train_even(const PtcGeom G, cons
   for (int j = 0; j < ITEMS; ++j)
 #pragma unroll
     for (int p = 0; p < PT_PART; ++p) {
-      double w = (double)s[j][p];
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(0xffffffffu, w, o);
+      const double w = s[j][p].warp_total();
       if (lane == 0 && warp + 8 * j < NV * 3) red[warp + 8 * j][p] = w;
     }
   __syncthreads();
@@ -424,7 +424,8 @@ __global__ void __launch_bounds__(256, 2) k_ptc_train_even(const PtcGeom G, cons
   }
 }
 
-// This block's part of M for NV pairs: part[pair][block][h' * 8 + k] (FP32 sums over the block's tiles). After
+// This block's part of M for NV pairs: part[pair][block][h' * 8 + k] (FP32 sums over the block's tiles, as in the
+// accumulators of a matrix instruction; FP64 over the blocks). After
 // the transports of b and d at a tile's odd sites each thread adds its share of the sites to a 4 x 4 corner of
 // the 8 x 8 inner products, which stay in registers over the tiles of a persistent grid.
 template <int NV>

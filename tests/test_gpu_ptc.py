@@ -262,3 +262,57 @@ def test_ptc_gradient_groups_and_tiles(hisq, dims, npairs):
                                      list(x.astype(np.complex128)))
     assert abs(loss - rl) <= 1e-5 * rl
     assert rel(g1, r1) <= 1e-5 and rel(g2, r2) <= 1e-5, (rel(g1, r1), rel(g2, r2))
+
+
+def test_ptc_loss_sums_over_many_tiles_per_block(hisq):
+    """|d|^2 and |x|^2 over the 40 or 41 tiles a block has at 32^3x24, every term exact in FP32: the identity network
+    and b = x + 1, x = 3497/2048 everywhere, so that the loss is 1 / x^2. Rounded once, to FP32: 2^-24, with a factor
+    of two. Plain FP32 running sums are off by 5.7e-7."""
+    import torch
+    L, xi = (32, 32, 32, 24), 3497 / 2048
+    lat = hisq.Lattice(L, precs=(0, 1))
+    links = torch.zeros((int(np.prod(L)), 4, 3, 3), dtype=torch.complex128, device="cuda")
+    lat.load(links, links)
+    net = hisq.Ptc(lat)
+    w1, w2 = np.zeros((8, 1, 9), np.complex64), np.zeros((1, 8, 9), np.complex64)
+    w1[0, 0, 0] = w2[0, 0, 0] = 1
+    net.set_weights(w1, w2)
+    for npairs in (1, 2, 4):
+        x = torch.full((npairs, lat.half, 3), xi, dtype=torch.complex64, device="cuda")
+        loss, g1, g2 = net.train_step(x + 1, x, npairs, 0.0)
+        assert abs(loss * xi * xi - 1) <= 2.0 ** -23, npairs
+        # dL/dconj W[0][0] = sum conj(b) d / |x|^2, the same for both layers
+        for g in (g1[0, 0, 0], g2[0, 0, 0]):
+            assert abs(g * xi * xi / (xi + 1) - 1) <= 2.0 ** -23, npairs
+
+
+@pytest.mark.parametrize("scale", [1e-18, 1e-6, 1e16])
+def test_ptc_gradients_over_many_tiles_and_scales(hisq, scale):
+    """Gradients over 28 tiles per block, at the ends of the inputs' range: against the same step with the inputs at
+    unit scale (the loss and gradients do not depend on a common factor of b and x), and loss and gradients together
+    by the network's linearity: with d = N(b) - x and N linear in each layer, Re <W1, G1> = Re <W2, G2> =
+    Re <N(b), d> / |x|^2, formed here in FP64. FP32 terms round by a few 2^-24 and a thread's FP32 sums have some 170
+    terms; 1e-5 as for the small lattices."""
+    import torch
+    L = (32, 32, 32, 16)
+    torch.manual_seed(3)
+    U = 0.6 * torch.randn(int(np.prod(L)), 4, 3, 3, dtype=torch.complex128, device="cuda")  # any matrices will do
+    lat = hisq.Lattice(L, precs=(0, 1)).load(U, U)
+    net = hisq.Ptc(lat)
+    W = [torch.view_as_complex(torch.view_as_real(torch.from_numpy(w.astype(np.complex64))).to(torch.bfloat16).float())
+         .numpy() for w in optc.init_weights(81)]
+    net.set_weights(*W)
+    b = torch.randn(4, lat.half, 3, dtype=torch.complex64, device="cuda")
+    x = torch.randn(4, lat.half, 3, dtype=torch.complex64, device="cuda")
+    loss1, a1, a2 = net.train_step(b, x, 4, 0.0)
+    z = torch.empty_like(b)
+    net.apply(z, b, 4)
+    z, t = z.to(torch.complex128), x.to(torch.complex128)
+    nx = t.abs().square().sum((1, 2))
+    zd = float(((z.conj() * (z - t)).real.sum((1, 2)) / nx).mean())
+    for w, g in zip(W, (a1, a2)):
+        # the apply rounds its activation to FP16: 2^-11 per entry, averaged over the sites
+        assert abs(float((w.conj() * g).real.sum()) - zd) <= 1e-4 * abs(zd)
+    loss, g1, g2 = net.train_step(b * scale, x * scale, 4, 0.0)
+    assert abs(loss - loss1) <= 1e-5 * loss1
+    assert rel(g1, a1) <= 1e-5 and rel(g2, a2) <= 1e-5
