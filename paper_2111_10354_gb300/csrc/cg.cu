@@ -1334,13 +1334,49 @@ __global__ void k_ms_rupdate(const S* r, S* r_out, const S* __restrict__ Ap, siz
   }
 }
 
+// Commits an iteration (one whole block): the recurrences, shifts that have converged, the counts and flags. npend:
+// slots whose updates the other shifts have still to take.
+__device__ __forceinline__ void ms_commit(MsState* st, int slot, int npend) {
+  const int b0 = st->base;
+  const int ns = st->nshift;
+  const double rr_new = st->rr_new, scale = st->scale, res2 = rr_new * scale * scale;
+  const int iter = st->iter + 1;
+  bool other = false;
+  for (int k = threadIdx.x; k < ns; k += blockDim.x) {
+    if (!st->active[k]) continue;
+    const double zn = st->zeta_new[slot][k];
+    st->zeta_old[k] = st->zeta[k];
+    st->zeta[k] = zn;
+    if (k == b0) continue;
+    if (zn * zn * res2 <= st->tol2[k]) {
+      st->active[k] = 0;
+      st->conv_iter[k] = iter;
+    } else {
+      other = true;
+    }
+  }
+  other = __syncthreads_or(other);
+  if (threadIdx.x != 0) return;
+  st->iter = iter;
+  st->cycle_iter += 1;
+  st->alpha_old = st->alpha;
+  st->beta_old = rr_new / st->rr;
+  st->rr = rr_new;
+  st->npend = npend;
+  if (st->active[b0] && !other && res2 <= st->tol2[b0]) {
+    st->active[b0] = 0;
+    st->conv_iter[b0] = iter;
+  }
+  if (!st->active[b0] || st->cycle_iter >= st->cycle_limit || st->breakdown || st->nonfinite) st->done = 1;
+}
+
 // The base system's update of this iteration: x += alpha p; p = r + beta p (x, p: the base shift's vectors).
 // X = double: x_k is the FP64 solution in true units (alpha_k * scale). X = float (FP32 Krylov
 // vectors): x_k is an FP32 correction in inner units, folded into the FP64 solutions once the
 // Krylov phase ends (k_ms_fold) -- two FP64 operations per entry and shift would otherwise bind the
 // streaming kernels to GB300's FP64 pipe. The FP64 verification and refinement that follow the FP32
 // Krylov phase correct what the FP32 accumulation loses.
-// Last block: commit the recurrences, freeze converged shifts, count the iteration.
+// Last block: ms_commit.
 template <typename S, typename X>
 __global__ void __launch_bounds__(256) k_ms_base(X* __restrict__ x, S* __restrict__ p, const S* __restrict__ r, size_t n,
                                                  MsState* st, int slot, unsigned* counter) {
@@ -1370,37 +1406,7 @@ __global__ void __launch_bounds__(256) k_ms_base(X* __restrict__ x, S* __restric
       Chunk<S>::store(p, i / K, pv);
     }
   }
-  if (!last_block_done(counter)) return;
-  const int ns = st->nshift;
-  const double rr_new = st->rr_new, scale = st->scale, res2 = rr_new * scale * scale;
-  const int iter = st->iter + 1;
-  bool other = false;
-  for (int k = threadIdx.x; k < ns; k += blockDim.x) {
-    if (!st->active[k]) continue;
-    const double zn = st->zeta_new[slot][k];
-    st->zeta_old[k] = st->zeta[k];
-    st->zeta[k] = zn;
-    if (k == b0) continue;
-    if (zn * zn * res2 <= st->tol2[k]) {
-      st->active[k] = 0;
-      st->conv_iter[k] = iter;
-    } else {
-      other = true;
-    }
-  }
-  other = __syncthreads_or(other);
-  if (threadIdx.x != 0) return;
-  st->iter = iter;
-  st->cycle_iter += 1;
-  st->alpha_old = st->alpha;
-  st->beta_old = rr_new / st->rr;
-  st->rr = rr_new;
-  st->npend = slot + 1;
-  if (st->active[b0] && !other && res2 <= st->tol2[b0]) {
-    st->active[b0] = 0;
-    st->conv_iter[b0] = iter;
-  }
-  if (!st->active[b0] || st->cycle_iter >= st->cycle_limit || st->breakdown || st->nonfinite) st->done = 1;
+  if (last_block_done(counter)) ms_commit(st, slot, slot + 1);
 }
 
 // The residuals of a group's iterations, by slot.
@@ -1411,20 +1417,25 @@ struct MsResiduals {
 
 // The pending updates of every shift but the base, slot by slot: x_k += alpha_k p_k; p_k = zeta_k' r + beta_k p_k.
 // Runs at the end of a group of iterations, also when the cycle is over (done) with some of its slots filled.
-template <typename S, typename X>
-__global__ void __launch_bounds__(256, 3) k_ms_update(X* __restrict__ x, S* __restrict__ p, const MsResiduals<S> rs,
+// ONE: a group of one iteration, which includes the base shift and commits the iteration: one shift, a poll interval
+// of 1, or the last iteration of 8 k + 1. k_ms_base and this kernel one after the other read r twice (one shift: 46.9 ms
+// a solve at 48^3x12 against 46.4, 7.29 at 16^4 against 6.80; four shifts polled every iteration at 48^3x12: 66.1
+// against 64.9).
+template <typename S, typename X, bool ONE>
+__global__ void __launch_bounds__(256, ONE ? 4 : 3) k_ms_update(X* __restrict__ x, S* __restrict__ p, const MsResiduals<S> rs,
                                                       size_t n, MsState* st, unsigned* counter) {
-  const int np = st->npend;
-  if (np == 0) return;  // uniform: the last block resets it
+  const int np = ONE ? !st->done : st->npend;
+  if (np == 0) return;  // uniform: only the last block changes done and npend
   using T = typename Real<S>::acc;
   using XT = typename Real<X>::acc;
   constexpr int K = Chunk<S>::K;
-  __shared__ XT s_ax[MAXR][MS_SLOTS];
-  __shared__ T s_z[MAXR][MS_SLOTS], s_b[MAXR][MS_SLOTS];
+  constexpr int Q = ONE ? 1 : MS_SLOTS;
+  __shared__ XT s_ax[MAXR][Q];
+  __shared__ T s_z[MAXR][Q], s_b[MAXR][Q];
   __shared__ int s_np[MAXR];  // slots of shift k to apply: a shift is active in the first so many (0: none)
   const int ns = st->nshift, b0 = st->base;
-  for (int i = threadIdx.x; i < ns * MS_SLOTS; i += blockDim.x) {
-    const int k = i / MS_SLOTS, q = i % MS_SLOTS;
+  for (int i = threadIdx.x; i < ns * Q; i += blockDim.x) {
+    const int k = i / Q, q = i % Q;
     if (q >= np) continue;
     s_ax[k][q] = XT(sizeof(X) == 8 ? st->alpha_k[q][k] * st->scale : st->alpha_k[q][k]);
     s_z[k][q] = T(st->zeta_new[q][k]);
@@ -1432,14 +1443,14 @@ __global__ void __launch_bounds__(256, 3) k_ms_update(X* __restrict__ x, S* __re
   }
   for (int k = threadIdx.x; k < ns; k += blockDim.x) {
     int c = 0;
-    while (k != b0 && c < np && st->act[c][k]) ++c;
+    while ((ONE || k != b0) && c < np && st->act[c][k]) ++c;
     s_np[k] = c;
   }
   __syncthreads();
   for (size_t i = (blockIdx.x * (size_t)blockDim.x + threadIdx.x) * K; i < n; i += (size_t)gridDim.x * blockDim.x * K) {
-    cplx<T> rv[MS_SLOTS][K];
+    cplx<T> rv[Q][K];
 #pragma unroll
-    for (int q = 0; q < MS_SLOTS; ++q)
+    for (int q = 0; q < Q; ++q)
       if (q < np) Chunk<S>::load(rs.r[q], i / K, rv[q]);
     for (int k = 0; k < ns; ++k) {
       const int c = s_np[k];
@@ -1450,7 +1461,7 @@ __global__ void __launch_bounds__(256, 3) k_ms_update(X* __restrict__ x, S* __re
       Chunk<S>::load(p, j / K, pv);
       load_k<X, K>(x, j, xv);
 #pragma unroll
-      for (int q = 0; q < MS_SLOTS; ++q) {
+      for (int q = 0; q < Q; ++q) {
         if (q >= c) break;
 #pragma unroll
         for (int e = 0; e < K; ++e) {
@@ -1464,7 +1475,9 @@ __global__ void __launch_bounds__(256, 3) k_ms_update(X* __restrict__ x, S* __re
       Chunk<S>::store(p, j / K, pv);
     }
   }
-  if (last_block_done(counter) && threadIdx.x == 0) st->npend = 0;
+  if (!last_block_done(counter)) return;
+  if (ONE) ms_commit(st, 0, 0);
+  else if (threadIdx.x == 0) st->npend = 0;
 }
 
 // r = b / scale; p_k = r; x_k = 0 (x: the FP64 solutions or the FP32 corrections, see k_ms_update).
@@ -1516,7 +1529,7 @@ __global__ void k_norm2(const double2* __restrict__ b, size_t n, double* partial
 // group's last iteration applies the other shifts' pending updates.
 template <typename S>
 static int ms_iteration(hisq_ctx* ctx, int lp, void* xacc, S* r, S* p, S* Ap, S* t, MsState* st, double* partials,
-                        double a_base, int base, int ns, int slot, int len) {
+                        double a_base, int base, int slot, int len) {
   const int sp = sizeof(S) == 8 ? HISQ_F64 : HISQ_F32;
   const size_t n = (size_t)ctx->g.half * 3;
   S* pb = p + (size_t)base * n * 2;
@@ -1544,19 +1557,24 @@ static int ms_iteration(hisq_ctx* ctx, int lp, void* xacc, S* r, S* p, S* Ap, S*
   auto buffer = [&](int q) { return r + (size_t)q * n * 2; };
   S* r_out = slot + 1 < len ? buffer(slot + 1) : r;
   k_ms_rupdate<S><<<grid, 256, 0, ctx->stream>>>(buffer(slot), r_out, Ap, n, st, slot, partials, ctx->d_counters + 7);
+  note_launch(ctx);
   using X = typename std::conditional<sizeof(S) == 8, double, float>::type;  // see k_ms_base
-  k_ms_base<S, X><<<grid, 256, 0, ctx->stream>>>((X*)xacc + (size_t)base * n * 2, pb, r_out, n, st, slot,
-                                                 ctx->d_counters + 8);
-  note_launch(ctx, 2);
-  if (slot + 1 == len) {
-    MsResiduals<S> rs;
-    for (int q = 0; q < MS_SLOTS; ++q) rs.r[q] = q + 1 < len ? buffer(q + 1) : r;
-    k_ms_update<S, X><<<blas_grid(ctx, 1, n / Chunk<S>::K, 3).x, 256, 0, ctx->stream>>>((X*)xacc, p, rs, n, st,
-                                                                                       ctx->d_counters + 11);
+  MsResiduals<S> rs;
+  for (int q = 0; q < MS_SLOTS; ++q) rs.r[q] = q + 1 < len ? buffer(q + 1) : r;
+  if (len == 1) {
+    k_ms_update<S, X, true><<<grid, 256, 0, ctx->stream>>>((X*)xacc, p, rs, n, st, ctx->d_counters + 11);
     note_launch(ctx);
+  } else {
+    k_ms_base<S, X><<<grid, 256, 0, ctx->stream>>>((X*)xacc + (size_t)base * n * 2, pb, r_out, n, st, slot,
+                                                   ctx->d_counters + 8);
+    note_launch(ctx);
+    if (slot + 1 == len) {
+      k_ms_update<S, X, false><<<blas_grid(ctx, 1, n / Chunk<S>::K, 3).x, 256, 0, ctx->stream>>>((X*)xacc, p, rs, n, st,
+                                                                                                ctx->d_counters + 11);
+      note_launch(ctx);
+    }
   }
   HISQ_CUDA(cudaGetLastError());
-  (void)ns;
   return HISQ_OK;
 }
 
@@ -1630,7 +1648,7 @@ static int run_multishift(hisq_ctx* ctx, double2* x, const double2* b, int ns, c
   auto run_iterations = [&]() -> int {  // a cycle, in groups of at most `slots` iterations
     for (int i = 0; i < cycle; ++i) {
       const int g0 = i / slots * slots, len = cycle - g0 < slots ? cycle - g0 : slots;
-      int rc = ms_iteration<S>(ctx, lp, xacc, r, p, Ap, t, st, partials, a_base, base, ns, i - g0, len);
+      int rc = ms_iteration<S>(ctx, lp, xacc, r, p, Ap, t, st, partials, a_base, base, i - g0, len);
       if (rc != HISQ_OK) return rc;
     }
     return HISQ_OK;

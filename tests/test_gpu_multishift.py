@@ -124,3 +124,24 @@ def test_multishift_group_lengths_bitwise(hisq, inner):
     assert min(its[0]) < max(its[0])
     for o in outs[1:]:
         assert torch.equal(o, outs[0])
+
+
+@pytest.mark.parametrize("inner", [0, 1])
+@pytest.mark.parametrize("nshift,poll", [(1, 1), (1, 10), (4, 1)])
+def test_multishift_launches_per_iteration_without_groups(hisq, inner, nshift, poll):
+    """One shift, or a poll after every iteration: nothing is deferred, and an iteration is four launches (two Dslash,
+    the residual, all shifts' vectors). Counted as the difference between 20 and 10 iterations."""
+    import torch
+    L = (8, 10, 12, 14)
+    fat, lng = hin.gen_links(L, 1234, 0.3, 0.1)
+    lat = hisq.Lattice(L, precs=(0, 1)).load(fat, lng)
+    b = torch.from_numpy(hin.gen_source(4321, lat.half, 1)).cuda()
+    x = torch.zeros((nshift, lat.half, 3), dtype=torch.complex128, device="cuda")
+    counts = []
+    for maxiter in (10, 10, 20):  # the first tunes
+        n0 = hisq.hisq_launch_count(lat.ctx)
+        with pytest.raises(hisq.HisqError) as e:
+            lat.multishift_cg(x, b, np.geomspace(1e-3, 1.0, nshift), 0.01, 1e-12, maxiter, inner_prec=inner, poll_every=poll)
+        assert e.value.code == hisq.HISQ_ENOCONV
+        counts.append(hisq.hisq_launch_count(lat.ctx) - n0)
+    assert counts[2] - counts[1] == 40
