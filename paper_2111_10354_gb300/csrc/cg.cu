@@ -371,9 +371,10 @@ __device__ __forceinline__ void finish_iteration(SolverState* st, const double* 
 //            block also commits the iteration (counts, flags, Lanczos record);
 //   phase 2: x += alpha p (X = double: the FP64 solution, X = float: the cycle's FP32 correction);
 //            p = r + beta p.
-// The first KEEP chunks of r a thread updates stay in registers for phase 2; further chunks are read
-// again. Each thread handles its chunks in batches of KEEP whose loads are all issued before any store. Vector traffic: Ap, r read and r written, then p, x (and r beyond KEEP) read and p, x written:
-// seven vector passes where an x/r update launch and a separate p update launch take nine.
+// The first KEEP chunks of r a thread updates are kept for phase 2, in registers but for some words of the FP32 and
+// FP64 forms that spill at 64 registers; further chunks are read again. Each thread handles its chunks in batches of
+// KEEP whose loads are all issued before any store. Vector traffic: Ap, r read and r written, then p, x (and r beyond
+// KEEP) read and p, x written: seven vector passes where an x/r update launch and a separate p update launch take nine.
 // One thread per block forms alpha and beta (and one warp the sums behind them): a division by every thread is
 // some 20 FP64 operations of 16 cycles per warp, microseconds with 32 resident warps per SM. With that and the
 // pair sums (SumAcc) a launch went from 19.3 to 12.8 us for five FP16 vectors on 20x12x28x10 and from 9.7 to 8.8 us
@@ -452,7 +453,11 @@ __global__ void __launch_bounds__(256, 4) k_cg_update(X* __restrict__ x, S* __re
     load_r_Ap(ib, rv, av);
     phase1(ib, rv, av);
   }
-  // the first batch of p and x is requested before the barrier, whose wait then covers its latency
+  // FP64 requests the first batch of p and x before the barrier, whose wait then covers its latency (24^3x16: 42.7 ms a
+  // solve against 42.9). FP32 and 16-bit vectors do not: the words held over the barrier spill, and each solve
+  // measured was slower with them (48^3x12: FP32 43.4 ms against 43.0, FP16 29.5 against 28.9; five FP16 vectors on
+  // 20x12x28x10 9.25 against 8.91).
+  constexpr bool EARLY = sizeof(S) == 8;
   cplx<T> p0[KEEP][K];
   cplx<XT> x0[KEEP][K];
   auto load_p_x = [&](size_t ib, cplx<T>(&pv)[KEEP][K], cplx<XT>(&xv)[KEEP][K]) {
@@ -465,7 +470,7 @@ __global__ void __launch_bounds__(256, 4) k_cg_update(X* __restrict__ x, S* __re
       }
     }
   };
-  if (active) load_p_x(i0, p0, x0);
+  if (EARLY && active) load_p_x(i0, p0, x0);
   const double bs = block_sum_acc(v, red);
   if (threadIdx.x == 0) partials[(size_t)rh * gridDim.x + blockIdx.x] = bs;
   unsigned gen;
@@ -511,6 +516,7 @@ __global__ void __launch_bounds__(256, 4) k_cg_update(X* __restrict__ x, S* __re
         }
       }
     };
+    if (!EARLY) load_p_x(i0, p0, x0);
     phase2(i0, keep, p0, x0);
     for (size_t ib = i0 + KEEP * stride; ib < nn; ib += KEEP * stride) {
       cplx<T> rv[KEEP][K], pv[KEEP][K];
