@@ -47,6 +47,7 @@ struct DslashKArgs {
   void* out;
   const void* in;
   size_t rhs_stride;  // sites between consecutive rhs vectors
+  int nvec;           // vectors of this launch
   const void* y;      // EPI_AXPY
   double a[16];       // per-rhs diagonal coefficient 4m^2 + sigma_r
   float af[16];       // the same rounded to FP32 (a conversion per thread would go through the FP64 pipe)

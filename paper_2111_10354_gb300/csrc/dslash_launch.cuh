@@ -2,9 +2,6 @@
 // nrhs into groups that share each link read and picks the launch form and block size
 // with the autotuner.
 #pragma once
-#include <string>
-#include <vector>
-
 #include "dslash_split.cuh"
 #include "tune.h"
 
@@ -34,50 +31,67 @@ inline void set_walk(const hisq_ctx* ctx, DslashKArgs& a, int zb) {
   a.walk_m_lt = ~0ull / (unsigned long long)ctx->g.L[3] + 1;
 }
 
+// The launch forms of one group of vectors: kernels and their launchers, in the order the tuner numbers them.
+struct DslashForms {
+  static constexpr int CAP = 12;  // 8 vectors have 9 forms, the most
+  const void* func[CAP];
+  cudaError_t (*run[CAP])(hisq_ctx* ctx, const DslashKArgs& a, int block);
+  int n = 0;
+  void add(const void* f, cudaError_t (*r)(hisq_ctx*, const DslashKArgs&, int)) {
+    func[n] = f;
+    run[n++] = r;
+  }
+};
+
 // One launch form: NR vectors per thread, TS threads per site (NR * TS vectors per launch); WALK: the
 // output sites in the tiled walk (walk_zb_for) instead of cb order.
-template <typename LR, typename SR, int NR, int EPI, bool COMP, int TS, bool WALK = false, bool PF = false>
-static TuneVariant dslash_variant(hisq_ctx* ctx, const DslashKArgs& a) {
-  // the launcher captures two pointers only, so std::function keeps it without a heap allocation
-  return TuneVariant{(const void*)dslash_kernel<LR, SR, NR, EPI, COMP, TS, PF>, [ctx, &a](int block) -> cudaError_t {
-                       int grid = (int)(((size_t)ctx->g.half * TS + block - 1) / block);
-                       // Plain launches in cb order: a grid of two resident waves with a grid-stride loop.
-                       // The tiled walk's plain launches take one site per thread: blocks are dispatched in
-                       // index order, so the sites in flight slide through the walk instead of each
-                       // resident wave of a grid-stride loop sweeping the whole lattice in turn (144^3x36:
-                       // DRAM traffic 1.13x -> 1.02x of the algorithmic bytes). Reducing launches: one wave
-                       // of the blocks that are resident together keeps the partials, and the finishing
-                       // block's sum over them, short (a grid of one site per thread made the per-vector
-                       // sums of the 8-vector form the launch's tail).
-                       int cap = WALK ? grid : max_grid_blocks(ctx, block);
-                       if (EPI == EPI_AXPY && a.partials) {
-                         int per_sm = 0;
-                         cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                             &per_sm, dslash_kernel<LR, SR, NR, EPI, COMP, TS, PF>, block, 0);
-                         cap = ctx->num_sms * (per_sm > 0 ? per_sm : 1);
-                       }
-                       if (grid > cap) grid = cap;
-                       DslashKArgs b = a;
-                       if (WALK) set_walk(ctx, b, walk_zb_for(ctx, NR * TS, 6 * sizeof(SR)));
-                       return launch_dependent(ctx, dslash_kernel<LR, SR, NR, EPI, COMP, TS, PF>, grid, block, b);
-                     }};
+template <typename LR, typename SR, int NR, int EPI, bool COMP, int TS, bool WALK, bool PF>
+static cudaError_t run_dslash(hisq_ctx* ctx, const DslashKArgs& a, int block) {
+  int grid = (int)(((size_t)ctx->g.half * TS + block - 1) / block);
+  // Plain launches in cb order: a grid of two resident waves with a grid-stride loop.
+  // The tiled walk's plain launches take one site per thread: blocks are dispatched in
+  // index order, so the sites in flight slide through the walk instead of each
+  // resident wave of a grid-stride loop sweeping the whole lattice in turn (144^3x36:
+  // DRAM traffic 1.13x -> 1.02x of the algorithmic bytes). Reducing launches: one wave
+  // of the blocks that are resident together keeps the partials, and the finishing
+  // block's sum over them, short (a grid of one site per thread made the per-vector
+  // sums of the 8-vector form the launch's tail).
+  int cap = WALK ? grid : max_grid_blocks(ctx, block);
+  if (EPI == EPI_AXPY && a.partials) {
+    int per_sm = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+        &per_sm, dslash_kernel<LR, SR, NR, EPI, COMP, TS, PF>, block, 0);
+    cap = ctx->num_sms * (per_sm > 0 ? per_sm : 1);
+  }
+  if (grid > cap) grid = cap;
+  DslashKArgs b = a;
+  if (WALK) set_walk(ctx, b, walk_zb_for(ctx, NR * TS, 6 * sizeof(SR)));
+  return launch_dependent(ctx, dslash_kernel<LR, SR, NR, EPI, COMP, TS, PF>, grid, block, b);
 }
 
-// One launch form of dslash_split_kernel: ngrp groups of NR vectors, HS threads per (site, group).
+template <typename LR, typename SR, int NR, int EPI, bool COMP, int TS, bool WALK = false, bool PF = false>
+static void add_dslash(DslashForms& f) {
+  f.add((const void*)dslash_kernel<LR, SR, NR, EPI, COMP, TS, PF>, run_dslash<LR, SR, NR, EPI, COMP, TS, WALK, PF>);
+}
+
+// One launch form of dslash_split_kernel: the launch's vectors in groups of NR, HS threads per (site, group).
 template <typename LR, typename SR, int NR, int EPI, int HS>
-static TuneVariant split_variant(hisq_ctx* ctx, const DslashKArgs& a, int ngrp = 1) {
-  return TuneVariant{(const void*)dslash_split_kernel<LR, SR, NR, EPI, HS>, [ctx, &a, ngrp](int block) -> cudaError_t {
-                       int grid = (int)(((size_t)ctx->g.half * HS + block - 1) / block);
-                       int cap = max_grid_blocks(ctx, block);
-                       if (EPI == EPI_AXPY && a.partials) {
-                         int per_sm = 0;
-                         cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                             &per_sm, dslash_split_kernel<LR, SR, NR, EPI, HS>, block, 0);
-                         cap = ctx->num_sms * (per_sm > 0 ? per_sm : 1);
-                       }
-                       if (grid > cap) grid = cap;
-                       return launch_dependent(ctx, dslash_split_kernel<LR, SR, NR, EPI, HS>, dim3(grid, ngrp), block, a);
-                     }};
+static cudaError_t run_split(hisq_ctx* ctx, const DslashKArgs& a, int block) {
+  int grid = (int)(((size_t)ctx->g.half * HS + block - 1) / block);
+  int cap = max_grid_blocks(ctx, block);
+  if (EPI == EPI_AXPY && a.partials) {
+    int per_sm = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+        &per_sm, dslash_split_kernel<LR, SR, NR, EPI, HS>, block, 0);
+    cap = ctx->num_sms * (per_sm > 0 ? per_sm : 1);
+  }
+  if (grid > cap) grid = cap;
+  return launch_dependent(ctx, dslash_split_kernel<LR, SR, NR, EPI, HS>, dim3(grid, a.nvec / NR), block, a);
+}
+
+template <typename LR, typename SR, int NR, int EPI, int HS>
+static void add_split(DslashForms& f) {
+  f.add((const void*)dslash_split_kernel<LR, SR, NR, EPI, HS>, run_split<LR, SR, NR, EPI, HS>);
 }
 
 // The split forms are offered where the site count times the shares fills the GPU at most twice (1024 threads
@@ -86,44 +100,43 @@ inline bool split_fits(const hisq_ctx* ctx, int shares) {
   return (double)ctx->g.half * shares <= 2.0 * ctx->num_sms * 1024;
 }
 
-static int launch_tuned(hisq_ctx* ctx, const char* key, const std::vector<TuneVariant>& v) {
+static int launch_tuned(hisq_ctx* ctx, const char* key, const DslashForms& f, const DslashKArgs& a) {
   int vi = 0, block = 0;
-  int rc = tuned_variant(ctx, key, v.data(), (int)v.size(), &vi, &block);
+  int rc = tuned_variant(ctx, key, f.func, f.n, [&](int i, int b) { return f.run[i](ctx, a, b); }, &vi, &block);
   if (rc != HISQ_OK) return rc;
-  HISQ_CUDA(v[vi].run(block));
+  HISQ_CUDA(f.run[vi](ctx, a, block));
   note_launch(ctx);
   return HISQ_OK;
 }
 
 // The forms of a group of NR vectors in one thread per site, in cb order and (groups of 1 and 5 to 8) in the
-// tiled walk, and, with few sites and uncompressed links, the split forms.
+// tiled walk, and, with few sites and uncompressed links, the split forms; added to f.
 template <typename LR, typename SR, int NR, int EPI, bool COMP>
-static std::vector<TuneVariant> group_forms(hisq_ctx* ctx, const DslashKArgs& a) {
-  std::vector<TuneVariant> v = {dslash_variant<LR, SR, NR, EPI, COMP, 1>(ctx, a)};
-  if (NR == 2) v.push_back(dslash_variant<LR, SR, 1, EPI, COMP, 2>(ctx, a));
+static void group_forms(DslashForms& f, const hisq_ctx* ctx) {
+  add_dslash<LR, SR, NR, EPI, COMP, 1>(f);
+  if (NR == 2) add_dslash<LR, SR, 1, EPI, COMP, 2>(f);
   if (NR == 4) {
-    v.push_back(dslash_variant<LR, SR, 2, EPI, COMP, 2>(ctx, a));
-    v.push_back(dslash_variant<LR, SR, 1, EPI, COMP, 4>(ctx, a));
+    add_dslash<LR, SR, 2, EPI, COMP, 2>(f);
+    add_dslash<LR, SR, 1, EPI, COMP, 4>(f);
   }
   if constexpr (NR == 8) {
-    v.push_back(dslash_variant<LR, SR, 4, EPI, COMP, 2>(ctx, a));
-    v.push_back(dslash_variant<LR, SR, 2, EPI, COMP, 4>(ctx, a));
-    v.push_back(dslash_variant<LR, SR, 8, EPI, COMP, 1, true>(ctx, a));
-    v.push_back(dslash_variant<LR, SR, 4, EPI, COMP, 2, true>(ctx, a));
-    v.push_back(dslash_variant<LR, SR, 2, EPI, COMP, 4, true>(ctx, a));
-    v.push_back(dslash_variant<LR, SR, 8, EPI, COMP, 1, false, true>(ctx, a));
-    v.push_back(dslash_variant<LR, SR, 8, EPI, COMP, 1, true, true>(ctx, a));
+    add_dslash<LR, SR, 4, EPI, COMP, 2>(f);
+    add_dslash<LR, SR, 2, EPI, COMP, 4>(f);
+    add_dslash<LR, SR, 8, EPI, COMP, 1, true>(f);
+    add_dslash<LR, SR, 4, EPI, COMP, 2, true>(f);
+    add_dslash<LR, SR, 2, EPI, COMP, 4, true>(f);
+    add_dslash<LR, SR, 8, EPI, COMP, 1, false, true>(f);
+    add_dslash<LR, SR, 8, EPI, COMP, 1, true, true>(f);
   }
-  if (NR == 1 || (NR > 4 && NR < 8)) v.push_back(dslash_variant<LR, SR, NR, EPI, COMP, 1, true>(ctx, a));
+  if (NR == 1 || (NR > 4 && NR < 8)) add_dslash<LR, SR, NR, EPI, COMP, 1, true>(f);
   if constexpr (!COMP) {
     if constexpr (NR == 1)
-      if (split_fits(ctx, 2)) v.push_back(split_variant<LR, SR, 1, EPI, 2>(ctx, a));
+      if (split_fits(ctx, 2)) add_split<LR, SR, 1, EPI, 2>(f);
     if constexpr (sizeof(LR) < 8 || NR == 1)
-      if (split_fits(ctx, 4)) v.push_back(split_variant<LR, SR, NR, EPI, 4>(ctx, a));
+      if (split_fits(ctx, 4)) add_split<LR, SR, NR, EPI, 4>(f);
     if constexpr (NR == 1)
-      if (split_fits(ctx, 8)) v.push_back(split_variant<LR, SR, 1, EPI, 8>(ctx, a));
+      if (split_fits(ctx, 8)) add_split<LR, SR, 1, EPI, 8>(f);
   }
-  return v;
 }
 
 // A group of nr vectors shares each link read. The launch forms differ in how the group is spread
@@ -131,37 +144,38 @@ static std::vector<TuneVariant> group_forms(hisq_ctx* ctx, const DslashKArgs& a)
 template <typename LR, typename SR, int EPI, bool COMP>
 static int launch_nr(hisq_ctx* ctx, const DslashKArgs& a, int nr) {
   char key[64];
+  DslashForms f;
   snprintf(key, sizeof key, "dslash/l%d/s%d/nr%d/e%d/c%d", Real<LR>::prec, Real<SR>::prec, nr, EPI, (int)COMP);
   if constexpr (sizeof(LR) == 8) {
     if (nr > 1 && split_fits(ctx, 2 * nr)) {  // FP64 on few sites: each vector in its own row of blocks
       snprintf(key, sizeof key, "dslash/l%d/s%d/ny%d/e%d", Real<LR>::prec, Real<SR>::prec, nr, EPI);
-      std::vector<TuneVariant> v = {split_variant<LR, SR, 1, EPI, 2>(ctx, a, nr)};
-      if (split_fits(ctx, 4 * nr)) v.push_back(split_variant<LR, SR, 1, EPI, 4>(ctx, a, nr));
-      if (split_fits(ctx, 8 * nr)) v.push_back(split_variant<LR, SR, 1, EPI, 8>(ctx, a, nr));
+      add_split<LR, SR, 1, EPI, 2>(f);
+      if (split_fits(ctx, 4 * nr)) add_split<LR, SR, 1, EPI, 4>(f);
+      if (split_fits(ctx, 8 * nr)) add_split<LR, SR, 1, EPI, 8>(f);
       // near the line the thread-per-site forms fill the FP64 pipe as well and read each link once for all the
       // vectors (8x10x14x34: two vectors 38.0 us, 38.8 split, four 74.0 and 75.3; 8^4: two vectors 21.2 and 7.2)
-      auto add = [&v](const std::vector<TuneVariant>& g) { v.insert(v.end(), g.begin(), g.end()); };
-      if (nr == 2) add(group_forms<LR, SR, 2, EPI, COMP>(ctx, a));
-      if (nr == 3) add(group_forms<LR, SR, 3, EPI, COMP>(ctx, a));
-      if (nr == 4) add(group_forms<LR, SR, 4, EPI, COMP>(ctx, a));
-      return launch_tuned(ctx, key, v);
+      if (nr == 2) group_forms<LR, SR, 2, EPI, COMP>(f, ctx);
+      if (nr == 3) group_forms<LR, SR, 3, EPI, COMP>(f, ctx);
+      if (nr == 4) group_forms<LR, SR, 4, EPI, COMP>(f, ctx);
+      return launch_tuned(ctx, key, f, a);
     }
   }
   switch (nr) {
-    case 1: return launch_tuned(ctx, key, group_forms<LR, SR, 1, EPI, COMP>(ctx, a));
-    case 2: return launch_tuned(ctx, key, group_forms<LR, SR, 2, EPI, COMP>(ctx, a));
-    case 3: return launch_tuned(ctx, key, group_forms<LR, SR, 3, EPI, COMP>(ctx, a));
-    case 4: return launch_tuned(ctx, key, group_forms<LR, SR, 4, EPI, COMP>(ctx, a));
+    case 1: group_forms<LR, SR, 1, EPI, COMP>(f, ctx); break;
+    case 2: group_forms<LR, SR, 2, EPI, COMP>(f, ctx); break;
+    case 3: group_forms<LR, SR, 3, EPI, COMP>(f, ctx); break;
+    case 4: group_forms<LR, SR, 4, EPI, COMP>(f, ctx); break;
   }
   if constexpr (sizeof(LR) < 8) {
     switch (nr) {
-      case 5: return launch_tuned(ctx, key, group_forms<LR, SR, 5, EPI, COMP>(ctx, a));
-      case 6: return launch_tuned(ctx, key, group_forms<LR, SR, 6, EPI, COMP>(ctx, a));
-      case 7: return launch_tuned(ctx, key, group_forms<LR, SR, 7, EPI, COMP>(ctx, a));
-      case 8: return launch_tuned(ctx, key, group_forms<LR, SR, 8, EPI, COMP>(ctx, a));
+      case 5: group_forms<LR, SR, 5, EPI, COMP>(f, ctx); break;
+      case 6: group_forms<LR, SR, 6, EPI, COMP>(f, ctx); break;
+      case 7: group_forms<LR, SR, 7, EPI, COMP>(f, ctx); break;
+      case 8: group_forms<LR, SR, 8, EPI, COMP>(f, ctx); break;
     }
   }
-  return set_error(HISQ_EINVAL, "unsupported rhs group %d", nr);
+  if (f.n == 0) return set_error(HISQ_EINVAL, "unsupported rhs group %d", nr);
+  return launch_tuned(ctx, key, f, a);
 }
 
 // Largest rhs group per launch: 8, because a group of 16 needs more than the 255 registers a thread can hold
@@ -192,6 +206,7 @@ int dslash_launch_t(hisq_ctx* ctx, const DslashCall& c) {
     a.out = (char*)c.out + (size_t)r0 * c.rhs_stride * site_bytes;
     a.in = (const char*)c.in + (size_t)r0 * c.rhs_stride * site_bytes;
     a.rhs_stride = c.rhs_stride;
+    a.nvec = nr;
     a.y = c.y ? (const char*)c.y + (size_t)r0 * c.rhs_stride * site_bytes : nullptr;
     for (int r = 0; r < 16; ++r) {
       a.a[r] = (c.a_rhs && r0 + r < c.nrhs) ? c.a_rhs[r0 + r] : c.a;

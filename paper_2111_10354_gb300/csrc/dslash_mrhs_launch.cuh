@@ -21,24 +21,22 @@ inline int mrhs_ts(int ngr) {
 }
 
 template <typename LR, typename SR, int NG, int EPI, bool COMP>
-static TuneVariant mrhs_variant(hisq_ctx* ctx, const MrhsArgs& a) {
-  return TuneVariant{(const void*)dslash_mrhs_kernel<LR, SR, NG, EPI, COMP>, [ctx, &a](int block) -> cudaError_t {
-                       MrhsArgs b = a;
-                       b.ts = mrhs_ts<NG>(a.ngr);
-                       if (block % b.ts) return cudaErrorInvalidConfiguration;
-                       int grid = (int)(((size_t)ctx->g.half * b.ts + block - 1) / block);
-                       int cap = max_grid_blocks(ctx, block);
-                       if (EPI == EPI_AXPY && a.partials) {
-                         // reducing launches: one wave of co-resident blocks keeps the partials short
-                         int per_sm = 0;
-                         cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-                             &per_sm, dslash_mrhs_kernel<LR, SR, NG, EPI, COMP>, block, 0);
-                         cap = ctx->num_sms * (per_sm > 0 ? per_sm : 1);
-                       }
-                       if (grid > cap) grid = cap;
-                       dslash_mrhs_kernel<LR, SR, NG, EPI, COMP><<<grid, block, 0, ctx->stream>>>(b);
-                       return cudaGetLastError();
-                     }};
+static cudaError_t run_mrhs(hisq_ctx* ctx, const MrhsArgs& a, int block) {
+  MrhsArgs b = a;
+  b.ts = mrhs_ts<NG>(a.ngr);
+  if (block % b.ts) return cudaErrorInvalidConfiguration;
+  int grid = (int)(((size_t)ctx->g.half * b.ts + block - 1) / block);
+  int cap = max_grid_blocks(ctx, block);
+  if (EPI == EPI_AXPY && a.partials) {
+    // reducing launches: one wave of co-resident blocks keeps the partials short
+    int per_sm = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+        &per_sm, dslash_mrhs_kernel<LR, SR, NG, EPI, COMP>, block, 0);
+    cap = ctx->num_sms * (per_sm > 0 ? per_sm : 1);
+  }
+  if (grid > cap) grid = cap;
+  dslash_mrhs_kernel<LR, SR, NG, EPI, COMP><<<grid, block, 0, ctx->stream>>>(b);
+  return cudaGetLastError();
 }
 
 // The launch forms for ngr granules per site: NG granules per thread with at most 32 threads per site
@@ -46,20 +44,25 @@ static TuneVariant mrhs_variant(hisq_ctx* ctx, const MrhsArgs& a) {
 template <typename LR, typename SR, int EPI, bool COMP>
 static int mrhs_launch_forms(hisq_ctx* ctx, const MrhsArgs& a, const char* key) {
   const int ngr = a.ngr;
-  TuneVariant v[3];
+  const void* func[3];
+  cudaError_t (*run[3])(hisq_ctx*, const MrhsArgs&, int);
   int nv = 0;
-  if (mrhs_ts<1>(ngr) <= 32) v[nv++] = mrhs_variant<LR, SR, 1, EPI, COMP>(ctx, a);
-  if (ngr >= 2 && mrhs_ts<2>(ngr) <= 32) v[nv++] = mrhs_variant<LR, SR, 2, EPI, COMP>(ctx, a);
+  auto add = [&](const void* f, cudaError_t (*r)(hisq_ctx*, const MrhsArgs&, int)) {
+    func[nv] = f;
+    run[nv++] = r;
+  };
+  if (mrhs_ts<1>(ngr) <= 32) add((const void*)dslash_mrhs_kernel<LR, SR, 1, EPI, COMP>, run_mrhs<LR, SR, 1, EPI, COMP>);
+  if (ngr >= 2 && mrhs_ts<2>(ngr) <= 32) add((const void*)dslash_mrhs_kernel<LR, SR, 2, EPI, COMP>, run_mrhs<LR, SR, 2, EPI, COMP>);
   // four granules per thread only where they are four FP32 granules (8 vectors): 16 vectors of 16-bit
   // storage spill
   if constexpr (std::is_same<SR, float>::value) {
-    if (ngr >= 4) v[nv++] = mrhs_variant<LR, SR, 4, EPI, COMP>(ctx, a);
+    if (ngr >= 4) add((const void*)dslash_mrhs_kernel<LR, SR, 4, EPI, COMP>, run_mrhs<LR, SR, 4, EPI, COMP>);
   }
   if (nv == 0) return set_error(HISQ_EINVAL, "no launch form for %d granules per site", ngr);
   int vi = 0, block = 0;
-  int rc = tuned_variant(ctx, key, v, nv, &vi, &block);
+  int rc = tuned_variant(ctx, key, func, nv, [&](int i, int b) { return run[i](ctx, a, b); }, &vi, &block);
   if (rc != HISQ_OK) return rc;
-  HISQ_CUDA(v[vi].run(block));
+  HISQ_CUDA(run[vi](ctx, a, block));
   note_launch(ctx);
   return HISQ_OK;
 }

@@ -498,12 +498,12 @@ __global__ void __launch_bounds__(SMEAR_BLOCK) k_project_u3(double2* out, const 
 // block size. All three passes are idempotent (their outputs are not read), so they can be timed.
 template <typename Kern, typename Launch>
 int launch_pass(hisq_ctx* ctx, const char* key, Kern k1, Kern k2, Launch launch) {
-  TuneVariant v[2] = {{(const void*)k1, [&](int b) { return launch(k1, b); }},
-                      {(const void*)k2, [&](int b) { return launch(k2, b); }}};
+  const void* func[2] = {(const void*)k1, (const void*)k2};
+  auto run = [&](int i, int b) { return launch(i == 0 ? k1 : k2, b); };
   int vi = 0, block = SMEAR_BLOCK;
-  int rc = tuned_variant(ctx, key, v, 2, &vi, &block);
+  int rc = tuned_variant(ctx, key, func, 2, run, &vi, &block);
   if (rc) return rc;
-  HISQ_CUDA(v[vi].run(block));
+  HISQ_CUDA(run(vi, block));
   note_launch(ctx);
   return HISQ_OK;
 }

@@ -6,8 +6,6 @@
 #pragma once
 #include <stdio.h>
 
-#include <functional>
-
 #include "internal.cuh"
 
 namespace hisq {
@@ -17,16 +15,12 @@ inline int max_grid_blocks(const hisq_ctx* ctx, int block) { return ctx->num_sms
 // Room per rhs in reduction-partials buffers (covers the smallest tuned block, 64).
 inline size_t partial_stride(const hisq_ctx* ctx) { return (size_t)ctx->num_sms * 64; }
 
-// One candidate kernel form for the tuner: its function (for the block-size limit) and a launcher
-// taking the block size.
-struct TuneVariant {
-  const void* func;
-  std::function<cudaError_t(int)> run;
-};
-
-// Times every (variant, block size) pair once per key and caches the fastest as
-// variant * 10000 + block. With one variant this is a plain block-size tuner.
-inline int tuned_variant(hisq_ctx* ctx, const char* key, const TuneVariant* v, int nv, int* vi_out, int* block_out) {
+// Times every (kernel form, block size) pair once per key and caches the fastest as form * 10000 + block. func[nv]: the
+// forms' kernels (for the block-size limit); run(form, block) launches one. With one form this is a plain block-size
+// tuner. The forms are plain pointers because every launch lists them, also of a tuned key, and launches on small
+// lattices are bound by the host (std::function objects in a std::vector: 2.9 us of its time a call at 8^4, now 2.7).
+template <typename Run>
+int tuned_variant(hisq_ctx* ctx, const char* key, const void* const* func, int nv, Run&& run, int* vi_out, int* block_out) {
   auto it = ctx->tune.find(key);
   if (it != ctx->tune.end() && it->second > 0) {
     *vi_out = it->second / 10000;
@@ -39,7 +33,7 @@ inline int tuned_variant(hisq_ctx* ctx, const char* key, const TuneVariant* v, i
     const int vi = -it->second / 10000, b = -it->second % 10000;
     cudaFuncAttributes fa;
     if (vi < nv && b >= 32 && b % 32 == 0 &&
-        cudaFuncGetAttributes(&fa, v[vi].func) == cudaSuccess && b <= fa.maxThreadsPerBlock) {
+        cudaFuncGetAttributes(&fa, func[vi]) == cudaSuccess && b <= fa.maxThreadsPerBlock) {
       it->second = -it->second;
       *vi_out = vi;
       *block_out = b;
@@ -52,7 +46,7 @@ inline int tuned_variant(hisq_ctx* ctx, const char* key, const TuneVariant* v, i
   HISQ_CUDA(cudaStreamIsCapturing(ctx->stream, &cap));
   if (!ctx->autotune || cap != cudaStreamCaptureStatusNone) {
     cudaFuncAttributes fa;
-    HISQ_CUDA(cudaFuncGetAttributes(&fa, v[0].func));
+    HISQ_CUDA(cudaFuncGetAttributes(&fa, func[0]));
     const int b = fa.maxThreadsPerBlock >= 256 ? 256 : 128;
     *vi_out = 0;
     *block_out = b;
@@ -69,13 +63,13 @@ inline int tuned_variant(hisq_ctx* ctx, const char* key, const TuneVariant* v, i
   int best_v = 0, best_b = 128;
   for (int i = 0; i < nv; ++i) {
     cudaFuncAttributes fa;
-    if (cudaFuncGetAttributes(&fa, v[i].func) != cudaSuccess) {
+    if (cudaFuncGetAttributes(&fa, func[i]) != cudaSuccess) {
       cudaGetLastError();
       continue;
     }
     for (int b : cands) {
       if (b > fa.maxThreadsPerBlock) continue;
-      cudaError_t err = v[i].run(b);  // warm-up
+      cudaError_t err = run(i, b);  // warm-up
       if (err != cudaSuccess) {
         cudaGetLastError();
         continue;
@@ -87,7 +81,7 @@ inline int tuned_variant(hisq_ctx* ctx, const char* key, const TuneVariant* v, i
       // launch of the first one do not decide between small kernels
       for (int reps = 3; timed; reps = 20) {
         cudaEventRecord(e0, ctx->stream);
-        for (int r = 0; r < reps; ++r) v[i].run(b);
+        for (int r = 0; r < reps; ++r) run(i, b);
         note_launch(ctx, reps);
         cudaEventRecord(e1, ctx->stream);
         timed = cudaEventSynchronize(e1) == cudaSuccess;
@@ -111,13 +105,6 @@ inline int tuned_variant(hisq_ctx* ctx, const char* key, const TuneVariant* v, i
   *vi_out = best_v;
   *block_out = best_b;
   return HISQ_OK;
-}
-
-template <typename Run>
-int tuned_block(hisq_ctx* ctx, const char* key, const void* func, Run run, int* block_out) {
-  TuneVariant v{func, run};
-  int vi = 0;
-  return tuned_variant(ctx, key, &v, 1, &vi, block_out);
 }
 
 }  // namespace hisq
