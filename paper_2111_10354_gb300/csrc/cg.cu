@@ -27,6 +27,7 @@
 
 #include "solver_common.cuh"
 #include "reduce_warp.cuh"
+#include "sizing.h"
 #include "trace.h"
 #include "tune.h"
 
@@ -1601,11 +1602,13 @@ static int run_multishift(hisq_ctx* ctx, double2* x, const double2* b, int ns, c
   double* partials = (double*)workspace(ctx, "ms_partials", 2 * MAXR * partial_stride(ctx) * sizeof(double));
   // the residuals of a group of iterations, taken last; shorter groups where more would not leave the
   // verification its room (at most 112 bytes an entry and shift)
+  const size_t held = ctx->ws["ms_r"].bytes;
   int slots = ns > 1 ? MS_SLOTS : 1;
-  if (slots > 1 && ctx->ws["ms_r"].bytes < slots * n * 2 * sizeof(S)) {
-    size_t free_b = 0, total_b = 0;
+  if (slots * n * 2 * sizeof(S) > held) {
+    size_t free_b = 0, total_b = 0, verify_held = 0;
     HISQ_CUDA(cudaMemGetInfo(&free_b, &total_b));
-    while (slots > 1 && slots * n * 2 * sizeof(S) + (size_t)ns * n * 128 > free_b) slots /= 2;
+    for (const char* w : {"cg_rhi", "cg_Ax", "cg_t64", "cg_r", "cg_p", "cg_Ap", "cg_t", "cg_e"}) verify_held += ctx->ws[w].bytes;
+    slots = ms_group_length(slots, n * 2 * sizeof(S), held, (size_t)ns * n * 128, verify_held, free_b);
   }
   S* r = nullptr;
   for (; slots >= 1 && !r; slots /= 2) r = (S*)workspace(ctx, "ms_r", slots * n * 2 * sizeof(S));
