@@ -751,7 +751,6 @@ struct CgBuffers {
   SolverState* st;
   double* partials;
   int rp = HISQ_F64;     // operator precision of the true residual: HISQ_F64 or HISQ_DF64
-  unsigned* rowc;        // per-rhs block counters of the row reductions [MAXR]
   bool il = false;       // inner vectors (r, p, Ap, t, e) in the rhs-interleaved layout [cb][color][rhs]
   int P = 0;             // il: rhs pairs per site (nrhs / 2)
   int il_block = 0;      // il: threads per block of the interleaved BLAS kernels (P x a power of two)
@@ -1000,10 +999,9 @@ static int run_cg(hisq_ctx* ctx, double2* x, const double2* b, size_t b_stride, 
   B.t = workspace(ctx, "cg_t", vbS);
   B.st = (SolverState*)workspace(ctx, "cg_state", sizeof(SolverState));
   B.partials = (double*)workspace(ctx, "cg_partials", 3 * MAXR * partial_stride(ctx) * sizeof(double));
-  B.rowc = (unsigned*)workspace(ctx, "cg_rowc", MAXR * sizeof(unsigned));
   B.e = mixed ? workspace(ctx, "cg_e", (size_t)nrhs * n * 2 * sizeof(float)) : (void*)x;
   SolverState* hst = (SolverState*)ctx->pinned;
-  if (!B.r_hi || !B.Ax || !B.t64 || !B.r || !B.p || !B.Ap || !B.t || !B.st || !B.partials || !B.e || !B.rowc)
+  if (!B.r_hi || !B.Ax || !B.t64 || !B.r || !B.p || !B.Ap || !B.t || !B.st || !B.partials || !B.e)
     return set_error(HISQ_ENOMEM, "solver workspace");
   // on request (vector_layout 1), mixed precision with an even number of rhs keeps its inner vectors
   // interleaved per site, so the Dslash reads each neighbour's nrhs vectors as one block
@@ -1016,7 +1014,6 @@ static int run_cg(hisq_ctx* ctx, double2* x, const double2* b, size_t b_stride, 
   }
   int prc = plan_update<S>(ctx, B, nrhs);
   if (prc != HISQ_OK) return prc;
-  HISQ_CUDA(cudaMemsetAsync(B.rowc, 0, MAXR * sizeof(unsigned), ctx->stream));
   if (mixed) HISQ_CUDA(cudaMemsetAsync(B.e, 0, (size_t)nrhs * n * 2 * sizeof(float), ctx->stream));
   auto fold = [&]() -> int {
     if (!mixed) return HISQ_OK;
@@ -1092,7 +1089,7 @@ static int run_cg(hisq_ctx* ctx, double2* x, const double2* b, size_t b_stride, 
                       "/" + std::to_string(cycle);
     char buf[64];
     for (const void* ptr : {(const void*)B.r, (const void*)B.p, (const void*)B.Ap, (const void*)B.t,
-                            (const void*)B.e, (const void*)B.st, (const void*)B.partials, (const void*)B.rowc}) {
+                            (const void*)B.e, (const void*)B.st, (const void*)B.partials}) {
       snprintf(buf, sizeof buf, "/%p", ptr);
       key += buf;
     }

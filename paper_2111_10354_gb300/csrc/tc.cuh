@@ -17,13 +17,9 @@ __device__ __forceinline__ uint32_t smem_addr(const void* p) {
   return (uint32_t)__cvta_generic_to_shared(p);
 }
 
-// Byte offset of element (row, col) in a K-major no-swizzle tile with K2 columns.
-__host__ __device__ __forceinline__ uint32_t kmajor_offset(int row, int col, int K2) {
-  return (uint32_t)((row >> 3) * (K2 >> 3) * 128 + (col >> 3) * 128 + (row & 7) * 16 + (col & 7) * 2);
-}
-
 // Shared-memory matrix descriptor (tcgen05 format): start address, LBO, SBO (all >> 4),
-// descriptor version 1 at bits 46-47, layout type 0 (no swizzle) at bits 61-63.
+// descriptor version 1 at bits 46-47, layout type 0 (no swizzle) at bits 61-63. The tile is K-major with K2 columns of
+// 16 bits: 8 x 8 blocks of 128 bytes, a row of 16 bytes each, the K2 / 8 blocks of 8 rows one after the other.
 __device__ __forceinline__ uint64_t desc_kmajor(uint32_t saddr, int K2) {
   const uint64_t lbo = 128, sbo = (uint64_t)(K2 >> 3) * 128;
   return (uint64_t)((saddr >> 4) & 0x3FFF) | (((lbo >> 4) & 0x3FFF) << 16) | (((sbo >> 4) & 0x3FFF) << 32) |
