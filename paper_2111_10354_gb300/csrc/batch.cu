@@ -172,9 +172,13 @@ __device__ __forceinline__ bool grid_last(unsigned* c) {
 // ------------------------------------------------------------------ batched Dslash
 // out_l = D in_l (EPI_PLAIN) or out_l = a_l y_l - D in_l with pAp_l = Re<y_l, out_l> and alpha_l = rr_l / pAp_l
 // (EPI_AXPY), for every lattice l whose skip[l] is 0. FP32 takes 80 registers (three blocks of 256 per SM): at 64, like
-// the single-lattice form, the tile walk spills (16 lattices, all active: 174 and 196 us against 164 and 181 us).
-template <typename LR, typename SR, int EPI>
-__global__ void __launch_bounds__(256, sizeof(LR) == 4 ? 3 : 0) k_bdslash(const BatchArgs a, int p, void* out, const void* in,
+// the single-lattice form, the tile walk spills (16 lattices, all active: 174 and 196 us against 164 and 181 us). NARROW:
+// 72 registers in blocks of up to 128, seven per SM. It spills more and is slower (those 16 lattices 53.0 ms a solve
+// against 51.4, six 16^4 20.8 against 18.9), except where its 14% more threads take all sites at once and 80
+// registers leave some for a second round (four 16^4: 13.8 against 15.6); FP32 is tuned over both.
+template <typename LR, typename SR, int EPI, bool NARROW>
+__global__ void __launch_bounds__(NARROW ? 128 : 256, NARROW ? 7 : sizeof(LR) == 4 ? 3 : 0)
+    k_bdslash(const BatchArgs a, int p, void* out, const void* in,
                                                                          const void* y, const int* skip, BatchState* st,
                                                                          double* partials, int red_row) {
   using A = typename Real<LR>::acc;
@@ -582,7 +586,10 @@ struct BatchBufs {
 template <typename LR, typename SR, int EPI>
 static int bdslash(hisq_batch* B, int p, void* out, const void* in, const void* y, const int* skip, BatchState* st,
                    double* partials, int red_row) {
-  auto kern = k_bdslash<LR, SR, EPI>;
+  constexpr int FORMS = sizeof(LR) == 4 ? 2 : 1;
+  decltype(&k_bdslash<LR, SR, EPI, false>) kerns[2] = {k_bdslash<LR, SR, EPI, false>, nullptr};
+  if constexpr (FORMS == 2) kerns[1] = k_bdslash<LR, SR, EPI, true>;
+  int form = 0;
   char key[64];
   snprintf(key, sizeof key, "bdslash/l%d/s%d/e%d", Real<LR>::prec, Real<SR>::prec, EPI);
   int block = 0;
@@ -590,40 +597,70 @@ static int bdslash(hisq_batch* B, int p, void* out, const void* in, const void* 
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   HISQ_CUDA(cudaStreamIsCapturing(B->stream, &cap));
   if (it != B->tune.end()) {
-    block = it->second;
+    form = it->second / 10000;
+    block = it->second % 10000;
   } else if (cap != cudaStreamCaptureStatusNone) {
     block = 128;
   } else {
-    // autotune the tile size: time each candidate (the launch is idempotent). 224 rather than 256: a 16^4 lattice's
-    // 32,768 sites are then 147 tiles for 152 SMs, and FP64 tiles are bound by their SM's FP64 pipe
-    static const int cands[] = {64, 128, 224};
+    // Autotune the form and the tile size: each whole number of warps from 64 sites to 256, by the time with all
+    // lattices active (three parts) and with the largest alone (one part; the launch is idempotent). How the tiles
+    // fall on the SMs decides, which no few sizes suit for every batch, and the tile that is best for all lattices may
+    // be the worst for the few of a solve's last cycles: FP64, 14^2x18x22 + 10x12x26x30 + 18^4, 256 is best with all
+    // active and gave 115.7 ms a solve, 96 108.1; four 16^4 57.5 with 224 and 60-63 with any other.
+    std::vector<int> act(2 * B->nlat, 1);
+    int largest = 0;
+    for (int l = 1; l < B->nlat; ++l)
+      if (B->lat[l]->g.half > B->lat[largest]->g.half) largest = l;
+    for (int l = 0; l < B->nlat; ++l) act[l] = 0;
+    act[B->nlat + largest] = 0;
+    int* d_act = (int*)bws(B, "tile_act", act.size() * sizeof(int));
+    if (!d_act) return set_error(HISQ_ENOMEM, "batch workspace");
+    HISQ_CUDA(cudaMemcpyAsync(d_act, act.data(), act.size() * sizeof(int), cudaMemcpyHostToDevice, B->stream));
+    HISQ_CUDA(cudaStreamSynchronize(B->stream));
     cudaEvent_t e0, e1;
     HISQ_CUDA(cudaEventCreate(&e0));
     HISQ_CUDA(cudaEventCreate(&e1));
     float best = 1e30f;
-    for (int c : cands) {
+    for (int k = 0; k < FORMS * 7; ++k) {
+      const int f = k / 7, c = 64 + 32 * (k % 7);
+      if (f == 1 && c > 128) continue;
+      auto kern = kerns[f];
       TileTable* T;
       int rc = tile_table(B, c, &T);
       if (rc != HISQ_OK) return rc;
       const BatchArgs a = batch_args(B, Real<LR>::prec, c, *T);
       const int grid = persistent_grid(B, (const void*)kern, c);
-      kern<<<grid, c, 0, B->stream>>>(a, p, out, in, y, skip, st, partials, red_row);
-      cudaEventRecord(e0, B->stream);
-      for (int r = 0; r < 3; ++r) kern<<<grid, c, 0, B->stream>>>(a, p, out, in, y, skip, st, partials, red_row);
-      cudaEventRecord(e1, B->stream);
-      B->launches += 4;
-      HISQ_CUDA(cudaEventSynchronize(e1));
-      float ms = 0;
-      cudaEventElapsedTime(&ms, e0, e1);
+      auto run = [&](const int* sk) { kern<<<grid, c, 0, B->stream>>>(a, p, out, in, y, sk, st, partials, red_row); };
+      run(d_act + B->nlat);  // warm-up
+      B->launches += 1;
+      auto timed = [&](const int* sk, float* ms) -> cudaError_t {  // one launch; short ones eight
+        for (int reps = 1;; reps = 8) {
+          cudaEventRecord(e0, B->stream);
+          for (int r = 0; r < reps; ++r) run(sk);
+          cudaEventRecord(e1, B->stream);
+          B->launches += reps;
+          const cudaError_t e = cudaEventSynchronize(e1);
+          if (e != cudaSuccess) return e;
+          cudaEventElapsedTime(ms, e0, e1);
+          *ms /= (float)reps;
+          if (reps == 8 || *ms >= 0.2f) return cudaSuccess;
+        }
+      };
+      float ms = 0, alone = 0;
+      HISQ_CUDA(timed(d_act, &ms));
+      HISQ_CUDA(timed(d_act + B->nlat, &alone));
+      ms = 3.f * ms + alone;
       if (ms < best) {
         best = ms;
+        form = f;
         block = c;
       }
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    B->tune[key] = block;
+    B->tune[key] = form * 10000 + block;
   }
+  auto kern = kerns[form];
   TileTable* T;
   int rc = tile_table(B, block, &T);
   if (rc != HISQ_OK) return rc;
@@ -719,7 +756,7 @@ static int run_batch(hisq_batch* B, double2* x, const double2* b, const double* 
   U.t = bws(B, "t", n * 2 * sizeof(S));
   U.e = mixed ? bws(B, "e", n * 2 * sizeof(float)) : (void*)x;
   U.st = (BatchState*)bws(B, "state", sizeof(BatchState));
-  // partials: 3 rows of one double per tile of the smallest tile size (64)
+  // partials: 4 rows of one double per tile of the smallest tile size (64)
   size_t max_tiles = 0;
   for (int l = 0; l < B->nlat; ++l) max_tiles += (B->lat[l]->g.half + 63) / 64;
   U.partials = (double*)bws(B, "partials", 4 * max_tiles * sizeof(double));
