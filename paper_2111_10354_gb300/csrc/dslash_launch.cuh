@@ -3,6 +3,7 @@
 // with the autotuner.
 #pragma once
 #include "dslash_split.cuh"
+#include "sizing.h"
 #include "tune.h"
 
 namespace hisq {
@@ -153,7 +154,7 @@ static int launch_nr(hisq_ctx* ctx, const DslashKArgs& a, int nr) {
       if (split_fits(ctx, 4 * nr)) add_split<LR, SR, 1, EPI, 4>(f);
       if (split_fits(ctx, 8 * nr)) add_split<LR, SR, 1, EPI, 8>(f);
       // near the line the thread-per-site forms fill the FP64 pipe as well and read each link once for all the
-      // vectors (8x10x14x34: two vectors 38.0 us, 38.8 split, four 74.0 and 75.3; 8^4: two vectors 21.2 and 7.2)
+      // vectors (8x10x14x34: two vectors 38.4 us, 39.1 split, four 74.2 and 75.7; 8^4: two vectors 21.2 and 7.2)
       if (nr == 2) group_forms<LR, SR, 2, EPI, COMP>(f, ctx);
       if (nr == 3) group_forms<LR, SR, 3, EPI, COMP>(f, ctx);
       if (nr == 4) group_forms<LR, SR, 4, EPI, COMP>(f, ctx);
@@ -189,15 +190,19 @@ static int max_group(const hisq_ctx* ctx) {
   return n;
 }
 
+// Whether the context holds compressed long links (two rows, third reconstructed) of the precision.
+template <typename LR>
+static bool compressed(const hisq_ctx* ctx) {
+  return sizeof(LR) < 8 && ctx->naik != 0.0 && ctx->long12[Real<LR>::prec] != nullptr;
+}
+
+// One launch per group of vectors, cut as given (LaunchCut).
 template <typename LR, typename SR>
-int dslash_launch_t(hisq_ctx* ctx, const DslashCall& c) {
+static int launch_groups(hisq_ctx* ctx, const DslashCall& c, int cut, int gmax) {
   const size_t site_bytes = 6 * sizeof(SR);
-  const int gmax = max_group<LR>(ctx);
   int r0 = 0;
   while (r0 < c.nrhs) {
-    const int left = c.nrhs - r0;
-    // groups of nearly equal size: the cost of a launch's link read is spread over all of them
-    const int ngrp = (left + gmax - 1) / gmax, nr = (left + ngrp - 1) / ngrp;
+    const int nr = next_group(cut, c.nrhs - r0, gmax);
     DslashKArgs a;
     a.g = ctx->g;
     a.links = ctx->links[Real<LR>::prec];
@@ -216,8 +221,7 @@ int dslash_launch_t(hisq_ctx* ctx, const DslashCall& c) {
     a.dot_out = c.dot_out ? c.dot_out + r0 : nullptr;
     a.counter = c.counter;
     a.skip = c.skip;
-    // compressed long links (two rows, third reconstructed) whenever the context keeps them
-    const bool comp = sizeof(LR) < 8 && ctx->naik != 0.0 && ctx->long12[Real<LR>::prec] != nullptr;
+    const bool comp = compressed<LR>(ctx);
     a.long12 = comp ? ctx->long12[Real<LR>::prec] : nullptr;
     a.blk12 = long12_block_bytes(Real<LR>::prec, ctx->g.half);
     a.inv_naik = comp ? (float)(1.0 / ctx->naik) : 0.f;
@@ -238,6 +242,26 @@ int dslash_launch_t(hisq_ctx* ctx, const DslashCall& c) {
     r0 += nr;
   }
   return HISQ_OK;
+}
+
+// D (or A's second half) on c.nrhs vectors. Where they can be cut in more than one way the tuner times each: no way is
+// best everywhere. Measured, us: FP32, 12 vectors, 8+4 27.3 at 16^4 and 392 at 48^3x12, 6+6 34.7 and 416; FP32, 9
+// vectors, 8+1 23.1 and 354, 5+4 26.9 and 342; double-float, 6 vectors at 32^3x8, 4+2 286, 3+3 371; FP64, 6 vectors,
+// 4+2 258 at 16^4 and 734 at 32^3x8, 3+3 194 and 765. The powers of two (2+1 for 3) matter for FP64 and double-float,
+// whose launch of three takes nearly as long as one of four.
+template <typename LR, typename SR>
+int dslash_launch_t(hisq_ctx* ctx, const DslashCall& c) {
+  const int gmax = max_group<LR>(ctx);
+  // few sites in FP64, where a launch is a row of blocks per vector: even groups (A of 10 vectors at 8^4: 59.5 us, 8+2 88)
+  if (sizeof(LR) == 8 && gmax > 4) return launch_groups<LR, SR>(ctx, c, CUT_EVEN, gmax);
+  int cuts[3], cut;
+  const int n = launch_cuts(c.nrhs, gmax, sizeof(LR) == 8, cuts);
+  if (n == 1) return launch_groups<LR, SR>(ctx, c, cuts[0], gmax);
+  char key[64];
+  snprintf(key, sizeof key, "dslash/l%d/s%d/cut%d/e%d/c%d", Real<LR>::prec, Real<SR>::prec, c.nrhs, c.epi, (int)compressed<LR>(ctx));
+  int rc = tuned_way(ctx, key, cuts, n, [&](int w) { return launch_groups<LR, SR>(ctx, c, w, gmax); }, &cut);
+  if (rc != HISQ_OK) return rc;
+  return launch_groups<LR, SR>(ctx, c, cut, gmax);
 }
 
 }  // namespace hisq

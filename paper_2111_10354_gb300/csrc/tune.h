@@ -15,6 +15,23 @@ inline int max_grid_blocks(const hisq_ctx* ctx, int block) { return ctx->num_sms
 // Room per rhs in reduction-partials buffers (covers the smallest tuned block, 64).
 inline size_t partial_stride(const hisq_ctx* ctx) { return (size_t)ctx->num_sms * 64; }
 
+// Milliseconds of one run() (idempotent launches on the context's stream, warmed up by the caller), or below 0 on an
+// error. Three runs; where those take less than 60 us in all, twenty, so that the events' own cost and the launch of
+// the first one do not decide between small kernels.
+template <typename Run>
+float time_launches(hisq_ctx* ctx, cudaEvent_t e0, cudaEvent_t e1, Run&& run) {
+  for (int reps = 3;; reps = 20) {
+    float ms = 0;
+    cudaEventRecord(e0, ctx->stream);
+    for (int r = 0; r < reps; ++r) run();
+    cudaEventRecord(e1, ctx->stream);
+    if (cudaEventSynchronize(e1) != cudaSuccess) return -1.f;
+    cudaEventElapsedTime(&ms, e0, e1);
+    ms /= (float)reps;
+    if (reps == 20 || ms >= 0.02f) return ms;
+  }
+}
+
 // Times every (kernel form, block size) pair once per key and caches the fastest as form * 10000 + block. func[nv]: the
 // forms' kernels (for the block-size limit); run(form, block) launches one. With one form this is a plain block-size
 // tuner. The forms are plain pointers because every launch lists them, also of a tuned key, and launches on small
@@ -75,22 +92,11 @@ int tuned_variant(hisq_ctx* ctx, const char* key, const void* const* func, int n
         continue;
       }
       note_launch(ctx);
-      float ms = 0;
-      bool timed = true;
-      // three launches; where those take less than 60 us in all, twenty, so that the events' own cost and the
-      // launch of the first one do not decide between small kernels
-      for (int reps = 3; timed; reps = 20) {
-        cudaEventRecord(e0, ctx->stream);
-        for (int r = 0; r < reps; ++r) run(i, b);
-        note_launch(ctx, reps);
-        cudaEventRecord(e1, ctx->stream);
-        timed = cudaEventSynchronize(e1) == cudaSuccess;
-        if (!timed) break;
-        cudaEventElapsedTime(&ms, e0, e1);
-        ms /= (float)reps;
-        if (reps == 20 || ms >= 0.02f) break;
-      }
-      if (!timed) break;
+      const float ms = time_launches(ctx, e0, e1, [&] {
+        run(i, b);
+        note_launch(ctx);
+      });
+      if (ms < 0.f) break;
       if (ms < best) {
         best = ms;
         best_v = i;
@@ -104,6 +110,49 @@ int tuned_variant(hisq_ctx* ctx, const char* key, const void* const* func, int n
   ctx->tune[key] = best_v * 10000 + best_b;
   *vi_out = best_v;
   *block_out = best_b;
+  return HISQ_OK;
+}
+
+// The fastest of n ways to make a call, each timed once per key (run(way) makes it and returns a status; its own launches
+// are tuned by its first run); kept as way + 1. Not timed inside a capture or with the tuner off: the first way.
+template <typename Run>
+int tuned_way(hisq_ctx* ctx, const char* key, const int* ways, int n, Run&& run, int* way) {
+  *way = ways[0];
+  auto it = ctx->tune.find(key);
+  if (it != ctx->tune.end()) {
+    const int v = it->second < 0 ? -it->second : it->second;  // negative: loaded from a report, unchecked
+    for (int i = 0; i < n; ++i)
+      if (ways[i] + 1 == v) {
+        it->second = v;
+        *way = ways[i];
+        return HISQ_OK;
+      }
+    ctx->tune.erase(it);
+  }
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  HISQ_CUDA(cudaStreamIsCapturing(ctx->stream, &cap));
+  if (!ctx->autotune || cap != cudaStreamCaptureStatusNone) return HISQ_OK;
+  cudaEvent_t e0, e1;
+  HISQ_CUDA(cudaEventCreate(&e0));
+  HISQ_CUDA(cudaEventCreate(&e1));
+  float best = 1e30f;
+  int rc = HISQ_OK;
+  for (int i = 0; i < n && rc == HISQ_OK; ++i) {
+    if ((rc = run(ways[i])) != HISQ_OK) break;
+    const float ms = time_launches(ctx, e0, e1, [&] {
+      const int r = run(ways[i]);
+      if (r != HISQ_OK) rc = r;
+    });
+    if (ms >= 0.f && ms < best) {
+      best = ms;
+      *way = ways[i];
+    }
+  }
+  cudaEventDestroy(e0);
+  cudaEventDestroy(e1);
+  if (rc != HISQ_OK) return rc;
+  HISQ_CUDA(cudaGetLastError());
+  ctx->tune[key] = *way + 1;
   return HISQ_OK;
 }
 

@@ -366,3 +366,33 @@ def test_odd_vector_groups_match_oracle(hisq, prec):
             got = from_device(y, prec)
             for r in range(nr):
                 assert rel_err(got[r], oracle.apply_A(L, ff, lf, 0.05, src[r])) <= 2 * TOL[prec], (nr, vi, r)
+
+
+@pytest.mark.parametrize("prec,nrhs", [(1, 9), (2, 12), (0, 5), (0, 7), (4, 3), (4, 6)])
+def test_every_way_to_cut_vectors_into_launches(hisq, prec, nrhs):
+    """Vectors that more than one sequence of launches can take (full groups and the rest, even groups, powers of two),
+    each forced through a loaded tune entry, the Dslash and A against the oracle; an entry that names no way is
+    dropped and the call tuned again. 16^4: too many sites for FP64's rows of blocks to take five vectors at once."""
+    L = (16, 16, 16, 16)
+    lat, ff, lf = setup(hisq, L)
+    sp = 0 if prec == 4 else prec
+    src = hin.gen_source(7300 + nrhs, lat.half, nrhs)
+    x = to_device(src, prec)
+    ref = [oracle.dslash(L, ff, lf, 0, src[r]) for r in range(nrhs)]
+    refA = [oracle.apply_A(L, ff, lf, 0.05, src[r]) for r in range(nrhs)]
+    taken = []
+    for way in (1, 2, 3, 9):
+        for epi in (0, 1):
+            key = "dslash/l%d/s%d/cut%d/e%d/c0 16x16x16x16 -> " % (prec, sp, nrhs, epi)
+            assert hisq.hisq_tune_load(lat.ctx, key + "%d\n" % way) == 1
+        y = empty_like_prec((nrhs, lat.half, 3), prec)
+        lat.dslash(0, y, x, prec, nrhs)
+        got = from_device(y, prec)
+        assert max(rel_err(got[r], ref[r]) for r in range(nrhs)) <= TOL[prec], way
+        lat.apply_A(y, x, 0.05, prec, nrhs)
+        got = from_device(y, prec)
+        assert max(rel_err(got[r], refA[r]) for r in range(nrhs)) <= 2 * TOL[prec], way
+        kept = [ln for ln in hisq.hisq_tune_report(lat.ctx).splitlines() if ln.startswith(key)]
+        assert len(kept) == 1 and kept[0] != key + "9"
+        taken.append(kept[0] == key + str(way))
+    assert sum(taken) == 2, taken  # each of these counts can be cut in two ways

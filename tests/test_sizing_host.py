@@ -43,3 +43,34 @@ def test_multishift_group_length_does_not_depend_on_earlier_solves(run):
         if room >= first * 1000 + 19600:  # the solve's own buffers fitted
             assert first == second == third
             assert other >= min(8, 2 * first)
+
+
+def test_launch_cuts_cover_the_vectors_and_differ(run):
+    """Every way to cut 1 to 64 vectors, for groups of 4 to 8: the groups add up, none exceeds its limit, the ways
+    offered differ, and the full groups come first (what an untuned call takes)."""
+    out = run("""
+  for (int gmax = 4; gmax <= 8; ++gmax)
+    for (int pow2 = 0; pow2 < 2; ++pow2)
+      for (int n = 1; n <= 64; ++n) {
+        int cuts[3];
+        const int k = launch_cuts(n, gmax, pow2 != 0, cuts);
+        for (int i = 0; i < k; ++i) {
+          printf("%d %d %d %d", gmax, pow2, n, cuts[i]);
+          for (int left = n; left > 0;) { const int g = next_group(cuts[i], left, gmax); printf(" %d", g); left -= g; }
+          printf("\\n");
+        }
+      }""")
+    ways = {}
+    for line in out:
+        gmax, pow2, n, cut, *groups = (int(v) for v in line.split())
+        assert sum(groups) == n and max(groups) <= gmax and min(groups) >= 1
+        if cut == 1:
+            assert len(groups) == -(-n // gmax) and max(groups) - min(groups) <= 1
+        if cut == 2:
+            assert all(g == gmax or g & (g - 1) == 0 for g in groups)
+        ways.setdefault((gmax, pow2, n), []).append((cut, groups))
+    for (gmax, pow2, n), w in ways.items():
+        assert w[0][0] == 0 and len(w[0][1]) == -(-n // gmax)
+        assert len({tuple(g) for _, g in w}) == len(w) <= 2 + pow2
+    assert [g for _, g in ways[8, 0, 12]] == [[8, 4], [6, 6]] and len(ways[8, 0, 7]) == 1
+    assert [g for _, g in ways[4, 1, 3]] == [[3], [2, 1]]
