@@ -107,3 +107,84 @@ def test_batch_errors(hisq):
     with pytest.raises(hisq.HisqError) as e:
         batch.cg(x, x.copy(), [0.1, 0.1], 1e-10, 100)  # no links
     assert e.value.code == hisq.HISQ_ENOLINKS
+
+
+def residuals(batch, mix, folded, masses, bs, x):
+    xs = x.cpu().numpy()
+    return [oracle.true_residual(m[0], *folded[l], masses[l], bs[l], xs[batch.offsets[l] // 3:batch.offsets[l + 1] // 3])
+            for l, m in enumerate(mix)]
+
+
+@pytest.mark.parametrize("inner", [0, 1])
+def test_batch_initial_guesses(hisq, inner):
+    """Guesses that are not zero, for some lattices or all (the FP64 operator at the start, which a zero guess skips),
+    the solution itself (no iterations), and one with a NaN (refused)."""
+    import torch
+    batch, folded, bs, b = build(hisq, SMALL_MIX, seed0=1100)
+    masses = [m[1] for m in SMALL_MIX]
+    bd = torch.from_numpy(b).cuda()
+    guess = torch.from_numpy(hin.gen_source(1150, len(b), 1)[0]).cuda()
+    for part in ((1, 3), (0, 1, 2, 3, 4)):
+        x = torch.zeros_like(bd)
+        for l in part:
+            x[batch.offsets[l] // 3:batch.offsets[l + 1] // 3] = guess[batch.offsets[l] // 3:batch.offsets[l + 1] // 3]
+        rc, st = batch.cg(x, bd, masses, 1e-10, 5000, inner_prec=inner)
+        assert rc == 0 and st["converged"] == 1
+        r = residuals(batch, SMALL_MIX, folded, masses, bs, x)
+        assert max(r) <= 1e-10, (part, r)
+        assert max(abs(a - c) for a, c in zip(r, st["lattice_residual"])) < 1e-11
+    x0 = x.clone()
+    rc, st = batch.cg(x, bd, masses, 1e-10, 5000, inner_prec=inner)
+    assert rc == 0 and max(st["lattice_iters"]) == 0 and torch.equal(x, x0)
+    x[7, 1] = float("nan")
+    with pytest.raises(hisq.HisqError) as e:
+        batch.cg(x, bd, masses, 1e-10, 5000, inner_prec=inner)
+    assert e.value.code == hisq.HISQ_ENONFINITE
+
+
+@pytest.mark.parametrize("inner", [0, 1])
+def test_batch_solves_one_after_the_other(hisq, inner):
+    """The iteration graph that a batch keeps: other masses, sources, solution buffers (FP64 accumulates in the
+    caller's), periods and links of one lattice, each solve judged by the oracle; and the first one again, bit for bit."""
+    import torch
+    batch, folded, bs, b = build(hisq, SMALL_MIX, seed0=1200)
+    masses = [m[1] for m in SMALL_MIX]
+    b2 = np.concatenate([hin.gen_source(1260 + l, len(v), 1)[0] for l, v in enumerate(bs)])
+    bs2 = [b2[batch.offsets[l] // 3:batch.offsets[l + 1] // 3] for l in range(len(bs))]
+    keep = []  # every x stays allocated, so each solve has a buffer of its own
+
+    def solve(src, srcs, ms, fold, **opts):
+        x = torch.zeros(src.shape, dtype=torch.complex128, device="cuda")
+        keep.append(x)
+        rc, st = batch.cg(x, torch.from_numpy(src).cuda(), ms, 1e-10, 5000, inner_prec=inner, **opts)
+        assert rc == 0 and st["converged"] == 1
+        assert max(residuals(batch, SMALL_MIX, fold, ms, srcs, x)) <= 1e-10
+        return x
+
+    first = solve(b, bs, masses, folded)
+    solve(b2, bs2, masses, folded)
+    solve(b2, bs2, [0.3 * m for m in masses[::-1]], folded)
+    solve(b, bs, masses, folded, reliable_period=17)
+    L = SMALL_MIX[2][0]
+    fat, lng = hin.gen_links(L, 1299, 0.3, 0.1)
+    batch.load(2, fat, lng)
+    other = list(folded)
+    other[2] = oracle.fold_links(L, fat.reshape(-1, 4, 3, 3), lng.reshape(-1, 4, 3, 3))
+    solve(b, bs, masses, other)
+    batch.load(2, *hin.gen_links(L, 1202, SMALL_MIX[2][2], 0.1))
+    assert torch.equal(solve(b, bs, masses, folded), first)
+
+
+def test_batch_shapes_of_no_workload(hisq):
+    """Extents that share no tile size: 12^4, 20^3x10, 28^3x6 and the smallest, light and heavy masses mixed, so that
+    lattices leave the iteration at different times."""
+    import torch
+    mix = [((12, 12, 12, 12), 0.01, 0.3), ((20, 20, 20, 10), 0.1, 0.35), ((28, 28, 28, 6), 0.03, 0.25),
+           ((4, 4, 4, 4), 0.2, 0.3), ((4, 10, 6, 26), 0.005, 0.4)]
+    batch, folded, bs, b = build(hisq, mix, seed0=1300)
+    masses = [m[1] for m in mix]
+    for inner in (1, 0):
+        x = torch.zeros(b.shape, dtype=torch.complex128, device="cuda")
+        rc, st = batch.cg(x, torch.from_numpy(b).cuda(), masses, 1e-10, 5000, inner_prec=inner)
+        assert rc == 0 and st["converged"] == 1
+        assert max(residuals(batch, mix, folded, masses, bs, x)) <= 1e-10

@@ -79,7 +79,7 @@ def test_cg_free_field_exact(hisq, inner):
 
 @pytest.mark.parametrize("inner,nrhs", [(0, 5), (1, 5), (2, 5), (1, 8), (1, 21), (3, 16)])
 def test_cg_multi_rhs(hisq, inner, nrhs):
-    """Groups of 8 and 16 vectors run with 2 and 4 threads per site; 21 = 16 + 4 + 1."""
+    """Counts that take one launch, and counts split into groups of nearly equal size (FP32: 21 = 7 + 7 + 7, 16 = 8 + 8)."""
     import torch
     L = (8, 10, 12, 14)
     lat, ff, lf = lattice(hisq, L, 7)
@@ -285,3 +285,37 @@ def test_cg_with_a_mass_whose_products_leave_fp32s_range(hisq, inner, nrhs):
     rc, st = lat.cg(x, torch.from_numpy(b).cuda(), mass, 1e-10, 200, nrhs=nrhs, inner_prec=inner)
     assert rc == 0 and st["converged"] == 1
     assert np.linalg.norm(4 * mass * mass * x.cpu().numpy() - b) <= 1e-10 * np.linalg.norm(b)
+
+
+# (link precision, vectors, tune key, forms): the forms whose threads share a site's hops; FP64 groups take a row of
+# blocks per vector
+SPLIT = [(1, 1, "nr1", (2, 3, 4)), (2, 1, "nr1", (2, 3, 4)), (1, 2, "nr2", (2,)), (2, 5, "nr5", (2,)), (1, 8, "nr8", (8,)),
+         (0, 1, "nr1", (2, 3, 4)), (0, 2, "ny2", (0, 1, 2)), (0, 5, "ny5", (0, 1, 2)), (0, 8, "ny8", (0, 1, 2))]
+
+
+@pytest.mark.parametrize("block", [64, 224])
+@pytest.mark.parametrize("prec,nrhs,name,forms", SPLIT)
+def test_cg_every_split_launch_form(hisq, prec, nrhs, name, forms, block):
+    """Mixed and plain FP64 CG with each split form forced for both Dslash launches: <p, A p> of every vector out of
+    the forms' own sums, the last block of a row partly empty. The forms add in different orders: iteration counts
+    may differ by a step or two."""
+    import torch
+    L = (4, 6, 8, 10)
+    dims = "%dx%dx%dx%d" % L
+    b = hin.gen_source(2004, oracle.volume(L) // 2, nrhs)
+    its = []
+    for vi in forms:
+        lat, ff, lf = lattice(hisq, L, 1004, precs=tuple({0, prec}))
+        for epi in (0, 1):
+            key = "dslash/l%d/s%d/%s/e%d%s" % (prec, 0 if prec == 0 else 1, name, epi, "/c0" if name[:2] == "nr" else "")
+            entry = "%s %s -> %d" % (key, dims, vi * 10000 + block)
+            assert hisq.hisq_tune_load(lat.ctx, entry + "\n") == 1
+        x = torch.zeros((nrhs, lat.half, 3), dtype=torch.complex128, device="cuda")
+        rc, st = lat.cg(x, torch.from_numpy(b).cuda(), 0.05, 1e-10, 4000, nrhs=nrhs, inner_prec=prec)
+        assert rc == 0 and st["converged"] == 1, vi
+        for r in range(nrhs):
+            assert oracle.true_residual(L, ff, lf, 0.05, b[r], x[r].cpu().numpy()) <= 1e-10, (vi, r)
+        assert entry in hisq.hisq_tune_report(lat.ctx)
+        its.append(st["iters"])
+        lat.close()
+    assert max(its) - min(its) <= 2, its

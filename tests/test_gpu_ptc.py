@@ -316,3 +316,51 @@ def test_ptc_gradients_over_many_tiles_and_scales(hisq, scale):
     loss, g1, g2 = net.train_step(b * scale, x * scale, 4, 0.0)
     assert abs(loss - loss1) <= 1e-5 * loss1
     assert rel(g1, a1) <= 1e-5 and rel(g2, a2) <= 1e-5
+
+
+def test_fcg_solves_one_after_the_other(hisq):
+    """The iteration graph that a context keeps for the flexible CG: other masses, sources, solution buffers, periods,
+    weights, a second network, links loaded anew and compressed long links, each solve judged by the oracle; and the
+    first solve again, bit for bit."""
+    import torch
+    naik = -1.0 / 24.0
+    fat, lng = hin.gen_links(L, 901, 0.35, 0.1)
+    fat2, lng2 = hin.gen_links(L, 902, 0.3, 0.1)
+    lat = hisq.Lattice(L, precs=(0, 1)).load(fat, lng)
+    fold = [oracle.fold_links(L, f.reshape(-1, 4, 3, 3), l.reshape(-1, 4, 3, 3)) for f, l in ((fat, lng), (fat2, lng2))]
+    Wa = optc.init_weights(91, scale=0.02)[0]
+    Wb = optc.init_weights(92, scale=0.03)[0]
+    Wa[0, 0, 0] = Wb[0, 0, 0] = 1.0
+
+    def network(W):
+        n = hisq.Ptc(lat)
+        n.set_tied(True)
+        n.set_weights(W, optc.tie(W))
+        return n
+
+    net, keep = network(Wa), []
+    src = hin.gen_source(903, lat.half, 2)
+
+    def solve(n, b, mass, links, **opts):
+        x = torch.zeros((1, lat.half, 3), dtype=torch.complex128, device="cuda")
+        keep.append(x)
+        rc, st = n.fcg(x, torch.from_numpy(b[None]).cuda(), mass, 1e-10, 3000, **opts)
+        assert rc == 0 and st["converged"] == 1
+        assert oracle.true_residual(L, *fold[links], mass, b, x.cpu().numpy()[0]) <= 1e-10
+        return x
+
+    first = solve(net, src[0], 0.05, 0)
+    solve(net, src[1], 0.05, 0)
+    solve(net, src[0], 0.2, 0)
+    solve(net, src[0], 0.05, 0, reliable_period=9)
+    net.set_weights(Wb, optc.tie(Wb))
+    solve(net, src[0], 0.05, 0)
+    second = network(Wa)
+    assert torch.equal(solve(second, src[0], 0.05, 0), first)
+    lat.load(fat2, lng2)
+    solve(second, src[0], 0.05, 1)
+    lat.compress_long(naik).load(fat, lng)
+    solve(second, src[0], 0.05, 0)
+    lat.compress_long(0.0).load(fat, lng)
+    net.set_weights(Wa, optc.tie(Wa))
+    assert torch.equal(solve(net, src[0], 0.05, 0), first)
