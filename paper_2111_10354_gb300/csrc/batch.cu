@@ -173,7 +173,7 @@ __device__ __forceinline__ bool grid_last(unsigned* c) {
 // out_l = D in_l (EPI_PLAIN) or out_l = a_l y_l - D in_l with pAp_l = Re<y_l, out_l> and alpha_l = rr_l / pAp_l
 // (EPI_AXPY), for every lattice l whose skip[l] is 0. FP32 takes 80 registers (three blocks of 256 per SM): at 64, like
 // the single-lattice form, the tile walk spills (16 lattices, all active: 174 and 196 us against 164 and 181 us). NARROW:
-// 72 registers in blocks of up to 128, seven per SM. It spills more and is slower (those 16 lattices 53.0 ms a solve
+// 72 registers in blocks of 128, seven per SM. It spills more and is slower (those 16 lattices 53.0 ms a solve
 // against 51.4, six 16^4 20.8 against 18.9), except where its 14% more threads take all sites at once and 80
 // registers leave some for a second round (four 16^4: 13.8 against 15.6); FP32 is tuned over both.
 template <typename LR, typename SR, int EPI, bool NARROW>
@@ -623,7 +623,7 @@ static int bdslash(hisq_batch* B, int p, void* out, const void* in, const void* 
     float best = 1e30f;
     for (int k = 0; k < FORMS * 7; ++k) {
       const int f = k / 7, c = 64 + 32 * (k % 7);
-      if (f == 1 && c > 128) continue;
+      if (f == 1 && c != 128) continue;  // the one size that fills an SM's 896 threads
       auto kern = kerns[f];
       TileTable* T;
       int rc = tile_table(B, c, &T);
@@ -631,10 +631,13 @@ static int bdslash(hisq_batch* B, int p, void* out, const void* in, const void* 
       const BatchArgs a = batch_args(B, Real<LR>::prec, c, *T);
       const int grid = persistent_grid(B, (const void*)kern, c);
       auto run = [&](const int* sk) { kern<<<grid, c, 0, B->stream>>>(a, p, out, in, y, sk, st, partials, red_row); };
-      run(d_act + B->nlat);  // warm-up
-      B->launches += 1;
-      auto timed = [&](const int* sk, float* ms) -> cudaError_t {  // one launch; short ones eight
-        for (int reps = 1;; reps = 8) {
+      if (k % 7 == 0 || f == 1) {  // warm-up of a kernel
+        run(d_act + B->nlat);
+        B->launches += 1;
+      }
+      // milliseconds of a launch: one; where it takes less than 0.4 ms two more, less than 0.1 four
+      auto timed = [&](const int* sk, float* ms, bool once) -> cudaError_t {
+        for (int reps = 1;; reps = *ms < 0.1f ? 4 : 2) {
           cudaEventRecord(e0, B->stream);
           for (int r = 0; r < reps; ++r) run(sk);
           cudaEventRecord(e1, B->stream);
@@ -643,12 +646,12 @@ static int bdslash(hisq_batch* B, int p, void* out, const void* in, const void* 
           if (e != cudaSuccess) return e;
           cudaEventElapsedTime(ms, e0, e1);
           *ms /= (float)reps;
-          if (reps == 8 || *ms >= 0.2f) return cudaSuccess;
+          if (once || reps > 1 || *ms >= 0.4f) return cudaSuccess;
         }
       };
       float ms = 0, alone = 0;
-      HISQ_CUDA(timed(d_act, &ms));
-      HISQ_CUDA(timed(d_act + B->nlat, &alone));
+      HISQ_CUDA(timed(d_act, &ms, false));
+      HISQ_CUDA(timed(d_act + B->nlat, &alone, ms >= 0.4f));
       ms = 3.f * ms + alone;
       if (ms < best) {
         best = ms;
