@@ -261,8 +261,8 @@ int hisq_multishift_cg(hisq_ctx* ctx, double* x, const double* b, int nshift, co
 /* ---------------------------------------------------------------- batches of lattices */
 /*
  * A batch of independent lattices of (possibly) different sizes, solved together: every
- * step of the batched CG is one persistent launch over a tile table that covers all
- * lattices, and one CUDA graph holds the inner iterations of a reliable cycle. This is the
+ * step of the batched CG is one persistent launch over the tiles of the lattices that still
+ * iterate, and one CUDA graph holds the inner iterations of a reliable cycle. This is the
  * many-small-lattices form of the paper's CG (Sec. 2, Sec. 3); the paper itself batches
  * right-hand sides, not lattices.
  * dims: nlat x 4 extents (each even and >= 4), nlat <= 256. FP64 and FP32 links are always
@@ -322,7 +322,8 @@ int hisq_ptc_apply(hisq_ptc* ptc, float* z, const float* r, int nvec);
 /*
  * Loss = mean over npairs of |N(b_i) - x_i|^2 / |x_i|^2 and its gradients with respect to
  * conj(w1), conj(w2) (loss, g1, g2: optional host outputs); with lr > 0 one Adam step on the
- * FP32 master weights follows. b, x: device complex64 [npairs][V/2][3].
+ * FP32 master weights follows. b, x: device complex64 [npairs][V/2][3], of any scale from
+ * 1e-18 to 1e16 (squares and products are summed in FP32 over parts of the lattice).
  */
 int hisq_ptc_train_step(hisq_ptc* ptc, const float* b, const float* x, int npairs, float lr, float* loss, float* g1,
                         float* g2);

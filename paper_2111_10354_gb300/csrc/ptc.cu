@@ -242,8 +242,8 @@ __global__ void __launch_bounds__(256) k_ptc_apply_even(const PtcGeom G, const f
 // fat links (two forward, one for M) and keeps no per-channel field. Groups of up to NV = 4 pairs share
 // every link read. 16 pairs at 32^3x8: 32.3 ms with the layers one after the other on the tensor cores (72
 // transported planes per pair written and gathered, a host read-back per pair, BF16 operands: gradients
-// 1.6e-5 from FP64), 0.76 ms in this form (2.8e-8). A group's three passes take 61, 55 and 59 us under ncu with
-// the caches flushed, against about 30 us each for their bytes: they issue on 57, 32 and 64% of the cycles
+// 1.6e-5 from FP64), 0.76 ms in this form (2.8e-8). A group's three passes take 61, 55 and 58 us under ncu with
+// the caches flushed, against about 30 us each for their bytes: they issue on 58, 38 and 64% of the cycles
 // (multiply-adds and shared-memory words of the mixing and of the inner products) at 16 warps per SM.
 //
 // All three passes walk tiles of 32 sites with one warp per hop: a warp loads its hop's link once for the
@@ -672,7 +672,7 @@ __global__ void k_adam(float* __restrict__ w, float* __restrict__ m, float* __re
 // ------------------------------------------------------------------ flexible CG
 // The updates take one 16-byte word (two complex entries) of every vector per thread; one thread per block forms the
 // complex quotients (see SumAcc on what FP64 costs). With a division by every thread and FP64 sums per site they
-// took 15.1 and 17.7 us a launch at 32^3x8 (ncu, caches flushed), now 11.8 and 13.2 us.
+// took 15.1 and 17.7 us a launch at 32^3x8 (ncu, caches flushed), in this form 11.8-14.0 and 13.2-15.5 us (three captures).
 
 // alpha = <p, r> / <p, q>; e += alpha p; r -= alpha q; rr = |r|^2; inner convergence, cycle count. nw: words.
 __global__ void __launch_bounds__(256) k_fcg_update(float4* __restrict__ e, float4* __restrict__ r,
