@@ -476,6 +476,13 @@ int hisq_selftest_bounded_wait(hisq_ctx* ctx);
  */
 int hisq_selftest_sum(hisq_ctx* ctx, const float* terms, long long n, int repeats, double* total);
 
+/*
+ * For tests: the form of a batch's Dslash that the batch would otherwise choose by timing. tile: sites per block, a
+ * multiple of 32 from 64 to 256; form: 0, or 1 (the FP32 kernels held to 72 registers, tile 128). Errors: HISQ_EINVAL.
+ * The paper has no counterpart.
+ */
+int hisq_selftest_batch_form(hisq_batch* batch, int form, int tile);
+
 #ifdef __cplusplus
 }
 #endif

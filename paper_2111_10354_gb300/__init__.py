@@ -131,6 +131,7 @@ def _load():
     lib.hisq_batch_vector_offset.restype = ctypes.c_longlong
     lib.hisq_batch_launch_count.argtypes = [vp]
     lib.hisq_batch_launch_count.restype = ctypes.c_longlong
+    lib.hisq_selftest_batch_form.argtypes = [vp, ip, ip]
     lib.hisq_batch_cg.argtypes = [vp, vp, vp, vp, dp, ip, ctypes.POINTER(hisq_solver_opts),
                                   ctypes.POINTER(hisq_solver_stats), vp, vp]
     lib.hisq_rational_apply.argtypes = [vp, vp, vp, dp, ip, vp, vp, dp, vp, ip, ctypes.POINTER(hisq_solver_opts),
@@ -417,6 +418,11 @@ def hisq_batch_vector_offset(batch, lattice: int) -> int:
 
 def hisq_batch_launch_count(batch) -> int:
     return int(_load().hisq_batch_launch_count(batch))
+
+
+def hisq_selftest_batch_form(batch, form: int, tile: int):
+    """Forces the form of a batch's Dslash (for tests)."""
+    _check(_load().hisq_selftest_batch_form(batch, form, tile), "hisq_selftest_batch_form")
 
 
 def hisq_batch_cg(batch, x, b, masses, rel_tol: float, maxiter: int, opts=None, raise_on_error=True):

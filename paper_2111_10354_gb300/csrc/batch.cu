@@ -999,6 +999,18 @@ long long hisq_batch_vector_offset(const hisq_batch* B, int lattice) {
   return lattice == B->nlat ? (long long)B->total_half * 3 : (long long)B->site_off[lattice] * 3;
 }
 
+int hisq_selftest_batch_form(hisq_batch* B, int form, int tile) {
+  if (!B) return set_error(HISQ_EINVAL, "null batch");
+  if ((form != 0 && form != 1) || tile < 64 || tile > 256 || tile % 32 || (form == 1 && tile != 128))
+    return set_error(HISQ_EINVAL, "no form %d with tiles of %d sites", form, tile);
+  release_batch_graphs(B);
+  for (int e : {EPI_PLAIN, EPI_AXPY}) {
+    B->tune["bdslash/l1/s1/e" + std::to_string(e)] = form * 10000 + tile;
+    B->tune["bdslash/l0/s0/e" + std::to_string(e)] = tile;
+  }
+  return HISQ_OK;
+}
+
 long long hisq_batch_launch_count(const hisq_batch* B) { return B ? B->launches : 0; }
 
 int hisq_batch_cg(hisq_batch* B, double* x, const double* b, const double* mass, double rel_tol, int maxiter,

@@ -5,8 +5,8 @@
 // number of threads: 16^4 has 32,768 sites per parity, 6.7 warps per SM, and each thread walks 16 hops whose
 // loads it waits for. HS = 8 gives every thread one forward and one backward hop and eight times the warps
 // (16^4 FP32, one vector: 12.5 -> 8.0 us a launch, back to back). In FP64, whose pipe takes a warp's operation in 16
-// cycles, it also spreads 8^4's 2,048 sites over all SMs (one vector: 21.0 -> 5.2 us); there the vectors go to gridDim.y with NR = 1, since
-// the links of a small lattice are in L2 and arithmetic is what FP64 pays for.
+// cycles, it also spreads 8^4's 2,048 sites over all SMs (one vector: 21.0 -> 5.2 us); there the vectors go to
+// gridDim.y with NR = 1, since the links of a small lattice are in L2 and arithmetic is what FP64 pays for.
 #pragma once
 #include "dslash_impl.cuh"
 

@@ -188,3 +188,28 @@ def test_batch_shapes_of_no_workload(hisq):
         rc, st = batch.cg(x, torch.from_numpy(b).cuda(), masses, 1e-10, 5000, inner_prec=inner)
         assert rc == 0 and st["converged"] == 1
         assert max(residuals(batch, mix, folded, masses, bs, x)) <= 1e-10
+
+
+@pytest.mark.parametrize("inner", [0, 1])
+def test_batch_every_form_and_tile(hisq, inner):
+    """Each tile the tuner may choose, and FP32's form in fewer registers, forced: lattices of fewer sites than a tile,
+    of a ragged number of tiles, and one of many, each solve judged by the oracle. The forms add in different orders:
+    iteration counts may differ by a step or two."""
+    import torch
+    mix = [((4, 4, 4, 4), 0.2, 0.3), ((6, 6, 10, 14), 0.05, 0.3), ((16, 16, 16, 16), 0.05, 0.3)]
+    batch, folded, bs, b = build(hisq, mix, seed0=1400)
+    masses = [m[1] for m in mix]
+    its = []
+    for form, tile in [(0, t) for t in range(64, 257, 32)] + ([(1, 128)] if inner == 1 else []):
+        hisq.hisq_selftest_batch_form(batch.h, form, tile)
+        x = torch.zeros(b.shape, dtype=torch.complex128, device="cuda")
+        rc, st = batch.cg(x, torch.from_numpy(b).cuda(), masses, 1e-10, 5000, inner_prec=inner)
+        assert rc == 0 and st["converged"] == 1
+        assert max(residuals(batch, mix, folded, masses, bs, x)) <= 1e-10, (form, tile)
+        its.append(st["lattice_iters"])
+    for l in range(len(mix)):
+        assert max(i[l] for i in its) - min(i[l] for i in its) <= 2, its
+    for form, tile in ((0, 32), (0, 100), (1, 64), (2, 128)):
+        with pytest.raises(hisq.HisqError) as e:
+            hisq.hisq_selftest_batch_form(batch.h, form, tile)
+        assert e.value.code == hisq.HISQ_EINVAL
